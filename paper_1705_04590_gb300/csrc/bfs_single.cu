@@ -31,6 +31,7 @@
 // Membership tests read only the current frontier; next is separate and
 // swapped in after the level (the reading of Algorithm 2 that keeps levels
 // exact).
+#include <algorithm>
 #include <climits>
 #include <cstdio>
 #include <cstring>
@@ -712,26 +713,106 @@ __device__ void task_phase(const SingleParams& p, int d, long long ntask, int* q
     acc_h += st.hv;
 }
 
-// parent_mode MIN_ID, after the last level: every reached v other than a root
-// takes the smallest neighbour one level closer, min{u in adj(v) : level(u) =
-// level(v) - 1} (on a directed graph the smallest u with u -> v; the (select2nd,
-// min) semiring of the top-down local discovery; rows are sorted, so the first
-// such u in the row).  Bottom-up levels over the
-// id-ordered rows already found exactly that parent; top-down claims did not.
-// One pass after the loop instead of one per top-down level keeps the level
-// loop's register budget free of it.
-__device__ void min_parent_pass(const SingleParams& p) {
-    const long long tid = gtid(), nth = gthreads();
-    for (long long v = tid; v < p.n; v += nth) {
-        const int lv = get_level(p, (int)v);
-        if (lv <= 0) continue;
-        long long s, e;
-        bu_row_of(p, (int)v, s, e);   // the neighbours (in-neighbours of a directed graph), id order
-        for (long long k = s; k < e; k++) {
-            const int u = __ldg(p.cols_bu + k);
-            if (get_level(p, u) == lv - 1) {
-                p.parent[v] = u;
-                break;
+// parent_mode MIN_ID: every reached v other than a root takes the smallest
+// neighbour one level closer, min{u in adj(v) : level(u) = level(v) - 1} (on a
+// directed graph the smallest u with u -> v; the (select2nd, min) semiring of
+// the top-down local discovery).  Bottom-up levels over the id-ordered rows
+// find exactly that parent (their first hit); a top-down claim takes whichever
+// edge wins.  So right after a top-down level its edges are walked once more,
+// the same way (rows, then chunk tasks), and an edge (u, v) into a vertex the
+// level discovered offers u by atomicMin: the winner's own u stands as the
+// first offer.  The work is that of the level itself, balanced like it,
+// whatever the degrees of the discovered vertices: finding the parents from the
+// discovered side instead has a thread scan each row up to its first hit, and a
+// hub found early scans most of a long one (R-MAT 20: 3.9 and 24 ms a search in
+// such a pass against 0.15 ms for the levels; with this one 0.17 ms in all).
+// Bound by its scattered level-byte reads, like the level.
+__device__ __forceinline__ void min_offer(const SingleParams& p, int d, int u, int v) {
+    if (get_level(p, v) == d + 1) atomicMin(p.parent + v, u);
+}
+
+__device__ void td_min_pass(const SingleParams& p, int d, const int* q, long long nf, long long ntask) {
+    const int lane = lane_id();
+    const long long gw = gtid() >> 5, nw = gthreads() >> 5;
+    const long long per = nf >= nw * 32 ? 32 : max(1LL, (nf + nw - 1) / nw);
+    for (long long base = gw * per; base < nf; base += nw * per) {
+        const long long i = base + lane;
+        int u = 0, deg = 0;
+        long long s = 0;
+        if (lane < per && i < nf) {
+            u = __ldcg(q + i);
+            long long e;
+            row_of(p, u, s, e);
+            deg = e - s > p.big_deg ? 0 : (int)(e - s);   // heavier rows: their chunk tasks
+        }
+        const int incl = warp_inclusive_scan(deg);
+        const int total = __shfl_sync(kFull, incl, 31);
+        const int excl = incl - deg;
+        for (int k0 = 0; k0 < total; k0 += 32) {
+            const int k = k0 + lane;
+            int j = 0;
+#pragma unroll
+            for (int step = 16; step >= 1; step >>= 1) {
+                const int c = __shfl_sync(kFull, incl, j + step - 1);
+                if (c <= k) j += step;
+            }
+            const long long sj = __shfl_sync(kFull, s, j);
+            const int exj = __shfl_sync(kFull, excl, j);
+            const int uj = __shfl_sync(kFull, u, j);
+            if (k < total) min_offer(p, d, uj, __ldg(p.cols + sj + (k - exj)));
+        }
+    }
+    const long long nt = ntask < p.task_cap ? ntask : p.task_cap;
+    for (long long t = gw; t < nt; t += nw) {
+        const int4 raw = __ldcg(reinterpret_cast<const int4*>(p.tasks + t));
+        const long long start = (long long)(unsigned)raw.x | ((long long)raw.y << 32);
+        for (int k = lane; k < raw.z; k += 32) min_offer(p, d, raw.w, __ldg(p.cols + start + k));
+    }
+}
+
+// ... and the vertices that cluster levels discovered (`lv`: one bit per level
+// byte; their frontiers live in shared memory and their rows are short), after
+// the last level: the first neighbour one level closer in each sorted row, a
+// lane per short row, the warp together for a longer one.
+__device__ void min_parent_rows(const SingleParams& p, const unsigned* lv) {
+    constexpr int kShort = 64;
+    const int lane = lane_id();
+    const long long nth = gthreads();
+    for (long long base = gtid() - lane; base < p.n; base += nth) {
+        const long long v = base + lane;
+        int want = -1;   // the parents' level
+        long long s = 0, e = 0;
+        if (v < p.n) {
+            const unsigned b = __ldcg(p.lv8 + v);
+            if (b != kLvUnseen && ((lv[b >> 5] >> (b & 31)) & 1u)) {
+                want = get_level(p, (int)v) - 1;
+                bu_row_of(p, (int)v, s, e);
+            }
+        }
+        if (want >= 0 && e - s <= kShort) {
+            for (long long k = s; k < e; k++) {
+                const int u = __ldg(p.cols_bu + k);
+                if (get_level(p, u) == want) {
+                    p.parent[v] = u;
+                    break;
+                }
+            }
+        }
+        unsigned m = __ballot_sync(kFull, want >= 0 && e - s > kShort);
+        while (m) {
+            const int L = __ffs(m) - 1;
+            m &= m - 1;
+            const long long rs = __shfl_sync(kFull, s, L), re = __shfl_sync(kFull, e, L);
+            const int w = __shfl_sync(kFull, want, L);
+            for (long long k0 = rs; k0 < re; k0 += 32) {
+                const long long k = k0 + lane;
+                const int u = k < re ? __ldg(p.cols_bu + k) : -1;
+                const unsigned hit = __ballot_sync(kFull, u >= 0 && get_level(p, u) == w);
+                if (hit) {
+                    const int pu = __shfl_sync(kFull, u, __ffs(hit) - 1);
+                    if (lane == 0) p.parent[base + L] = pu;
+                    break;
+                }
             }
         }
     }
@@ -1724,8 +1805,17 @@ __device__ bool clu_wait(const SingleParams& p, unsigned long long epi, CluState
 
 // ------------------------------------------------------------------ kernel
 
+// kMinId: the launch also makes the parents the minimum-id ones (parent_mode
+// MIN_ID with both arrays there); a variant of its own, so that the passes for it
+// take no registers from the other searches.
+template <bool kMinId>
 __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(SingleParams p) {
     Ctrl* c = p.ctrl;
+    __shared__ unsigned s_clu_lv[kMinId ? 8 : 1];   // level bytes that cluster levels discovered
+    if constexpr (kMinId) {
+        if (threadIdx.x < 8) s_clu_lv[threadIdx.x] = 0u;
+        __syncthreads();
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) c->t_enter = globaltimer_ns();
     init_phase(p);
     if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
@@ -1771,6 +1861,14 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 cluster_levels(p, qsel ? p.queue1 : p.queue0, d, nf, mf, mu, reached, epi, t_start, cs);
             } else if (!clu_wait(p, epi, cs)) {
                 return;
+            }
+            if constexpr (kMinId) {
+                if (threadIdx.x == 0)
+                    for (int L = d + 1; L <= cs.d; L++) {
+                        const int b = min(L, (int)kLvDeep);
+                        s_clu_lv[b >> 5] |= 1u << (b & 31);
+                        if (b == kLvDeep) break;
+                    }
             }
             d = cs.d;
             reached = cs.reached;
@@ -1825,6 +1923,13 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             nf_next = (long long)ld_relaxed64(&c->tail[snext]);
+            if constexpr (kMinId) {
+                if (nf_next > 0) {
+                    td_min_pass(p, d, qcur, nf, nt);
+                    // the next level writes this queue and the task list
+                    if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+                }
+            }
             qsel ^= 1;
         } else {
             if (prev == TD) {
@@ -1915,9 +2020,12 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
         c->t_levels = globaltimer_ns();
     }
     // every level ended at a grid barrier, so all staged bytes are visible here
-    if (p.parent_mode == BFS_PARENT_MIN_ID && p.parent && p.level) {
-        min_parent_pass(p);
-        if (p.lv8 && !grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+    if constexpr (kMinId) {
+        if (epi > 0) {
+            __syncthreads();
+            min_parent_rows(p, s_clu_lv);
+            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+        }
     }
     if (p.lv8) {
         materialise(p);
@@ -1942,11 +2050,20 @@ __device__ __forceinline__ long long block_words(const SingleParams& p, int b) {
 // column in its tile (b, block(k)) by binary search over JC, and claims the
 // column's rows -- all in block b, so claims are CTA-local bit operations on
 // the block's visited words held in shared memory (the sparse accumulator).
+// For minimum-id parents s_old keeps those words as the level found them: every
+// edge (k, u) into a vertex not reached before the level offers k by atomicMin
+// (as unsigned numbers: the -1 of an unreached vertex is the largest), so the
+// level ends with the minimum in place.
 __device__ void td_dcsc_phase(const SingleParams& p, int d, const int* qcur, long long nf, int* qnext, int snext,
-                              unsigned* s_own, unsigned long long& acc_m) {
+                              unsigned* s_own, unsigned* s_old, unsigned long long& acc_m) {
     const int b = blockIdx.x, lane = lane_id();
     const long long nbw = block_words(p, b), wbase = (long long)b * p.Bw;
-    for (long long w = threadIdx.x; w < nbw; w += blockDim.x) s_own[w] = __ldcg(p.visited + wbase + w);
+    const bool min_id = p.parent_mode == BFS_PARENT_MIN_ID && p.parent;
+    for (long long w = threadIdx.x; w < nbw; w += blockDim.x) {
+        const unsigned x = __ldcg(p.visited + wbase + w);
+        s_own[w] = x;
+        if (min_id) s_old[w] = x;
+    }
     __syncthreads();
     unsigned long long* tail = &p.ctrl->tail[snext];
     WarpStage st = warp_stage_dcsc();
@@ -1992,12 +2109,14 @@ __device__ void td_dcsc_phase(const SingleParams& p, int d, const int* qcur, lon
                 const unsigned bit = 1u << (ul & 31);
                 if (!(s_own[ul >> 5] & bit)) claimed = !(atomicOr(s_own + (ul >> 5), bit) & bit);
                 u = (int)((long long)b * p.B + ul);
+                if (min_id && !(s_old[ul >> 5] & bit))
+                    atomicMin(reinterpret_cast<unsigned*>(p.parent) + u, (unsigned)kj);
             }
             const unsigned cm = __ballot_sync(kFull, claimed);
             if (cm) {
                 if (claimed) {
                     st.buf[st.cnt + __popc(cm & lanemask_lt())] = u;
-                    if (p.parent) p.parent[u] = kj;
+                    if (p.parent && !min_id) p.parent[u] = kj;
                     if (p.level) p.level[u] = d + 1;
                 }
                 st.cnt += __popc(cm);
@@ -2155,7 +2274,7 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             unsigned long long am = 0;
-            td_dcsc_phase(p, d, qcur, nf, qnext, snext, s_own, am);
+            td_dcsc_phase(p, d, qcur, nf, qnext, snext, s_own, s_seg, am);
             block_add4(0, am, 0, 0, nullptr, &c->accm[snext], nullptr, nullptr);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             nf_next = (long long)ld_relaxed64(&c->tail[snext]);
@@ -2202,7 +2321,6 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
         c->num_levels = d + 1;
         c->reached = reached;
     }
-    if (p.parent_mode == BFS_PARENT_MIN_ID && p.parent && p.level) min_parent_pass(p);
 }
 
 // ------------------------------------------------------------------ allocation-free variant
@@ -2253,6 +2371,26 @@ using bfsk::Ctrl;
 using bfsk::SingleParams;
 using bfsk::Task;
 
+// the CSR kernel's variant (kMinId)
+static const void* csr_kernel(bool min_id) {
+    return min_id ? (const void*)bfsk::bfs_single_kernel<true> : (const void*)bfsk::bfs_single_kernel<false>;
+}
+
+// resident CTAs per SM of the CSR kernel: of the variant that fits fewer
+static cudaError_t csr_occupancy(int* per_sm) {
+    *per_sm = INT_MAX;
+    for (bool m : {false, true}) {
+        int nb = 0;
+        cudaError_t e = cudaFuncSetAttribute(csr_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)bfsk::kSingleDynSmem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, csr_kernel(m), bfsk::kBlock, bfsk::kSingleDynSmem);
+        if (e != cudaSuccess) return e;
+        *per_sm = std::min(*per_sm, nb);
+    }
+    return cudaSuccess;
+}
+
 bfs_status single_prepare(bfs_graph* g, cudaStream_t s) { return single_prepare_work(g, g->single, s, 0); }
 
 // Work buffers of one single-source search state on graph g; grid > 0 caps the
@@ -2290,10 +2428,7 @@ bfs_status single_prepare_work(bfs_graph* g, SingleWork& w, cudaStream_t s, int 
     w.rec_cap = rec_cap;
     w.bytes = total;
     int nb = 0;
-    BFS_CUDA_TRY(cudaFuncSetAttribute(bfsk::bfs_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)bfsk::kSingleDynSmem));
-    BFS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bfsk::bfs_single_kernel, bfsk::kBlock,
-                                                               bfsk::kSingleDynSmem));
+    BFS_CUDA_TRY(csr_occupancy(&nb));
     if (nb < 1) return fail(BFS_ERR_UNSUPPORTED, "BFS kernel cannot be resident on this device");
     w.block = bfsk::kBlock;
     w.grid = nb * g->sm_count;
@@ -2427,7 +2562,6 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         int li = 0;
         while ((1 << li) < C) li++;
         if (w.clu_grid[li] == 0) {
-            BFS_CUDA_TRY(cudaFuncSetAttribute(bfsk::bfs_single_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = (unsigned)C;
@@ -2439,8 +2573,13 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
             cfg.dynamicSmemBytes = dyn;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            int ncl = 0;
-            BFS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&ncl, bfsk::bfs_single_kernel, &cfg));
+            int ncl = INT_MAX;
+            for (bool m : {false, true}) {
+                int k = 0;
+                BFS_CUDA_TRY(cudaFuncSetAttribute(csr_kernel(m), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+                BFS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&k, csr_kernel(m), &cfg));
+                ncl = std::min(ncl, k);
+            }
             w.clu_grid[li] = ncl > 0 ? ncl * C : -1;
         }
         const int g2 = (grid < w.clu_grid[li] ? grid : w.clu_grid[li]) / C * C;
@@ -2457,6 +2596,8 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         p.clu_nf = (long long)C * (bfsk::kCluCap / 2);
         p.clu_mf = (long long)C * bfsk::kCluEdgesPerCta;
     }
+    const bool min_id = opt.parent_mode == BFS_PARENT_MIN_ID && parent;
+    void* args[] = {&p};
     BFS_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(Ctrl), s));
     if (k > 1) BFS_CUDA_TRY(cudaMemcpyAsync(w.queue0, roots_host, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, s));
     if (C > 1) {
@@ -2474,11 +2615,10 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         cfg.stream = s;
         cfg.attrs = at;
         cfg.numAttrs = 2;
-        BFS_CUDA_TRY(cudaLaunchKernelEx(&cfg, bfsk::bfs_single_kernel, p));
+        BFS_CUDA_TRY(cudaLaunchKernelExC(&cfg, csr_kernel(min_id), args));
         return BFS_OK;
     }
-    void* args[] = {&p};
-    const void* fn = dcsc ? (const void*)bfsk::bfs_dcsc_kernel : (const void*)bfsk::bfs_single_kernel;
+    const void* fn = dcsc ? (const void*)bfsk::bfs_dcsc_kernel : csr_kernel(min_id);
     BFS_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, dyn, s));
     return BFS_OK;
 }
@@ -2560,10 +2700,7 @@ extern "C" bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int3
             BFS_CUDA_TRY(cudaGetSymbolAddress(&ptr, bfsk::g_noalloc_scratch));
             int sms = 0, occ = 0;
             BFS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            BFS_CUDA_TRY(cudaFuncSetAttribute(bfsk::bfs_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)bfsk::kSingleDynSmem));
-            BFS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bfsk::bfs_single_kernel, bfsk::kBlock,
-                                                                       bfsk::kSingleDynSmem));
+            BFS_CUDA_TRY(csr_occupancy(&occ));
             if (occ < 1) return fail(BFS_ERR_UNSUPPORTED, "BFS kernel cannot be resident on this device");
             g_noalloc_sms[dev] = sms;
             g_noalloc_grid[dev] = occ * sms;
@@ -2617,7 +2754,7 @@ extern "C" bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int3
     BFS_CUDA_TRY(cudaGetLastError());
     BFS_CUDA_TRY(cudaMemsetAsync(p.ctrl, 0, sizeof(bfsk::Ctrl), s));
     void* args[] = {&p};
-    BFS_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)bfsk::bfs_single_kernel, dim3(grid), dim3(bfsk::kBlock),
+    BFS_CUDA_TRY(cudaLaunchCooperativeKernel(csr_kernel(false), dim3(grid), dim3(bfsk::kBlock),
                                              args, bfsk::kSingleDynSmem, s));
     return BFS_OK;
 }
