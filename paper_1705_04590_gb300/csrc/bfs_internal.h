@@ -65,6 +65,7 @@ struct MultiWork {
     unsigned long long* seen = nullptr;   // [n] lane masks
     unsigned long long* front = nullptr;  // [n]
     unsigned long long* next = nullptr;   // [n]
+    unsigned long long* planes = nullptr; // [4n] level planes (bfs_run_multi; null: not allocated)
     void* ctrl = nullptr;                 // bfsk::MCtrl
     void* tasks = nullptr;                // bfsk::MTask[task_cap]
     void* hubmask = nullptr;              // uint64[task_cap] lane masks of chunked rows
@@ -74,6 +75,7 @@ struct MultiWork {
     int* q1 = nullptr;
     size_t bytes = 0;
     int grid = 0, block = 0;
+    int pgrid = 0;                        // launch grid of the parent kernels
 };
 
 struct DcscTiles {

@@ -11,6 +11,11 @@
 //             stop once every missing lane is covered; next[u] = acc & miss
 //   apply:    seen |= next, front = next, next = 0; for each new lane bit i of
 //             v: level_i[v] = iteration + 1 - start_i.
+// A batch keeps the levels bit-sliced while it runs (64 lanes x 4 bits = one
+// 32-byte sector per vertex) and writes the 64 level rows once, at the end, in
+// whole lines; a search deeper than four bits hold writes the rows it has then
+// and goes on writing them directly.  The same sectors give the minimum-id
+// parents: one read of a neighbour's sector compares all 64 lanes at once.
 // Direction per iteration from the union frontier with the same rule as the
 // single-source search (m_f * alpha > m_u; n_f * beta < n).  Levels do not
 // depend on it.
@@ -31,7 +36,11 @@
 namespace bfsk {
 
 constexpr int kMBlock = 512;
-constexpr int kMChunk = 2048;     // edges per top-down chunk task
+constexpr int kMChunk = 512;      // edges per top-down chunk task
+constexpr int kMBigDeg = 256;     // rows above this become chunk tasks (the task lists are sized for it)
+constexpr int kPullChunk = 1024;  // ids per chunk task of a long row (pulls, parents)
+constexpr int kPullSteps = 16;    // 16-id steps a 4-lane group pulls before the rest of the row becomes tasks
+constexpr int kPlaneMax = 15;     // largest level + 1 that the four planes hold
 constexpr unsigned kMFull = 0xffffffffu;
 
 __device__ __forceinline__ long long m_gtid() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
@@ -226,21 +235,39 @@ __device__ void ms_tasks_phase(const MultiParams& p, MCtrl* c, int slot, int* tq
         const long long start = (long long)(unsigned)raw.x | ((long long)raw.y << 32);
         const int len = raw.z, h = raw.w;
         const unsigned long long f = ldcg64(p.hubmask + h);
-        for (int k0 = 0; k0 < len; k0 += 32) {
-            const int k = k0 + lane;
-            const bool act = k < len;
-            const int u = act ? __ldg(p.cols + start + k) : 0;
-            ms_push(p, f, u, act, st, tq, tlen);
+        // four edges per lane per step: the ids, then the seen masks in flight together
+        for (int k0 = 0; k0 < len; k0 += 128) {
+            int u[4];
+            unsigned long long nb[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int k = k0 + q * 32 + lane;
+                u[q] = k < len ? __ldg(p.cols + start + k) : -1;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) nb[q] = u[q] >= 0 ? f & ~ldcg64(p.seen + u[q]) : 0ull;
+            bool first[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) first[q] = nb[q] && atomicOr(p.next + u[q], nb[q]) == 0ull;
+#pragma unroll
+            for (int q = 0; q < 4; q++) m_append(st, tq, tlen, first[q], u[q]);
         }
     }
     m_block_flush(st, tq, tlen);
 }
 
 // Bottom-up pull: a warp owns 32 consecutive vertices; each lane ORs the
-// frontier masks of its first 8 neighbours, then rows with lanes still
-// missing continue warp-cooperatively 32 neighbours at a time.
-__device__ void ms_bu_phase(const MultiParams& p, unsigned long long active) {
-    const int lane = lane_id();
+// frontier masks of its first 8 neighbours.  Rows with lanes still missing then
+// go on in groups of 4 lanes, 8 rows per warp at a time, 16 neighbours a step
+// until every missing lane is covered; a row that is not done after kPullSteps
+// steps becomes chunk tasks of kPullChunk ids for all warps (ms_bu_tasks_phase).
+// Bound by dependent reads (ids, then masks): one row at a time per warp left
+// two thirds of the cycles waiting at the level's barrier for the warps whose
+// vertices had long rows (R-MAT 20, 64 roots).
+__device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned long long active) {
+    __shared__ unsigned char s_pend[kMBlock / 32][32];
+    __shared__ unsigned long long s_acc[kMBlock / 32][32];
+    const int lane = lane_id(), wib = threadIdx.x >> 5, grp = lane >> 2, gl = lane & 3;
     const long long gw = m_gtid() >> 5, nw = m_gthreads() >> 5;
     for (long long base = gw * 32; base < p.n; base += nw * 32) {
         const long long u = base + lane;
@@ -266,25 +293,100 @@ __device__ void ms_bu_phase(const MultiParams& p, unsigned long long active) {
             }
             pos = a + 8;
         }
-        unsigned pend = __ballot_sync(kMFull, miss && (acc & miss) != miss && pos < e);
-        while (pend) {
-            const int L = __ffs(pend) - 1;
-            pend &= pend - 1;
-            const long long ps = __shfl_sync(kMFull, pos, L), pe = __shfl_sync(kMFull, e, L);
+        const bool more = miss && (acc & miss) != miss && pos < e;
+        const unsigned pend = __ballot_sync(kMFull, more);
+        const int np = __popc(pend);
+        if (more) s_pend[wib][__popc(pend & lanemask_lt())] = (unsigned char)lane;
+        __syncwarp();
+        for (int r0 = 0; r0 < np; r0 += 8) {
+            const bool has = r0 + grp < np;
+            const int L = has ? (int)s_pend[wib][r0 + grp] : 0;
+            long long q = __shfl_sync(kMFull, pos, L);
+            const long long qe = __shfl_sync(kMFull, e, L);
             const unsigned long long mL = __shfl_sync(kMFull, miss, L);
             unsigned long long aL = __shfl_sync(kMFull, acc, L);
-            for (long long q0 = ps; q0 < pe; q0 += 32) {
-                const long long q = q0 + lane;
+            bool live = has;
+            for (int step = 0; step < kPullSteps && __any_sync(kMFull, live); step++) {
                 unsigned long long x = 0;
-                if (q < pe) x = ldcg64(p.front + __ldg(p.cols_bu + q));
-                aL |= warp_or64(x);
-                if ((aL & mL) == mL) break;
+                const long long q4 = q + 4 * gl;   // a multiple of 4: the window was aligned
+                if (live && q4 < qe) {
+                    const int4 y = __ldg(reinterpret_cast<const int4*>(p.cols_bu + q4));
+                    const int ids[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                    for (int t = 0; t < 4; t++)
+                        if (q4 + t < qe) x |= ldcg64(p.front + ids[t]);
+                }
+                x |= __shfl_xor_sync(kMFull, x, 1);
+                x |= __shfl_xor_sync(kMFull, x, 2);
+                if (live) {
+                    aL |= x;
+                    q += 16;
+                    live = (aL & mL) != mL && q < qe;
+                }
             }
-            if (lane == L) acc = aL;
+            if (has && gl == 0) {
+                s_acc[wib][L] = aL;
+                if (live) {
+                    const long long nch = (qe - q + kPullChunk - 1) / kPullChunk;
+                    const unsigned long long t0 = atomicAdd(&c->ntask[slot], (unsigned long long)nch);
+                    for (long long k = 0; k < nch; k++) {
+                        const long long ti = (long long)t0 + k;
+                        if (ti >= p.task_cap) {
+                            raise_status(&c->b, kDevOverflow);
+                            break;
+                        }
+                        MTask t;
+                        t.start = q + k * kPullChunk;
+                        t.len = (int)min((long long)kPullChunk, qe - t.start);
+                        t.v = (int)(base + L);
+                        p.tasks[ti] = t;
+                    }
+                }
+            }
         }
+        __syncwarp();
+        if (more) acc = s_acc[wib][lane];
         const unsigned long long nb = acc & miss;
         if (nb) p.next[u] = nb;
+        __syncwarp();
     }
+}
+
+// The chunks of long rows: a warp each, four ids per lane per step; a row's
+// chunks meet in its next mask.
+__device__ void ms_bu_tasks_phase(const MultiParams& p, MCtrl* c, int slot, unsigned long long active) {
+    const int lane = lane_id();
+    const long long gw = m_gtid() >> 5, nw = m_gthreads() >> 5;
+    const long long nt = min((long long)ld_relaxed64(&c->ntask[slot]), p.task_cap);
+    for (long long t = gw; t < nt; t += nw) {
+        const int4 raw = __ldcg(reinterpret_cast<const int4*>(p.tasks + t));
+        const long long start = (long long)(unsigned)raw.x | ((long long)raw.y << 32);
+        const int len = raw.z, v = raw.w;
+        const unsigned long long miss = active & ~ldcg64(p.seen + v) & ~ldcg64(p.next + v);
+        unsigned long long acc = 0;
+        for (int k0 = 0; k0 < len && (acc & miss) != miss; k0 += 128) {
+            int u[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int k = k0 + q * 32 + lane;
+                u[q] = k < len ? __ldg(p.cols_bu + start + k) : -1;
+            }
+            unsigned long long x = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (u[q] >= 0) x |= ldcg64(p.front + u[q]);
+            acc |= warp_or64(x);
+        }
+        if (lane == 0 && (acc & miss)) atomicOr(p.next + v, acc & miss);
+    }
+}
+
+// Levels of the lanes in x at vertex v, found by iteration `iter`: into the
+// planes while they hold it (one sector of v), else straight into the rows.
+__device__ __forceinline__ void ms_set_planes(const MultiParams& p, long long v, unsigned long long x, int val) {
+#pragma unroll
+    for (int b = 0; b < 4; b++)
+        if ((val >> b) & 1) p.planes[4 * v + b] = ldcg64(p.planes + 4 * v + b) | x;
 }
 
 // Apply over the touched vertices (after a top-down level, whose phase already
@@ -293,7 +395,7 @@ __device__ void ms_bu_phase(const MultiParams& p, unsigned long long active) {
 // every active lane has now seen (subtracted from m_u) and which lanes found
 // anything.
 __device__ void ms_apply_phase(const MultiParams& p, MCtrl* c, int slot, int iter, unsigned long long active,
-                               const LaneSmem& L, const int* tq, long long tlen) {
+                               const LaneSmem& L, bool direct, const int* tq, long long tlen) {
     const long long tid = m_gtid(), nth = m_gthreads();
     unsigned long long am = 0, adone = 0, found = 0;
     for (long long i = tid; i < tlen; i += nth) {
@@ -307,7 +409,8 @@ __device__ void ms_apply_phase(const MultiParams& p, MCtrl* c, int slot, int ite
         const long long deg = __ldg(p.off + v + 1) - __ldg(p.off + v);
         am += (unsigned long long)deg;
         if ((s & active) != active && ((s | x) & active) == active) adone += (unsigned long long)deg;
-        unsigned long long bits = x;
+        if (!direct) ms_set_planes(p, v, x, iter + 2);
+        unsigned long long bits = direct ? x : 0ull;
         while (bits) {
             const int i2 = __ffsll((long long)bits) - 1;
             bits &= bits - 1;
@@ -324,7 +427,7 @@ __device__ void ms_apply_phase(const MultiParams& p, MCtrl* c, int slot, int ite
 // anyway): the same updates as ms_apply_phase, old frontier bits dropped in
 // the same pass, and the new frontier listed in queue nq.
 __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int iter, unsigned long long active,
-                                   const LaneSmem& L, int* nq, unsigned long long* nlen) {
+                                   const LaneSmem& L, bool direct, int* nq, unsigned long long* nlen) {
     const long long tid = m_gtid(), nth = m_gthreads();
     MStage st = m_stage();
     unsigned long long an = 0, am = 0, adone = 0, found = 0;
@@ -339,6 +442,7 @@ __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int
                 p.seen[v] = s | x;
                 p.front[v] = x;
                 found |= x;
+                if (!direct) ms_set_planes(p, v, x, iter + 2);
                 const long long deg = __ldg(p.off + v + 1) - __ldg(p.off + v);
                 an += 1;
                 am += (unsigned long long)deg;
@@ -350,7 +454,7 @@ __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int
         // level rows: the warp walks the lanes any of its 32 vertices gained, one
         // lane at a time, so each store instruction writes consecutive vertices of
         // one row (a lane-by-lane walk per thread would scatter every store)
-        unsigned long long ub = warp_or64(x);
+        unsigned long long ub = direct ? warp_or64(x) : 0ull;
         while (ub) {
             const int i2 = __ffsll((long long)ub) - 1;
             ub &= ub - 1;
@@ -371,6 +475,41 @@ __device__ void ms_clear_phase(const MultiParams& p) {
         p.seen[v] = 0ull;
         p.front[v] = 0ull;
         p.next[v] = 0ull;
+        if (p.planes) {
+            const ulonglong2 z = make_ulonglong2(0ull, 0ull);
+            reinterpret_cast<ulonglong2*>(p.planes)[2 * v] = z;
+            reinterpret_cast<ulonglong2*>(p.planes)[2 * v + 1] = z;
+        }
+    }
+}
+
+// The level rows from the planes, every active lane's row whole: a warp takes
+// 32 consecutive vertices and writes one line of each row in turn.  Bound by the
+// rows' bytes (64 rows of R-MAT 22: 1.07 GB); a -1 fill and a scattered store
+// per (lane, vertex) moved each line two or three times.  Eight lanes' four bits
+// are first woven into one word of nibbles.
+__device__ __forceinline__ unsigned ms_spread8(unsigned x) {
+    x = (x | (x << 12)) & 0x000F000Fu;
+    x = (x | (x << 6)) & 0x03030303u;
+    return (x | (x << 3)) & 0x11111111u;
+}
+
+__device__ void ms_rows_phase(const MultiParams& p, unsigned long long active) {
+    const long long tid = m_gtid(), nth = m_gthreads();
+    const int k = __popcll(active);   // lanes 0..k-1
+    for (long long v = tid; v < p.n; v += nth) {
+        const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2*>(p.planes) + 2 * v);
+        const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2*>(p.planes) + 2 * v + 1);
+        int* row = p.level0 + v;
+        for (int i0 = 0; i0 < k; i0 += 8, row += 8 * p.n) {
+            const unsigned w = ms_spread8((unsigned)(a.x >> i0) & 0xFFu) | ms_spread8((unsigned)(a.y >> i0) & 0xFFu) << 1 |
+                               ms_spread8((unsigned)(b.x >> i0) & 0xFFu) << 2 |
+                               ms_spread8((unsigned)(b.y >> i0) & 0xFFu) << 3;
+            int* r = row;
+#pragma unroll
+            for (int i = 0; i < 8; i++, r += p.n)
+                if (i0 + i < k) *r = (int)((w >> (4 * i)) & 15u) - 1;
+        }
     }
 }
 
@@ -389,7 +528,7 @@ __device__ void ms_fill_rows(const MultiParams& p, unsigned long long mask, cons
 // Seed lanes in `mask` at their roots (atomics: several lanes may share a
 // root); a root not yet in the frontier joins the frontier queue.  Run by the
 // first warp (64 lanes at most -> two rounds).
-__device__ void ms_seed_phase(const MultiParams& p, unsigned long long mask, const LaneSmem& L, int* fq,
+__device__ void ms_seed_phase(const MultiParams& p, unsigned long long mask, const LaneSmem& L, bool direct, int* fq,
                               unsigned long long* flen) {
     if (m_gtid() >= 32) return;
     MStage st = m_stage();
@@ -401,7 +540,8 @@ __device__ void ms_seed_phase(const MultiParams& p, unsigned long long mask, con
             r = p.roots[i];
             atomicOr(p.seen + r, 1ull << i);
             add = atomicOr(p.front + r, 1ull << i) == 0ull;
-            L.rows[i][r] = 0;
+            if (direct) L.rows[i][r] = 0;
+            else atomicOr(p.planes + 4 * (long long)r, 1ull << i);
         }
         m_append(st, fq, flen, add, r);
     }
@@ -422,10 +562,11 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
     load_lanes(p, L);
     MCtrl* c = p.ctrl;
     const unsigned long long active = p.active;
+    bool direct = p.planes == nullptr;
     ms_clear_phase(p);
-    ms_fill_rows(p, active, L);
+    if (direct) ms_fill_rows(p, active, L);
     if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-    ms_seed_phase(p, active, L, p.q0, &c->qlen[0]);
+    ms_seed_phase(p, active, L, direct, p.q0, &c->qlen[0]);
     if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
     // level-0 statistics from the (few) distinct roots, identical in every CTA
     long long mf = 0, mu = p.nnz;
@@ -452,6 +593,12 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
         const long long flen = (long long)ld_relaxed64(&c->qlen[qsel]);
         unsigned long long* tlen = &c->qlen[qsel ^ 1];
         const int dir = ms_decide(p, prev, flen, mf, mu);
+        if (!direct && it + 2 > kPlaneMax) {
+            // deeper than the planes: the rows as they stand (every CTA is past the last
+            // apply's barrier; the first write into a row from here on is after the next)
+            ms_rows_phase(p, active);
+            direct = true;
+        }
         if (dir == 0) {
             ms_td_phase(p, c, slot, fq, flen, tq, tlen);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
@@ -459,29 +606,176 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
                 ms_tasks_phase(p, c, slot, tq, tlen);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
-            ms_apply_phase(p, c, slot, it, active, L, tq, (long long)ld_relaxed64(tlen));
+            ms_apply_phase(p, c, slot, it, active, L, direct, tq, (long long)ld_relaxed64(tlen));
         } else {
-            ms_bu_phase(p, active);
+            ms_bu_phase(p, c, slot, active);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            ms_apply_all_phase(p, c, slot, it, active, L, tq, tlen);
+            if (ld_relaxed64(&c->ntask[slot]) > 0) {
+                ms_bu_tasks_phase(p, c, slot, active);
+                if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+            }
+            ms_apply_all_phase(p, c, slot, it, active, L, direct, tq, tlen);
         }
         if (m_gtid() == 0) c->qlen[qsel] = 0;   // the old frontier's queue collects the next touched set
         if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
         const long long nt = (long long)ld_relaxed64(&c->accn[slot]);
         qsel ^= 1;
         if (nt == 0) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) c->iterations = it + 1;
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                c->iterations = it + 1;
+                c->direct = direct ? 1u : 0u;
+            }
             break;
         }
         mu -= (long long)ld_relaxed64(&c->mdone[slot]);
         mf = (long long)ld_relaxed64(&c->accm[slot]);
         prev = dir;
     }
+    if (!direct) ms_rows_phase(p, active);
 }
 
-// parent_i[v] = min{u in adj(v) : level_i[u] = level_i[v] - 1} (rows sorted: first hit), root -> itself.
+// Minimum-id parents of a batch: parent_i[v] = min{u in adj(v) : level_i[u] =
+// level_i[v] - 1} (rows sorted: the first such u), a root's its own, -1 where not
+// reached.  From the planes: with t the bit-sliced (level + 1) - 1 of v's lanes,
+// one sector read of a neighbour u says in a few word operations for which of the 64
+// lanes u is a parent, so a row is read once for all lanes and left as soon as
+// every lane has its parent (lane by lane over the level rows, one thread per
+// vertex, R-MAT 18 with 40 roots took 47 ms).  A lane takes a vertex, a warp 32
+// consecutive ones; their parents gather in shared memory so that every output
+// row gets whole lines.  Lanes at level 1 need no search: their only parent is
+// the root.  Rows above kMBigDeg become chunk tasks for ms_parent_tasks_kernel:
+// a hub's parent in a lane with a small frontier may be anywhere in its row.
+constexpr int kPBlock = 256;
+constexpr int kPTileRow = 33;   // 32 vertices, padded against bank conflicts
+constexpr size_t kParentSmem = sizeof(int) * 64 * kPTileRow * (kPBlock / 32);
+
+struct LanePlanes {
+    unsigned long long p0, p1, p2, p3;
+};
+__device__ __forceinline__ LanePlanes ms_planes(const MultiParams& p, long long v) {
+    const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(p.planes) + 2 * v);
+    const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(p.planes) + 2 * v + 1);
+    return {a.x, a.y, b.x, b.y};
+}
+// bit-sliced decrement (lanes holding 0 wrap; callers mask them)
+__device__ __forceinline__ LanePlanes ms_minus1(const LanePlanes& a) {
+    const unsigned long long b1 = ~a.p0, b2 = b1 & ~a.p1, b3 = b2 & ~a.p2;
+    return {~a.p0, a.p1 ^ b1, a.p2 ^ b2, a.p3 ^ b3};
+}
+__device__ __forceinline__ unsigned long long ms_equal(const LanePlanes& a, const LanePlanes& b) {
+    return ~((a.p0 ^ b.p0) | (a.p1 ^ b.p1) | (a.p2 ^ b.p2) | (a.p3 ^ b.p3));
+}
+// lanes at level >= 2: the ones whose parent has to be looked for
+__device__ __forceinline__ unsigned long long ms_searching(const LanePlanes& a) { return a.p2 | a.p3 | (a.p0 & a.p1); }
+
+__global__ void __launch_bounds__(kPBlock) ms_parent_planes_kernel(MultiParams p, int* parent0) {
+    extern __shared__ int s_tile[];
+    __shared__ int s_root[64];
+    MCtrl* c = p.ctrl;
+    if (c->direct || c->b.status != kDevOk) return;
+    if (threadIdx.x < 64) s_root[threadIdx.x] = p.roots[threadIdx.x];
+    __syncthreads();
+    const int lane = lane_id(), k = __popcll(p.active);
+    int* tile = s_tile + (threadIdx.x >> 5) * 64 * kPTileRow;
+    const long long gw = m_gtid() >> 5, nw = m_gthreads() >> 5;
+    for (long long base = gw * 32; base < p.n; base += nw * 32) {
+        const long long v = base + lane;
+        LanePlanes a = {0, 0, 0, 0};
+        if (v < p.n) a = ms_planes(p, v);
+        const unsigned long long reached = a.p0 | a.p1 | a.p2 | a.p3;
+        const unsigned long long root = a.p0 & ~(a.p1 | a.p2 | a.p3), one = a.p1 & ~(a.p0 | a.p2 | a.p3);
+        for (int i = 0; i < k; i++)
+            tile[i * kPTileRow + lane] = (root >> i) & 1ull ? (int)v : (one >> i) & 1ull ? s_root[i] : -1;
+        unsigned long long need = reached & ms_searching(a);
+        if (need) {
+            const LanePlanes t = ms_minus1(a);
+            const long long s = __ldg(p.off + v), e = __ldg(p.off + v + 1);
+            if (e - s > kMBigDeg) {
+                const long long nch = (e - s + kPullChunk - 1) / kPullChunk;
+                const unsigned long long t0 = atomicAdd(&c->nptask, (unsigned long long)nch);
+                for (long long j = 0; j < nch && (long long)t0 + j < p.task_cap; j++) {
+                    MTask m;
+                    m.start = s + j * kPullChunk;
+                    m.len = (int)min((long long)kPullChunk, e - m.start);
+                    m.v = (int)v;
+                    p.tasks[t0 + j] = m;
+                }
+                need = 0;
+            }
+            for (long long q = s; need && q < e; q += 4) {
+                int u[4];
+                LanePlanes b[4];
+#pragma unroll
+                for (int j = 0; j < 4; j++) u[j] = __ldg(p.cols + min(q + j, e - 1));
+#pragma unroll
+                for (int j = 0; j < 4; j++) b[j] = ms_planes(p, u[j]);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    unsigned long long hit = ms_equal(b[j], t) & need;
+                    need &= ~hit;
+                    while (hit) {
+                        const int i = __ffsll((long long)hit) - 1;
+                        hit &= hit - 1;
+                        tile[i * kPTileRow + lane] = u[j];
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (v < p.n) {
+            int* o = parent0 + v;
+            for (int i = 0; i < k; i++, o += p.n) *o = tile[i * kPTileRow + lane];
+        }
+        __syncwarp();
+    }
+}
+
+// The long rows' chunks: a warp reads 32 ids and their sectors per step; the
+// lowest warp lane that offers search lane i a parent is the chunk's smallest,
+// and the chunks meet by atomicMin (unsigned: -1 is the largest).
+__global__ void __launch_bounds__(kPBlock) ms_parent_tasks_kernel(MultiParams p, int* parent0) {
+    const MCtrl* c = p.ctrl;
+    if (c->direct || c->b.status != kDevOk) return;
+    const int lane = lane_id();
+    const long long gw = m_gtid() >> 5, nw = m_gthreads() >> 5;
+    const long long nt = min((long long)c->nptask, p.task_cap);
+    for (long long ti = gw; ti < nt; ti += nw) {
+        const MTask m = p.tasks[ti];
+        const LanePlanes a = ms_planes(p, m.v), t = ms_minus1(a);
+        unsigned long long need = (a.p0 | a.p1 | a.p2 | a.p3) & ms_searching(a);
+        for (int k0 = 0; k0 < m.len && need; k0 += 32) {
+            const int kk = k0 + lane;
+            int u = -1;
+            unsigned long long hit = 0;
+            if (kk < m.len) {
+                u = __ldg(p.cols + m.start + kk);
+                hit = ms_equal(ms_planes(p, u), t) & need;
+            }
+            const unsigned long long any = warp_or64(hit);
+            if (!any) continue;
+            need &= ~any;
+            // drop the search lanes that a lower warp lane (a smaller id) offers too
+            unsigned long long pre = hit;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long y = __shfl_up_sync(kMFull, pre, o);
+                if (lane >= o) pre |= y;
+            }
+            pre = __shfl_up_sync(kMFull, pre, 1);
+            if (lane > 0) hit &= ~pre;
+            while (hit) {
+                const int i = __ffsll((long long)hit) - 1;
+                hit &= hit - 1;
+                atomicMin(reinterpret_cast<unsigned*>(parent0 + (long long)i * p.n + m.v), (unsigned)u);
+            }
+        }
+    }
+}
+
+// The same over the level rows, for a search that outgrew its planes.
 __global__ void ms_parent_kernel(MultiParams p, int* const* prow) {
     __shared__ LaneSmem L;
+    if (!p.ctrl->direct) return;
     load_lanes(p, L);
     const long long tid = m_gtid(), nth = m_gthreads();
     for (int i = 0; i < 64; i++) {
@@ -544,7 +838,7 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_serve_kernel(MultiParams p, in
     if (newmask | drop) {
         ms_fill_rows(p, newmask, L);
         if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-        ms_seed_phase(p, newmask, L, qsel ? p.q1 : p.q0, &c->qlen[qsel]);
+        ms_seed_phase(p, newmask, L, true, qsel ? p.q1 : p.q0, &c->qlen[qsel]);
         if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
     }
     long long mf = c->s_mf;
@@ -571,11 +865,15 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_serve_kernel(MultiParams p, in
                 ms_tasks_phase(p, c, slot, tq, tlen);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
-            ms_apply_phase(p, c, slot, it, active, L, tq, (long long)ld_relaxed64(tlen));
+            ms_apply_phase(p, c, slot, it, active, L, true, tq, (long long)ld_relaxed64(tlen));
         } else {
-            ms_bu_phase(p, active);
+            ms_bu_phase(p, c, slot, active);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            ms_apply_all_phase(p, c, slot, it, active, L, tq, tlen);
+            if (ld_relaxed64(&c->ntask[slot]) > 0) {
+                ms_bu_tasks_phase(p, c, slot, active);
+                if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+            }
+            ms_apply_all_phase(p, c, slot, it, active, L, true, tq, tlen);
         }
         if (tid == 0) c->qlen[qsel] = 0;
         if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
@@ -612,7 +910,8 @@ static size_t mask_bytes(const bfs_graph* g) { return sizeof(unsigned long long)
 bfs_status multi_alloc(bfs_graph* g, MultiWork& w, cudaStream_t s) {
     if (w.ready) return BFS_OK;
     const size_t nb = mask_bytes(g);
-    const long long task_cap = g->nnz / bfsk::kMChunk + g->nnz / 256 + 1024;
+    // chunks of rows above kMBigDeg: at most nnz / chunk whole ones and one rest per row
+    const long long task_cap = g->nnz / bfsk::kMChunk + g->nnz / bfsk::kMBigDeg + 1024;
     w.seen = (unsigned long long*)mem_of(g, w).alloc(nb, s);
     w.front = (unsigned long long*)mem_of(g, w).alloc(nb, s);
     w.next = (unsigned long long*)mem_of(g, w).alloc(nb, s);
@@ -635,6 +934,11 @@ bfs_status multi_alloc(bfs_graph* g, MultiWork& w, cudaStream_t s) {
     if (occ < 1) return fail(BFS_ERR_UNSUPPORTED, "multi-source kernel cannot be resident");
     w.block = bfsk::kMBlock;
     w.grid = occ * g->sm_count;
+    BFS_CUDA_TRY(cudaFuncSetAttribute(bfsk::ms_parent_planes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)bfsk::kParentSmem));
+    BFS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bfsk::ms_parent_planes_kernel, bfsk::kPBlock,
+                                                               bfsk::kParentSmem));
+    w.pgrid = std::max(1, occ) * g->sm_count;
     BFS_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(MCtrl), s));
     BFS_CUDA_TRY(cudaMemsetAsync(w.lanes, 0, sizeof(bfsk::LaneTable), s));
     w.ready = true;
@@ -647,6 +951,7 @@ void multi_free(bfs_graph* g, MultiWork& w) {
     mem_of(g, w).release(w.seen, nb, nullptr);
     mem_of(g, w).release(w.front, nb, nullptr);
     mem_of(g, w).release(w.next, nb, nullptr);
+    mem_of(g, w).release(w.planes, 4 * nb, nullptr);
     mem_of(g, w).release(w.ctrl, sizeof(MCtrl), nullptr);
     mem_of(g, w).release(w.tasks, sizeof(MTask) * (size_t)w.task_cap, nullptr);
     mem_of(g, w).release(w.hubmask, sizeof(unsigned long long) * (size_t)w.task_cap, nullptr);
@@ -658,7 +963,16 @@ void multi_free(bfs_graph* g, MultiWork& w) {
     w.mem = keep;
 }
 
-bfs_status multi_prepare(bfs_graph* g, cudaStream_t s) { return multi_alloc(g, g->multi, s); }
+bfs_status multi_prepare(bfs_graph* g, cudaStream_t s) {
+    MultiWork& w = g->multi;
+    if (w.ready) return BFS_OK;
+    bfs_status st = multi_alloc(g, w, s);
+    if (st != BFS_OK) return st;
+    // 32 bytes per vertex of level planes; without room for them the rows are written directly
+    w.planes = (unsigned long long*)mem_of(g, w).alloc(4 * mask_bytes(g), s);
+    if (w.planes) w.bytes += 4 * mask_bytes(g);
+    return BFS_OK;
+}
 void multi_release(bfs_graph* g) { multi_free(g, g->multi); }
 
 static MultiParams multi_params(bfs_graph* g, MultiWork& w, const bfs_options& opt) {
@@ -685,7 +999,8 @@ static MultiParams multi_params(bfs_graph* g, MultiWork& w, const bfs_options& o
     p.mode = opt.mode == BFS_MODE_RANDOM ? BFS_MODE_DO : opt.mode;
     p.alpha = opt.alpha;
     p.beta = opt.beta;
-    p.big_deg = opt.td_big_degree > 0 ? opt.td_big_degree : 256;
+    p.planes = w.planes;
+    p.big_deg = std::max(opt.td_big_degree, bfsk::kMBigDeg);
     p.timeout_ns = (unsigned long long)(opt.timeout_ms > 0 ? opt.timeout_ms : 10000) * 1000000ull;
     p.expected = (unsigned)w.grid + (unsigned)(g->debug_barrier_extra > 0 ? g->debug_barrier_extra : 0);
     return p;
@@ -710,10 +1025,17 @@ bfs_status multi_launch(bfs_graph* g, const int32_t* roots_host, int32_t k, int3
         BFS_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(MCtrl), s));
         MultiParams p = multi_params(g, w, opt);
         p.active = (kk == 64) ? ~0ull : ((1ull << kk) - 1ull);
+        p.level0 = t.rows[0];
         void* args[] = {&p};
         BFS_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)bfsk::bfs_multi_kernel, dim3(w.grid), dim3(w.block),
                                                  args, 0, s));
         if (parent) {
+            if (p.planes) {
+                bfsk::ms_parent_planes_kernel<<<w.pgrid, bfsk::kPBlock, bfsk::kParentSmem, s>>>(p, t.prow[0]);
+                BFS_CUDA_TRY(cudaGetLastError());
+                bfsk::ms_parent_tasks_kernel<<<w.pgrid, bfsk::kPBlock, 0, s>>>(p, t.prow[0]);
+                BFS_CUDA_TRY(cudaGetLastError());
+            }
             bfsk::LaneTable* lt = reinterpret_cast<bfsk::LaneTable*>(w.lanes);
             bfsk::ms_parent_kernel<<<w.grid, w.block, 0, s>>>(p, lt->prow);
             BFS_CUDA_TRY(cudaGetLastError());

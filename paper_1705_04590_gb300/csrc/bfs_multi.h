@@ -9,7 +9,7 @@ namespace bfsk {
 struct MTask {
     long long start;
     int len;
-    int v;        // index of the row's first chunk task: its lane mask is hubmask[v]
+    int v;        // top-down: index of the row's first chunk task (its lane mask is hubmask[v]); else the vertex
 };
 
 // Control block of a multi-source launch / server slot.
@@ -21,6 +21,9 @@ struct MCtrl {
     unsigned long long ntask[3];   // top-down chunk tasks
     unsigned long long found[3];   // lanes that found at least one vertex
     long long iterations;
+    unsigned long long nptask;     // chunk tasks of the parent pass over long rows
+    unsigned direct;               // 1: the search outgrew its level planes, the level rows were written as it went
+    unsigned pad_direct;
     // server slot state carried across launches (bfs_serve_kernel)
     long long s_done;              // iterations run by the last launch
     unsigned long long s_finished; // lanes whose search ended in the last launch
@@ -53,6 +56,10 @@ struct MultiParams {
     unsigned long long* seen;
     unsigned long long* front;
     unsigned long long* next;
+    // [4n] level planes: bit i of planes[4v + b] is bit b of (lane i's level of v) + 1,
+    // 0 while not reached (null: the level rows are written as the search goes)
+    unsigned long long* planes;
+    int* level0;                   // with planes: row of lane 0; lane i's is level0 + i * n
     MCtrl* ctrl;
     MTask* tasks;
     unsigned long long* hubmask;   // [task_cap] lane masks of chunked rows

@@ -52,3 +52,34 @@ def test_min_parents_of_top_down_levels(gpu_lib, shape, layout, cluster):
         assert np.array_equal(level.cpu().numpy(), want), mode
         assert np.array_equal(parent.cpu().numpy(), oracle.min_parent(ref, want.astype(np.int32))), mode
     g.close()
+
+
+@pytest.mark.parametrize("k", [1, 7, 64, 70])
+@pytest.mark.parametrize("shape", ["rmat", "star", "hubs", "path14", "path15", "path16", "comb", "er"])
+def test_multi_rows_and_parents(gpu_lib, shape, k):
+    """Batches whose levels end just inside and just past the level planes (depth 14 / 15),
+    whose rows are longer than a group pulls before they become tasks, that do not fill
+    their lanes, with both row orders and both directions alone."""
+    bfs = gpu_lib
+    rng = np.random.default_rng(3)
+    e = {"rmat": lambda: graphgen.rmat(12, seed=6), "star": lambda: graphgen.star(4001),
+         # two hubs that share 3000 leaves, ids scattered: long rows with late hits
+         "hubs": lambda: graphgen.EdgeList(3002, np.repeat(np.array([17, 2900], np.int32), 3002),
+                                           np.tile(rng.permutation(3002).astype(np.int32), 2)),
+         "path14": lambda: graphgen.path(15), "path15": lambda: graphgen.path(16), "path16": lambda: graphgen.path(17),
+         "comb": lambda: _comb(40, 300), "er": lambda: graphgen.erdos_renyi(3333, 9000, seed=2)}[shape]()
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, hub_first=True)
+    roots = rng.choice(graphgen.pick_roots(e, 64, 5), k).tolist()
+    want = np.stack([oracle.levels(ref, r) for r in roots])
+    pmin = np.stack([oracle.min_parent(ref, w) for w in want])
+    level, parent = _buffers(e.n, k)
+    for mode in (bfs.MODE_DO, bfs.MODE_TD_ONLY, bfs.MODE_BU_ONLY):
+        for rows in (bfs.BU_ROWS_BY_ID, bfs.BU_ROWS_HUB_FIRST):
+            level.fill_(-7)
+            parent.fill_(-7)
+            g.run_multi(roots, level, parent=parent, opts=bfs.options(mode=mode, bu_rows=rows))
+            g.sync()
+            assert np.array_equal(level.cpu().numpy().reshape(k, e.n), want), (mode, rows)
+            assert np.array_equal(parent.cpu().numpy().reshape(k, e.n), pmin), (mode, rows)
+    g.close()
