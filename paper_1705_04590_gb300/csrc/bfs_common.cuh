@@ -34,22 +34,32 @@ struct BarrierState {
 };
 constexpr unsigned long long kAbortBit = 1ull << 63;
 
+// Counters of one level, one 128-byte line: a CTA reads them with one request
+// after the barrier that completes them (grid_sync_read).
+struct __align__(128) LevelCtr {
+    unsigned long long tail;       // length of the queue holding the slot's frontier
+    unsigned long long accn;       // size of the frontier (bottom-up producer)
+    unsigned long long accm;       // degree sum of the frontier
+    unsigned long long scanned;    // bottom-up searchers of the level producing it
+    unsigned long long examined;   // serial early-exit examinations of that level
+    unsigned long long ntask;      // top-down edge-chunk tasks of that level
+    unsigned long long nmiss;      // bottom-up first-probe misses left to phase B (miss-list length)
+    unsigned long long nmiss_in;   // ... resolved by their chunk's warp in phase A
+    unsigned long long dsum_out;   // directed graphs: out-degree sum of the frontier
+    unsigned long long dsum_in;    // directed graphs: in-degree sum of the frontier
+    unsigned long long heavy;      // top-down: its vertices above the cluster-level degree cap
+    __host__ __device__ void zero() {
+        tail = accn = accm = scanned = examined = ntask = nmiss = nmiss_in = dsum_out = dsum_in = heavy = 0;
+    }
+};
+constexpr int kCtrWords = 11;
+
 // Control block of one single-source launch: zeroed by the host
-// (cudaMemsetAsync) before every launch.  Counters indexed [slot] rotate over
-// levels (slot = level % 3).
+// (cudaMemsetAsync) before every launch.  The level counters rotate (slot =
+// level % 3).
 struct Ctrl {
     BarrierState b;
-    unsigned long long tail[3];      // length of the queue holding frontier `slot`
-    unsigned long long accn[3];      // size of frontier `slot` (bottom-up producer)
-    unsigned long long accm[3];      // degree sum of frontier `slot`
-    unsigned long long scanned[3];   // bottom-up searchers of the level producing frontier `slot`
-    unsigned long long examined[3];  // serial early-exit examinations of that level
-    unsigned long long ntask[3];     // top-down edge-chunk tasks of that level
-    unsigned long long nmiss[3];     // bottom-up first-probe misses left to phase B (miss-list length)
-    unsigned long long nmiss_in[3];  // ... resolved by their chunk's warp in phase A
-    unsigned long long dsum_out[3];  // directed graphs: out-degree sum of frontier `slot`
-    unsigned long long dsum_in[3];   // directed graphs: in-degree sum of frontier `slot`
-    unsigned long long heavy[3];     // top-down: vertices of frontier `slot` above the cluster-level degree cap
+    LevelCtr lv[3];
     // cluster levels (levels run by thread-block cluster 0 alone while the frontier is small)
     unsigned long long clu_gen;      // episodes finished: the waiting CTAs resume when it reaches theirs
     unsigned long long clu_prog;     // last level the cluster started (progress for the waiters' time limit)
@@ -171,31 +181,52 @@ __device__ __forceinline__ void raise_status(BarrierState* c, unsigned code) {
 // The arrival is one acquire-release atomic by thread 0 after the CTA barrier:
 // it publishes the CTA's writes and, for the last arriver, acquires everyone
 // else's; waiters acquire through their polling load.
-__device__ __forceinline__ bool grid_sync(BarrierState* c, unsigned expected, uint64_t timeout_ns) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long old;
-        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(&c->count) : "memory");
-        const unsigned long long target = ((old & ~kAbortBit) / expected + 1ull) * expected;
-        unsigned long long cur = old + 1ull;
-        if (!(cur & kAbortBit) && cur < target) {
-            const uint64_t t0 = globaltimer_ns();
-            unsigned spins = 0;
-            while (true) {
-                cur = ld_acquire64(&c->count);
-                if ((cur & kAbortBit) || cur >= target) break;
-                if (++spins > 32u) {
-                    __nanosleep(32);
-                    if ((spins & 63u) == 0u && globaltimer_ns() - t0 > timeout_ns) {
-                        raise_status(c, kDevTimeout);
-                        cur = kAbortBit;
-                        break;
-                    }
+__device__ __forceinline__ bool grid_wait(BarrierState* c, unsigned expected, uint64_t timeout_ns) {
+    unsigned long long old;
+    asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(&c->count) : "memory");
+    const unsigned long long target = ((old & ~kAbortBit) / expected + 1ull) * expected;
+    unsigned long long cur = old + 1ull;
+    if (!(cur & kAbortBit) && cur < target) {
+        const uint64_t t0 = globaltimer_ns();
+        unsigned spins = 0;
+        while (true) {
+            cur = ld_acquire64(&c->count);
+            if ((cur & kAbortBit) || cur >= target) break;
+            if (++spins > 32u) {
+                __nanosleep(32);
+                if ((spins & 63u) == 0u && globaltimer_ns() - t0 > timeout_ns) {
+                    raise_status(c, kDevTimeout);
+                    cur = kAbortBit;
+                    break;
                 }
             }
         }
-        s_ok = (cur & kAbortBit) ? 0 : 1;
+    }
+    return !(cur & kAbortBit);
+}
+
+__device__ __forceinline__ bool grid_sync(BarrierState* c, unsigned expected, uint64_t timeout_ns) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) s_ok = grid_wait(c, expected, timeout_ns) ? 1 : 0;
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// The barrier, and then `words` counters (at most 32, one line) into shared
+// memory by the first warp of each CTA.  Read by every warp instead, the
+// counters' one L2 line serves 16 times the requests one after another: 2.5 us
+// a counter at 304 CTAs of 16 warps, as long as the barrier itself.
+__device__ __forceinline__ bool grid_sync_read(BarrierState* c, unsigned expected, uint64_t timeout_ns,
+                                               const void* src, void* dst, int words) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) s_ok = grid_wait(c, expected, timeout_ns) ? 1 : 0;
+        __syncwarp();
+        if ((int)threadIdx.x < words)
+            static_cast<unsigned long long*>(dst)[threadIdx.x] =
+                ld_relaxed64(static_cast<const unsigned long long*>(src) + threadIdx.x);
     }
     __syncthreads();
     return s_ok != 0;

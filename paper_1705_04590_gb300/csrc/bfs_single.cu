@@ -140,6 +140,11 @@ struct SingleParams {
 
 constexpr int TD = 0, BU = 1;
 
+// the grid barrier, then the counters of level slot `slot` into the CTA's copy
+__device__ __forceinline__ bool level_sync(const SingleParams& p, int slot, LevelCtr& ctr) {
+    return grid_sync_read(&p.ctrl->b, p.expected, p.timeout_ns, &p.ctrl->lv[slot], &ctr, kCtrWords);
+}
+
 __device__ __forceinline__ int decide_dir(const SingleParams& p, int prev, long long nf, long long mf,
                                           long long mu, int d) {
     switch (p.mode) {
@@ -416,8 +421,8 @@ __device__ void init_phase(const SingleParams& p) {
     }
     if (single && tid == 0) {
         p.queue0[0] = (int)r;
-        p.ctrl->tail[0] = 1ull;
-        p.ctrl->accm[0] = (unsigned long long)deg_of(p, r);
+        p.ctrl->lv[0].tail = 1ull;
+        p.ctrl->lv[0].accm = (unsigned long long)deg_of(p, r);
     }
 }
 
@@ -437,8 +442,8 @@ __device__ void seed_roots_phase(const SingleParams& p) {
             mi += (unsigned long long)(e - s);
         }
     }
-    block_add4(m, mi, 0, 0, &p.ctrl->accm[0], &p.ctrl->dsum_in[0], nullptr, nullptr);
-    if (tid == 0) p.ctrl->tail[0] = (unsigned long long)p.nroots;
+    block_add4(m, mi, 0, 0, &p.ctrl->lv[0].accm, &p.ctrl->lv[0].dsum_in, nullptr, nullptr);
+    if (tid == 0) p.ctrl->lv[0].tail = (unsigned long long)p.nroots;
 }
 
 // ------------------------------------------------------------------ top-down
@@ -604,7 +609,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
                          bool nodeg, unsigned long long& acc_m, unsigned long long& acc_h) {
     const int lane = lane_id();
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
-    unsigned long long* tail = &p.ctrl->tail[snext];
+    unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
     st.nodeg = nodeg;
     st.pf = !nodeg && nf < kPrefetchNf;
@@ -632,7 +637,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
             const int bu = __shfl_sync(kFull, u, L);
             const long long nch = (be - bs + p.td_chunk - 1) / p.td_chunk;
             unsigned long long t0 = 0;
-            if (lane == 0) t0 = atomicAdd(&p.ctrl->ntask[snext], (unsigned long long)nch);
+            if (lane == 0) t0 = atomicAdd(&p.ctrl->lv[snext].ntask, (unsigned long long)nch);
             t0 = __shfl_sync(kFull, t0, 0);
             for (long long c = lane; c < nch; c += 32) {
                 const long long ti = (long long)t0 + c;
@@ -674,7 +679,7 @@ __device__ void task_phase(const SingleParams& p, int d, long long ntask, int* q
                            unsigned long long& acc_m, unsigned long long& acc_h) {
     const int lane = lane_id();
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
-    unsigned long long* tail = &p.ctrl->tail[snext];
+    unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
     st.nodeg = nodeg;
     const long long nt = ntask < p.task_cap ? ntask : p.task_cap;
@@ -1696,19 +1701,7 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
             out.done = done;
             if (lead) {
                 // the grid resumes at level L with every per-level counter slot clear
-                for (int k = 0; k < 3; k++) {
-                    c->tail[k] = 0;
-                    c->accn[k] = 0;
-                    c->accm[k] = 0;
-                    c->scanned[k] = 0;
-                    c->examined[k] = 0;
-                    c->ntask[k] = 0;
-                    c->nmiss[k] = 0;
-                    c->nmiss_in[k] = 0;
-                    c->dsum_out[k] = 0;
-                    c->dsum_in[k] = 0;
-                    c->heavy[k] = 0;
-                }
+                for (int k = 0; k < 3; k++) c->lv[k].zero();
                 c->clu_spill = 0;
                 c->clu_d = out.d;
                 c->clu_nf = nf;
@@ -1805,224 +1798,232 @@ __device__ bool clu_wait(const SingleParams& p, unsigned long long epi, CluState
 
 // ------------------------------------------------------------------ kernel
 
+// State of the level loop, one copy per CTA in shared memory: its thread 0 moves it
+// on after each level.  Held in registers by every thread it would take a third
+// of a thread's 64 from the phases.
+struct LoopState {
+    long long nf, mf, mu, reached;   // frontier size and degree sum, degree sum of the unreached, vertices reached
+    unsigned long long t_start, t_mid;
+    unsigned long long epi;          // cluster episodes so far
+    int d, prev, qsel, bsel;         // level; last direction; which queue / bitmap holds the frontier
+    int no_clu;                      // the level a cluster episode just handed back (the grid takes it)
+};
+
 // kMinId: the launch also makes the parents the minimum-id ones (parent_mode
-// MIN_ID with both arrays there); a variant of its own, so that the passes for it
-// take no registers from the other searches.
-template <bool kMinId>
+// MIN_ID with both arrays there).  kHub: bottom-up steps scan the hub-first rows
+// (p.first is there).  kClu: the launch is in clusters and runs cluster levels.
+// Variants, so that the passes of one take no registers from another (all in
+// one kernel: 24 to 290 bytes of spills per thread; apart: none to 36 without
+// cluster levels).
+template <bool kMinId, bool kHub, bool kClu>
 __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(SingleParams p) {
     Ctrl* c = p.ctrl;
-    __shared__ unsigned s_clu_lv[kMinId ? 8 : 1];   // level bytes that cluster levels discovered
-    if constexpr (kMinId) {
+    __shared__ unsigned s_clu_lv[kMinId && kClu ? 8 : 1];   // level bytes that cluster levels discovered
+    __shared__ LevelCtr s_ctr;                      // the last completed level's counters
+    __shared__ volatile LoopState S;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    if constexpr (kMinId && kClu) {
         if (threadIdx.x < 8) s_clu_lv[threadIdx.x] = 0u;
-        __syncthreads();
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) c->t_enter = globaltimer_ns();
+    if (lead) c->t_enter = globaltimer_ns();
     init_phase(p);
-    if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) c->t_init = globaltimer_ns();
+    if (!level_sync(p, 0, s_ctr)) return;
+    if (lead) c->t_init = globaltimer_ns();
     if (p.nroots == 1 && gtid() == 0) {
         if (p.parent) p.parent[p.root0] = p.root0;
         set_level(p, p.root0, 0);
     }
     if (p.nroots > 1) {
         seed_roots_phase(p);
-        if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+        if (!level_sync(p, 0, s_ctr)) return;
     }
-    long long nf = p.nroots;
-    long long mf = (long long)ld_relaxed64(&c->accm[0]);
-    long long mu = p.nnz - mf;
-    if (p.directed) {
-        // m_u sums in-degrees: the edges a bottom-up step could still examine
-        long long rin = 0;
-        if (p.nroots == 1) {
-            long long s0, e0;
-            bu_row_of(p, p.root0, s0, e0);
-            rin = e0 - s0;
-        } else {
-            rin = (long long)ld_relaxed64(&c->dsum_in[0]);
+    if (threadIdx.x == 0) {
+        S.nf = p.nroots;
+        S.reached = p.nroots;
+        S.mf = (long long)s_ctr.accm;
+        long long rin = (long long)s_ctr.accm;
+        if (p.directed) {
+            // m_u sums in-degrees: the edges a bottom-up step could still examine
+            if (p.nroots == 1) {
+                long long s0, e0;
+                bu_row_of(p, p.root0, s0, e0);
+                rin = e0 - s0;
+            } else {
+                rin = (long long)s_ctr.dsum_in;
+            }
         }
-        mu = p.nnz - rin;
+        S.mu = p.nnz - rin;
+        S.d = 0;
+        S.prev = TD;
+        S.qsel = 0;
+        S.bsel = 0;
+        S.epi = 0;
+        S.no_clu = -1;
+        S.t_start = lead ? globaltimer_ns() : 0;
     }
-    long long reached = nf;
-    int prev = TD, qsel = 0, bsel = 0, d = 0;
-    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    const uint64_t t_start = lead ? globaltimer_ns() : 0;
     // cluster levels only in a launch whose clusters have the size the parameters name
-    const bool clu_on = p.clu_c > 1 && clu_nranks() == (unsigned)p.clu_c;
-    unsigned long long epi = 0;
-    int no_clu = -1;   // the level a cluster episode just handed back (the grid takes it)
+    const bool clu_on = kClu && p.clu_c > 1 && clu_nranks() == (unsigned)p.clu_c;
     while (true) {
-        const int dir = decide_dir(p, prev, nf, mf, mu, d);
-        if (clu_on && dir == TD && prev == TD && d != no_clu && nf <= p.clu_nf && mf <= p.clu_mf &&
-            (d == 0 ? mf <= (long long)p.clu_big : ld_relaxed64(&c->heavy[d % 3]) == 0ull)) {
-            epi++;
+        __syncthreads();   // S is settled
+        const int dir = decide_dir(p, S.prev, S.nf, S.mf, S.mu, S.d);
+        if constexpr (kClu) if (clu_on && dir == TD && S.prev == TD && S.d != S.no_clu && S.nf <= p.clu_nf && S.mf <= p.clu_mf &&
+            (S.d == 0 ? S.mf <= (long long)p.clu_big : s_ctr.heavy == 0ull)) {
             CluState cs;
             if (clu_id() == 0) {
-                cluster_levels(p, qsel ? p.queue1 : p.queue0, d, nf, mf, mu, reached, epi, t_start, cs);
-            } else if (!clu_wait(p, epi, cs)) {
+                cluster_levels(p, S.qsel ? p.queue1 : p.queue0, S.d, S.nf, S.mf, S.mu, S.reached, S.epi + 1, S.t_start, cs);
+            } else if (!clu_wait(p, S.epi + 1, cs)) {
                 return;
             }
-            if constexpr (kMinId) {
-                if (threadIdx.x == 0)
-                    for (int L = d + 1; L <= cs.d; L++) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                if constexpr (kMinId) {
+                    for (int L = S.d + 1; L <= cs.d; L++) {
                         const int b = min(L, (int)kLvDeep);
                         s_clu_lv[b >> 5] |= 1u << (b & 31);
                         if (b == kLvDeep) break;
                     }
+                }
+                S.epi = S.epi + 1;
+                S.d = cs.d;
+                S.reached = cs.reached;
+                S.nf = cs.nf;
+                S.mf = cs.mf;
+                S.mu = cs.mu;
+                S.prev = TD;
+                S.qsel = 0;   // the frontier is back in queue0
+                S.no_clu = cs.d;
             }
-            d = cs.d;
-            reached = cs.reached;
             if (cs.done) break;
-            nf = cs.nf;
-            mf = cs.mf;
-            mu = cs.mu;
-            prev = TD;
-            qsel = 0;   // the frontier is back in queue0
-            no_clu = d;
             continue;
         }
-        const int scur = d % 3, snext = (d + 1) % 3, sfree = (d + 2) % 3;
+        // the level's counters collect in lv[snext]; the slot after it is cleared
+        const int snext = (S.d + 1) % 3;
         if (lead) {
-            c->tail[sfree] = 0;
-            c->accn[sfree] = 0;
-            c->accm[sfree] = 0;
-            c->scanned[sfree] = 0;
-            c->examined[sfree] = 0;
-            c->ntask[sfree] = 0;
-            c->nmiss[sfree] = 0;
-            c->nmiss_in[sfree] = 0;
-            c->dsum_out[sfree] = 0;
-            c->dsum_in[sfree] = 0;
-            c->heavy[sfree] = 0;
+            c->lv[(S.d + 2) % 3].zero();
+            S.t_mid = 0;
         }
-        long long nf_next, scanned = 0, examined = mf, aux = 0, misses = 0;
-        uint64_t t_mid = 0;
-        int* qcur = qsel ? p.queue1 : p.queue0;
-        int* qnext = qsel ? p.queue0 : p.queue1;
-        unsigned* fcur = bsel ? p.front1 : p.front0;
-        unsigned* fnext = bsel ? p.front0 : p.front1;
         if (dir == TD) {
-            if (prev == BU) {
-                bitmap_to_queue(p, fcur, fnext, qcur, &c->tail[scur]);
+            if (S.prev == BU) {
+                bitmap_to_queue(p, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                                S.qsel ? p.queue1 : p.queue0, &c->lv[S.d % 3].tail);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
-            unsigned long long am = 0, ah = 0;
-            unsigned long long* gh = clu_on ? &c->heavy[snext] : nullptr;
-            // a directed graph sums the new frontier's degrees after the level
-            const bool nodeg = p.directed != 0;
-            td_phase(p, d, qcur, nf, qnext, snext, nodeg, am, ah);
-            block_add4(ah, am, 0, 0, gh, &c->accm[snext], nullptr, nullptr);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            const long long nt = (long long)ld_relaxed64(&c->ntask[snext]);
-            aux = nt;
-            if (lead) t_mid = globaltimer_ns();
-            if (nt > 0) {
-                unsigned long long am2 = 0, ah2 = 0;
-                task_phase(p, d, nt, qnext, snext, nodeg, am2, ah2);
-                block_add4(ah2, am2, 0, 0, gh, &c->accm[snext], nullptr, nullptr);
-                if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+            {
+                unsigned long long am = 0, ah = 0;
+                // a directed graph sums the new frontier's degrees after the level
+                td_phase(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, S.qsel ? p.queue0 : p.queue1, snext,
+                         p.directed != 0, am, ah);
+                block_add4(ah, am, 0, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm, nullptr, nullptr);
             }
-            nf_next = (long long)ld_relaxed64(&c->tail[snext]);
+            if (!level_sync(p, snext, s_ctr)) return;
+            if (lead) S.t_mid = globaltimer_ns();
+            if (s_ctr.ntask > 0) {
+                unsigned long long am = 0, ah = 0;
+                task_phase(p, S.d, (long long)s_ctr.ntask, S.qsel ? p.queue0 : p.queue1, snext, p.directed != 0, am, ah);
+                block_add4(ah, am, 0, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm, nullptr, nullptr);
+                if (!level_sync(p, snext, s_ctr)) return;
+            }
             if constexpr (kMinId) {
-                if (nf_next > 0) {
-                    td_min_pass(p, d, qcur, nf, nt);
+                if (s_ctr.tail > 0) {
+                    td_min_pass(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, (long long)s_ctr.ntask);
                     // the next level writes this queue and the task list
                     if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
                 }
             }
-            qsel ^= 1;
         } else {
-            if (prev == TD) {
-                queue_to_bitmap(p, qcur, nf, fcur);
+            if (S.prev == TD) {
+                queue_to_bitmap(p, S.qsel ? p.queue1 : p.queue0, S.nf, S.bsel ? p.front1 : p.front0);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
-            // over the hub-first rows accm[snext] collects the degrees of the searchers
-            // left unvisited (the new frontier's degree sum is m_u minus that), over the
-            // id-ordered rows those of the vertices found
-            unsigned long long an = 0, am = 0, asc = 0, aex = 0;
-            // the queues are idle during bottom-up levels (a preceding queue -> bitmap
-            // conversion ended at the barrier above)
-            int* longlist = qnext;
-            int* misslist = qcur;
-            if (p.first)
-                bu_compact(p, d, fcur, fnext, misslist, &c->nmiss[snext], &c->nmiss_in[snext], longlist,
-                           &c->ntask[snext], an, am, asc, aex);
-            else
-                bu_phase_a(p, d, fcur, fnext, longlist, &c->ntask[snext], an, am, asc, aex);
-            block_add4(an, am, asc, aex, &c->accn[snext], &c->accm[snext], &c->scanned[snext],
-                       &c->examined[snext]);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            if (lead) t_mid = globaltimer_ns();
-            if (p.first) {
-                const long long nmiss = (long long)ld_relaxed64(&c->nmiss[snext]);
-                misses = nmiss + (long long)ld_relaxed64(&c->nmiss_in[snext]);
-                if (nmiss > 0) {
+            // over the hub-first rows accm collects the degrees of the searchers left
+            // unvisited (the new frontier's degree sum is m_u minus that), over the
+            // id-ordered rows those of the vertices found.  The queues are idle during
+            // bottom-up levels (a preceding queue -> bitmap conversion ended at the
+            // barrier above): one holds the long list, the other the miss list
+            {
+                unsigned long long an = 0, am = 0, asc = 0, aex = 0;
+                if constexpr (kHub)
+                    bu_compact(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                               S.qsel ? p.queue1 : p.queue0, &c->lv[snext].nmiss, &c->lv[snext].nmiss_in,
+                               S.qsel ? p.queue0 : p.queue1, &c->lv[snext].ntask, an, am, asc, aex);
+                else
+                    bu_phase_a(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                               S.qsel ? p.queue0 : p.queue1, &c->lv[snext].ntask, an, am, asc, aex);
+                block_add4(an, am, asc, aex, &c->lv[snext].accn, &c->lv[snext].accm, &c->lv[snext].scanned,
+                           &c->lv[snext].examined);
+            }
+            if (!level_sync(p, snext, s_ctr)) return;
+            if (lead) S.t_mid = globaltimer_ns();
+            if constexpr (kHub) {
+                if (s_ctr.nmiss > 0) {
                     unsigned long long bn = 0, bm = 0, bex = 0;
-                    bu_misses(p, d, fcur, fnext, misslist, nmiss, longlist, &c->ntask[snext], bn, bm, bex);
-                    block_add4(bn, bm, 0, bex, &c->accn[snext], &c->accm[snext], nullptr, &c->examined[snext]);
-                    if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+                    bu_misses(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                              S.qsel ? p.queue1 : p.queue0, (long long)s_ctr.nmiss, S.qsel ? p.queue0 : p.queue1,
+                              &c->lv[snext].ntask, bn, bm, bex);
+                    block_add4(bn, bm, 0, bex, &c->lv[snext].accn, &c->lv[snext].accm, nullptr, &c->lv[snext].examined);
+                    if (!level_sync(p, snext, s_ctr)) return;
                 }
             }
-            const long long nlong = (long long)ld_relaxed64(&c->ntask[snext]);
-            aux = nlong;
-            if (nlong > 0) {
+            if (s_ctr.ntask > 0) {
                 unsigned long long bn = 0, bm = 0, bex = 0;
-                bu_phase_b(p, d, fcur, fnext, longlist, nlong, p.first ? kHead : kWin, p.first != nullptr, bn, bm,
-                           bex);
-                block_add4(bn, bm, 0, bex, &c->accn[snext], &c->accm[snext], nullptr, &c->examined[snext]);
-                if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+                bu_phase_b(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                           S.qsel ? p.queue0 : p.queue1, (long long)s_ctr.ntask, kHub ? kHead : kWin, kHub, bn, bm, bex);
+                block_add4(bn, bm, 0, bex, &c->lv[snext].accn, &c->lv[snext].accm, nullptr, &c->lv[snext].examined);
+                if (!level_sync(p, snext, s_ctr)) return;
             }
-            nf_next = (long long)ld_relaxed64(&c->accn[snext]);
-            scanned = (long long)ld_relaxed64(&c->scanned[snext]);
-            examined = (long long)ld_relaxed64(&c->examined[snext]);
-            bsel ^= 1;
         }
-        const long long macc = (long long)ld_relaxed64(&c->accm[snext]);
-        long long mf_next = (dir == BU && p.first) ? mu - macc : macc;
-        long long mu_drop = mf_next;   // undirected: in- and out-degree sums coincide
+        // the new frontier: a queue (the one written) after a top-down level, else a bitmap
         if (p.directed) {
             unsigned long long so = 0, si = 0;
             if (dir == TD)
-                frontier_degree_sums(p, qsel ? p.queue1 : p.queue0, nf_next, nullptr, so, si);
+                frontier_degree_sums(p, S.qsel ? p.queue0 : p.queue1, (long long)s_ctr.tail, nullptr, so, si);
             else
-                frontier_degree_sums(p, nullptr, 0, bsel ? p.front1 : p.front0, so, si);
-            block_add4(so, si, 0, 0, &c->dsum_out[snext], &c->dsum_in[snext], nullptr, nullptr);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            mf_next = (long long)ld_relaxed64(&c->dsum_out[snext]);
-            mu_drop = (long long)ld_relaxed64(&c->dsum_in[snext]);
+                frontier_degree_sums(p, nullptr, 0, S.bsel ? p.front0 : p.front1, so, si);
+            block_add4(so, si, 0, 0, &c->lv[snext].dsum_out, &c->lv[snext].dsum_in, nullptr, nullptr);
+            if (!level_sync(p, snext, s_ctr)) return;
         }
-        if (lead && d < p.rec_cap) {
-            bfs_level_record r;
-            r.dir = dir;
-            r.misses = (int)misses;
-            r.nf = nf;
-            r.mf = mf;
-            r.nnext = nf_next;
-            r.mnext = mf_next;
-            r.scanned = scanned;
-            r.examined = examined;
-            r.t_ns = (long long)(globaltimer_ns() - t_start);
-            r.aux = aux;
-            r.t_mid_ns = t_mid ? (long long)(t_mid - t_start) : 0;
-            p.rec[d] = r;
+        const long long nf_next = (long long)(dir == TD ? s_ctr.tail : s_ctr.accn);
+        if (threadIdx.x == 0) {
+            const long long macc = (long long)s_ctr.accm;
+            const long long mf_next = p.directed ? (long long)s_ctr.dsum_out : (kHub && dir == BU) ? S.mu - macc : macc;
+            if (lead && S.d < p.rec_cap) {
+                bfs_level_record r;
+                r.dir = dir;
+                r.misses = kHub && dir == BU ? (int)(s_ctr.nmiss + s_ctr.nmiss_in) : 0;
+                r.nf = S.nf;
+                r.mf = S.mf;
+                r.nnext = nf_next;
+                r.mnext = mf_next;
+                r.scanned = dir == BU ? (long long)s_ctr.scanned : 0;
+                r.examined = dir == BU ? (long long)s_ctr.examined : S.mf;
+                r.t_ns = (long long)(globaltimer_ns() - S.t_start);
+                r.aux = (long long)s_ctr.ntask;
+                r.t_mid_ns = S.t_mid ? (long long)(S.t_mid - S.t_start) : 0;
+                p.rec[S.d] = r;
+            }
+            if (nf_next > 0) {
+                S.reached = S.reached + nf_next;
+                // what the unreached lose: in-degrees (undirected: both sums coincide)
+                S.mu = S.mu - (p.directed ? (long long)s_ctr.dsum_in : mf_next);
+                S.nf = nf_next;
+                S.mf = mf_next;
+                if (dir == TD) S.qsel = S.qsel ^ 1;
+                else S.bsel = S.bsel ^ 1;
+                S.prev = dir;
+                S.d = S.d + 1;
+            }
         }
         if (nf_next == 0) break;
-        reached += nf_next;
-        mu -= mu_drop;
-        nf = nf_next;
-        mf = mf_next;
-        prev = dir;
-        d++;
     }
     if (lead) {
-        c->num_levels = d + 1;
-        c->reached = reached;
+        c->num_levels = S.d + 1;
+        c->reached = S.reached;
         c->t_levels = globaltimer_ns();
     }
     // every level ended at a grid barrier, so all staged bytes are visible here
-    if constexpr (kMinId) {
-        if (epi > 0) {
-            __syncthreads();
+    if constexpr (kMinId && kClu) {
+        __syncthreads();
+        if (S.epi > 0) {
             min_parent_rows(p, s_clu_lv);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
         }
@@ -2035,6 +2036,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             c->t_done = globaltimer_ns();
     }
 }
+
 
 // ------------------------------------------------------------------ DCSC tiles
 
@@ -2065,7 +2067,7 @@ __device__ void td_dcsc_phase(const SingleParams& p, int d, const int* qcur, lon
         if (min_id) s_old[w] = x;
     }
     __syncthreads();
-    unsigned long long* tail = &p.ctrl->tail[snext];
+    unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage_dcsc();
     const int wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
     for (long long base = (long long)wib * 32; base < nf; base += (long long)nwb * 32) {
@@ -2235,18 +2237,19 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
     unsigned* s_own = dyn;
     unsigned* s_seg = dyn + p.Bw;
     Ctrl* c = p.ctrl;
+    __shared__ LevelCtr s_ctr;   // the last completed level's counters
     init_phase(p);
-    if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+    if (!level_sync(p, 0, s_ctr)) return;
     if (p.nroots == 1 && gtid() == 0) {
         if (p.parent) p.parent[p.root0] = p.root0;
         if (p.level) p.level[p.root0] = 0;
     }
     if (p.nroots > 1) {
         seed_roots_phase(p);
-        if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+        if (!level_sync(p, 0, s_ctr)) return;
     }
     long long nf = p.nroots;
-    long long mf = (long long)ld_relaxed64(&c->accm[0]);
+    long long mf = (long long)s_ctr.accm;
     long long mu = p.nnz - mf;
     long long reached = nf;
     int prev = TD, qsel = 0, bsel = 0, d = 0;
@@ -2255,14 +2258,7 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
     while (true) {
         const int dir = decide_dir(p, prev, nf, mf, mu, d);
         const int scur = d % 3, snext = (d + 1) % 3, sfree = (d + 2) % 3;
-        if (lead) {
-            c->tail[sfree] = 0;
-            c->accn[sfree] = 0;
-            c->accm[sfree] = 0;
-            c->scanned[sfree] = 0;
-            c->examined[sfree] = 0;
-            c->ntask[sfree] = 0;
-        }
+        if (lead) c->lv[sfree].zero();
         long long nf_next, scanned = 0, examined = mf;
         int* qcur = qsel ? p.queue1 : p.queue0;
         int* qnext = qsel ? p.queue0 : p.queue1;
@@ -2270,14 +2266,14 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
         unsigned* fnext = bsel ? p.front0 : p.front1;
         if (dir == TD) {
             if (prev == BU) {
-                bitmap_to_queue(p, fcur, fnext, qcur, &c->tail[scur]);
+                bitmap_to_queue(p, fcur, fnext, qcur, &c->lv[scur].tail);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             unsigned long long am = 0;
             td_dcsc_phase(p, d, qcur, nf, qnext, snext, s_own, s_seg, am);
-            block_add4(0, am, 0, 0, nullptr, &c->accm[snext], nullptr, nullptr);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            nf_next = (long long)ld_relaxed64(&c->tail[snext]);
+            block_add4(0, am, 0, 0, nullptr, &c->lv[snext].accm, nullptr, nullptr);
+            if (!level_sync(p, snext, s_ctr)) return;
+            nf_next = (long long)s_ctr.tail;
             qsel ^= 1;
         } else {
             if (prev == TD) {
@@ -2286,14 +2282,14 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
             }
             unsigned long long an = 0, am = 0, asc = 0, aex = 0;
             bu_dcsc_phase(p, d, fcur, fnext, s_own, s_seg, an, am, asc, aex);
-            block_add4(an, am, asc, aex, &c->accn[snext], &c->accm[snext], &c->scanned[snext], &c->examined[snext]);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            nf_next = (long long)ld_relaxed64(&c->accn[snext]);
-            scanned = (long long)ld_relaxed64(&c->scanned[snext]);
-            examined = (long long)ld_relaxed64(&c->examined[snext]);
+            block_add4(an, am, asc, aex, &c->lv[snext].accn, &c->lv[snext].accm, &c->lv[snext].scanned, &c->lv[snext].examined);
+            if (!level_sync(p, snext, s_ctr)) return;
+            nf_next = (long long)s_ctr.accn;
+            scanned = (long long)s_ctr.scanned;
+            examined = (long long)s_ctr.examined;
             bsel ^= 1;
         }
-        const long long mf_next = (long long)ld_relaxed64(&c->accm[snext]);
+        const long long mf_next = (long long)s_ctr.accm;
         if (lead && d < p.rec_cap) {
             bfs_level_record r;
             r.dir = dir;
@@ -2371,20 +2367,34 @@ using bfsk::Ctrl;
 using bfsk::SingleParams;
 using bfsk::Task;
 
-// the CSR kernel's variant (kMinId)
-static const void* csr_kernel(bool min_id) {
-    return min_id ? (const void*)bfsk::bfs_single_kernel<true> : (const void*)bfsk::bfs_single_kernel<false>;
+// the CSR kernel's variants: any parent over the id-ordered rows, over the hub-first
+// rows, and minimum-id parents (id-ordered rows only); each without and with
+// cluster levels
+enum CsrVariant { kCsrId, kCsrHub, kCsrMin, kCsrVariants };
+static const void* csr_kernel(int variant, bool clu) {
+    using namespace bfsk;
+    switch (variant) {
+        case kCsrHub:
+            return clu ? (const void*)bfs_single_kernel<false, true, true>
+                       : (const void*)bfs_single_kernel<false, true, false>;
+        case kCsrMin:
+            return clu ? (const void*)bfs_single_kernel<true, false, true>
+                       : (const void*)bfs_single_kernel<true, false, false>;
+        default:
+            return clu ? (const void*)bfs_single_kernel<false, false, true>
+                       : (const void*)bfs_single_kernel<false, false, false>;
+    }
 }
 
-// resident CTAs per SM of the CSR kernel: of the variant that fits fewer
+// resident CTAs per SM of the CSR kernel: of the variant that fits fewest
 static cudaError_t csr_occupancy(int* per_sm) {
     *per_sm = INT_MAX;
-    for (bool m : {false, true}) {
+    for (int m = 0; m < 2 * kCsrVariants; m++) {
+        const void* fn = csr_kernel(m >> 1, m & 1);
         int nb = 0;
-        cudaError_t e = cudaFuncSetAttribute(csr_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)bfsk::kSingleDynSmem);
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bfsk::kSingleDynSmem);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, csr_kernel(m), bfsk::kBlock, bfsk::kSingleDynSmem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, bfsk::kBlock, bfsk::kSingleDynSmem);
         if (e != cudaSuccess) return e;
         *per_sm = std::min(*per_sm, nb);
     }
@@ -2574,10 +2584,10 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
             cfg.attrs = at;
             cfg.numAttrs = 1;
             int ncl = INT_MAX;
-            for (bool m : {false, true}) {
+            for (int m = 0; m < kCsrVariants; m++) {
                 int k = 0;
-                BFS_CUDA_TRY(cudaFuncSetAttribute(csr_kernel(m), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-                BFS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&k, csr_kernel(m), &cfg));
+                BFS_CUDA_TRY(cudaFuncSetAttribute(csr_kernel(m, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+                BFS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&k, csr_kernel(m, true), &cfg));
                 ncl = std::min(ncl, k);
             }
             w.clu_grid[li] = ncl > 0 ? ncl * C : -1;
@@ -2596,7 +2606,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         p.clu_nf = (long long)C * (bfsk::kCluCap / 2);
         p.clu_mf = (long long)C * bfsk::kCluEdgesPerCta;
     }
-    const bool min_id = opt.parent_mode == BFS_PARENT_MIN_ID && parent;
+    const int variant = opt.parent_mode == BFS_PARENT_MIN_ID && parent ? kCsrMin : p.first ? kCsrHub : kCsrId;
     void* args[] = {&p};
     BFS_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(Ctrl), s));
     if (k > 1) BFS_CUDA_TRY(cudaMemcpyAsync(w.queue0, roots_host, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, s));
@@ -2615,10 +2625,10 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         cfg.stream = s;
         cfg.attrs = at;
         cfg.numAttrs = 2;
-        BFS_CUDA_TRY(cudaLaunchKernelExC(&cfg, csr_kernel(min_id), args));
+        BFS_CUDA_TRY(cudaLaunchKernelExC(&cfg, csr_kernel(variant, true), args));
         return BFS_OK;
     }
-    const void* fn = dcsc ? (const void*)bfsk::bfs_dcsc_kernel : csr_kernel(min_id);
+    const void* fn = dcsc ? (const void*)bfsk::bfs_dcsc_kernel : csr_kernel(variant, false);
     BFS_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, dyn, s));
     return BFS_OK;
 }
@@ -2754,7 +2764,7 @@ extern "C" bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int3
     BFS_CUDA_TRY(cudaGetLastError());
     BFS_CUDA_TRY(cudaMemsetAsync(p.ctrl, 0, sizeof(bfsk::Ctrl), s));
     void* args[] = {&p};
-    BFS_CUDA_TRY(cudaLaunchCooperativeKernel(csr_kernel(false), dim3(grid), dim3(bfsk::kBlock),
+    BFS_CUDA_TRY(cudaLaunchCooperativeKernel(csr_kernel(kCsrId, false), dim3(grid), dim3(bfsk::kBlock),
                                              args, bfsk::kSingleDynSmem, s));
     return BFS_OK;
 }
