@@ -287,6 +287,12 @@ __device__ __forceinline__ int get_level(const SingleParams& p, int u) {
 __device__ __forceinline__ long long gtid() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ long long gthreads() { return (long long)gridDim.x * blockDim.x; }
 
+// This warp's number in the grid, counted across the CTAs first: the first few
+// warps of a small frontier or bitmap then sit on as many SMs.
+__device__ __forceinline__ long long spread_warp() {
+    return (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+}
+
 // Fill a[0..n) with -1, using 16-byte stores for the aligned body.
 __device__ void fill_minus_one(int* a, long long n) {
     const long long tid = gtid(), nth = gthreads();
@@ -608,7 +614,7 @@ __device__ __forceinline__ WarpStage warp_stage_dcsc() { return warp_stage_in(g_
 __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long long nf, int* qnext, int snext,
                          bool nodeg, unsigned long long& acc_m, unsigned long long& acc_h) {
     const int lane = lane_id();
-    const long long gw = gtid() >> 5, nw = gthreads() >> 5;
+    const long long gw = spread_warp(), nw = gthreads() >> 5;
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
     st.nodeg = nodeg;
@@ -969,7 +975,17 @@ __device__ __forceinline__ void long_flush(WarpStage& st, int* longlist, unsigne
     st.cnt = 0;
 }
 
-// Bottom-up, phase A.  A warp takes 32 completed-bitmap words (1024
+// Bitmap words that a warp takes at a time in a bottom-up sweep: 32 (a word per
+// lane) on bitmaps with that many for every warp of the grid, down to one on small
+// ones, whose sweep would otherwise be the work of a few warps (R-MAT 12: 4 of
+// 4864; its dense level 50 us with 32 words, 13 us with one).
+__device__ __forceinline__ int bu_chunk_words(long long W, long long nwarps) {
+    int k = 32;
+    while (k > 1 && (long long)k * nwarps > W) k >>= 1;
+    return k;
+}
+
+// Bottom-up, phase A.  A warp takes up to 32 completed-bitmap words (1024
 // vertices) at a time and compacts the unvisited ones with a warp prefix sum;
 // each lane then handles one searcher per round: its row offsets, one aligned
 // window of 8 ids (two int4 loads) and 8 frontier probes.  The rounds are
@@ -979,7 +995,7 @@ __device__ __forceinline__ void long_flush(WarpStage& st, int* longlist, unsigne
 // whose row continues past the window without a hit goes on the long list
 // (phase B).  Found vertices are collected per word in shared memory and
 // written as whole next-frontier / completed words (the warp owns its words).
-__device__ __forceinline__ int bu_locate(int k, int T, int incl, int excl, unsigned todo, long long ch) {
+__device__ __forceinline__ int bu_locate(int k, int T, int incl, int excl, unsigned todo, long long wbase) {
     int j = 0;
 #pragma unroll
     for (int step = 16; step >= 1; step >>= 1) {
@@ -989,7 +1005,7 @@ __device__ __forceinline__ int bu_locate(int k, int T, int incl, int excl, unsig
     const int exj = __shfl_sync(kFull, excl, j);
     const unsigned tj = __shfl_sync(kFull, todo, j);
     if (k >= T) return -1;
-    return (int)((ch * 32 + j) * 32 + (long long)__fns(tj, 0, k - exj + 1));
+    return (int)((wbase + j) * 32 + (long long)__fns(tj, 0, k - exj + 1));
 }
 
 __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, unsigned* fnext, int* longlist,
@@ -997,22 +1013,23 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
                            unsigned long long& acc_sc, unsigned long long& acc_ex) {
     __shared__ unsigned s_next[kBlock / 32][32];
     const int lane = lane_id(), wib = threadIdx.x >> 5;
-    const long long nchunk = (p.W + 31) / 32;
     const int4 z4 = make_int4(0, 0, 0, 0);
     s_next[wib][lane] = 0u;
     WarpStage lst = warp_stage();   // long-list entries, appended in batches
     __syncwarp();
-    const long long gw = gtid() >> 5, nw = gthreads() >> 5;
-    for (long long ch = gw; ch < nchunk; ch += nw) {
-        const long long w = ch * 32 + lane;
-        const unsigned cw = (w < p.W) ? __ldcg(p.visited + w) : kFull;
+    const long long gw = spread_warp(), nw = gthreads() >> 5;
+    const int cwords = bu_chunk_words(p.W, nw);
+    for (long long wbase = gw * cwords; wbase < p.W; wbase += nw * cwords) {
+        const long long w = wbase + lane;
+        const bool own = lane < cwords && w < p.W;
+        const unsigned cw = own ? __ldcg(p.visited + w) : kFull;
         const unsigned todo = ~cw;
         const int cnt = __popc(todo);
         const int incl = warp_inclusive_scan(cnt);
         const int T = __shfl_sync(kFull, incl, 31);
         const int excl = incl - cnt;
         // pipeline prologue: round 0 offsets + window, round 1 offsets
-        int u0 = bu_locate(lane, T, incl, excl, todo, ch);
+        int u0 = bu_locate(lane, T, incl, excl, todo, wbase);
         long long s0 = 0, e0 = 0;
         if (u0 >= 0) {
             bu_row_of_stream(p, u0, s0, e0);
@@ -1023,14 +1040,14 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
             xa0 = ld_stream4(src);
             if (kWin == 8 && (s0 & ~3LL) + 4 < e0) xb0 = ld_stream4(src + 1);
         }
-        int u1 = bu_locate(32 + lane, T, incl, excl, todo, ch);
+        int u1 = bu_locate(32 + lane, T, incl, excl, todo, wbase);
         long long s1 = 0, e1 = 0;
         if (u1 >= 0) {
             bu_row_of_stream(p, u1, s1, e1);
         }
         for (int base = 0; base < T; base += 32) {
             // round r+2: offsets
-            const int u2 = bu_locate(base + 64 + lane, T, incl, excl, todo, ch);
+            const int u2 = bu_locate(base + 64 + lane, T, incl, excl, todo, wbase);
             long long s2 = 0, e2 = 0;
             if (u2 >= 0) {
                 bu_row_of_stream(p, u2, s2, e2);
@@ -1068,7 +1085,7 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
                     acc_m += (unsigned long long)(e0 - s0);
                     if (p.parent) p.parent[u0] = pick(ids, t);
                     set_level(p, u0, d + 1);
-                    atomicOr(&s_next[wib][(u0 >> 5) - ch * 32], 1u << (u0 & 31));
+                    atomicOr(&s_next[wib][(u0 >> 5) - wbase], 1u << (u0 & 31));
                 } else if (rb + kWin < e0) {
                     to_long = true;       // examinations counted by phase B
                 } else {
@@ -1092,7 +1109,7 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
         }
         __syncwarp();
         const unsigned nx = s_next[wib][lane];
-        if (w < p.W) {
+        if (own) {
             fnext[w] = nx;
             if (nx) p.visited[w] = cw | nx;
         }
@@ -1145,7 +1162,7 @@ constexpr int kInlineMisses = BFS_INLINE_MISSES;
 // so no global atomics, and kept out of `pfirst`: these parents are stored); a
 // row that goes on is appended to the long list (phase C resumes it at 7).
 __device__ __forceinline__ void chunk_misses(const SingleParams& p, int d, const unsigned* fcur, WarpStage& st,
-                                             unsigned* cmiss, long long ch, int* longlist, unsigned long long* longcnt,
+                                             unsigned* cmiss, long long wbase, int* longlist, unsigned long long* longcnt,
                                              unsigned long long& acc_left, unsigned long long& acc_ex) {
     const int lane = lane_id();
     __syncwarp();
@@ -1175,7 +1192,7 @@ __device__ __forceinline__ void chunk_misses(const SingleParams& p, int d, const
                     acc_ex += (unsigned long long)(t + 1);
                     if (p.parent) p.parent[v] = pick(ids, t);
                     set_level(p, v, d + 1);
-                    atomicOr(cmiss + ((v >> 5) - ch * 32), 1u << (v & 31));
+                    atomicOr(cmiss + ((v >> 5) - wbase), 1u << (v & 31));
                 } else if (deg > kHead) {
                     to_long = true;       // examinations counted by phase C
                 } else {
@@ -1206,15 +1223,16 @@ __device__ void bu_compact(const SingleParams& p, int d, const unsigned* fcur, u
     s_cmiss[threadIdx.x >> 5][lane_id()] = 0u;
     const int lane = lane_id(), wib = threadIdx.x >> 5;
     unsigned short* list = g_list[wib];
-    const long long nchunk = (p.W + 31) / 32;
     s_cnext[wib][lane] = 0u;
     WarpStage mst = warp_stage();
     unsigned long long nmiss_w = 0;   // warp-uniform
     __syncwarp();
-    const long long gw = gtid() >> 5, nw = gthreads() >> 5;
-    for (long long ch = gw; ch < nchunk; ch += nw) {
-        const long long w = ch * 32 + lane;
-        const unsigned cw = (w < p.W) ? __ldcg(p.visited + w) : kFull;
+    const long long gw = spread_warp(), nw = gthreads() >> 5;
+    const int cwords = bu_chunk_words(p.W, nw);
+    for (long long wbase = gw * cwords; wbase < p.W; wbase += nw * cwords) {
+        const long long w = wbase + lane;
+        const bool own = lane < cwords && w < p.W;
+        const unsigned cw = own ? __ldcg(p.visited + w) : kFull;
         unsigned todo = ~cw;
         const int cnt = __popc(todo);
         const int incl = warp_inclusive_scan(cnt);
@@ -1226,7 +1244,7 @@ __device__ void bu_compact(const SingleParams& p, int d, const unsigned* fcur, u
             list[pos++] = (unsigned short)(lane * 32 + b);
         }
         __syncwarp();
-        const long long vbase = ch * 1024;
+        const long long vbase = wbase * 32;
         // round r's searcher: vertex vbase + list[32 r + lane], or none past T
         auto who = [&](int r) -> int { const int k = 32 * r + lane; return k < T ? (int)(vbase + list[k]) : -1; };
         auto plane = [&](int u) -> int { return u >= 0 ? ld_stream32(p.first + u) : 0; };
@@ -1247,7 +1265,7 @@ __device__ void bu_compact(const SingleParams& p, int d, const unsigned* fcur, u
                 if (hit) {
                     set_level(p, u0, d + 1);
                     if (!p.pfirst && p.parent) p.parent[u0] = f0 & (int)~kMore;
-                    atomicOr(&s_cnext[wib][(u0 >> 5) - ch * 32], 1u << (u0 & 31));
+                    atomicOr(&s_cnext[wib][(u0 >> 5) - wbase], 1u << (u0 & 31));
                 } else if (!miss) {
                     acc_left += 1;
                 }
@@ -1267,13 +1285,13 @@ __device__ void bu_compact(const SingleParams& p, int d, const unsigned* fcur, u
             long_flush(mst, misslist, misscnt);
         } else if (mst.cnt > 0) {
             nmiss_w += (unsigned long long)mst.cnt;
-            chunk_misses(p, d, fcur, mst, s_cmiss[wib], ch, longlist, longcnt, acc_left, acc_ex);
+            chunk_misses(p, d, fcur, mst, s_cmiss[wib], wbase, longlist, longcnt, acc_left, acc_ex);
         }
         __syncwarp();
         const unsigned nf = s_cnext[wib][lane];   // first-probe hits: parent = the plane entry
         const unsigned nx = nf | s_cmiss[wib][lane];
         s_cmiss[wib][lane] = 0u;
-        if (w < p.W) {
+        if (own) {
             fnext[w] = nx;
             if (nx) {
                 p.visited[w] = cw | nx;

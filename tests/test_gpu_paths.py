@@ -83,3 +83,30 @@ def test_multi_rows_and_parents(gpu_lib, shape, k):
             assert np.array_equal(level.cpu().numpy().reshape(k, e.n), want), (mode, rows)
             assert np.array_equal(parent.cpu().numpy().reshape(k, e.n), pmin), (mode, rows)
     g.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4096, 4097, 40_000, 155_649, 320_001])
+@pytest.mark.parametrize("hub", [False, True])
+def test_bottom_up_chunk_widths(gpu_lib, n, hub):
+    """Bottom-up sweeps whose warps take 1 to 32 bitmap words each (the width follows the
+    bitmap's size), with a ragged last word: levels, parents and the searchers' counts."""
+    bfs = gpu_lib
+    e = graphgen.erdos_renyi(n, 4 * n, seed=n) if n > 1 else graphgen.from_pairs(1, [(0, 0)])
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    scan = oracle.hub_first(ref) if hub else ref
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, hub_first=hub)
+    level, parent = _buffers(e.n)
+    rows = bfs.BU_ROWS_HUB_FIRST if hub else bfs.BU_ROWS_BY_ID
+    for root in ([0, n // 2] if n > 1 else [0]):
+        want = oracle.levels(ref, root)
+        for mode, omode in ((bfs.MODE_BU_ONLY, oracle.MODE_BU), (bfs.MODE_DO, oracle.MODE_DO)):
+            info = g.run(root, parent=parent, level=level, opts=bfs.options(mode=mode, bu_rows=rows), stats=True,
+                         record_levels=256)
+            lv = level.cpu().numpy()
+            assert np.array_equal(lv, want), (root, mode)
+            assert oracle.certify(ref, root, lv, parent.cpu().numpy(), labels) == (0, -1), (root, mode)
+            s = oracle.do_schedule(scan, want, omode)
+            for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext", "scanned", "examined"]):
+                assert np.array_equal(info["records"][:, col], getattr(s, name)), (root, mode, name)
+    g.close()
