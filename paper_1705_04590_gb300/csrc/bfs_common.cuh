@@ -34,25 +34,29 @@ struct BarrierState {
 };
 constexpr unsigned long long kAbortBit = 1ull << 63;
 
-// Counters of one level, one 128-byte line: a CTA reads them with one request
-// after the barrier that completes them (grid_sync_read).
-struct __align__(128) LevelCtr {
+// Counters of one level, two 128-byte lines: a CTA reads them with one request
+// each after the barrier that completes them (grid_sync_read).
+constexpr int kHubClasses = 13;
+struct __align__(256) LevelCtr {
     unsigned long long tail;       // length of the queue holding the slot's frontier
     unsigned long long accn;       // size of the frontier (bottom-up producer)
     unsigned long long accm;       // degree sum of the frontier
     unsigned long long scanned;    // bottom-up searchers of the level producing it
     unsigned long long examined;   // serial early-exit examinations of that level
-    unsigned long long ntask;      // top-down edge-chunk tasks of that level
+    unsigned long long ntask;      // bottom-up: length of that level's long list
     unsigned long long nmiss;      // bottom-up first-probe misses left to phase B (miss-list length)
     unsigned long long nmiss_in;   // ... resolved by their chunk's warp in phase A
     unsigned long long dsum_out;   // directed graphs: out-degree sum of the frontier
     unsigned long long dsum_in;    // directed graphs: in-degree sum of the frontier
     unsigned long long heavy;      // top-down: its vertices above the cluster-level degree cap
+    unsigned long long pad[5];
+    unsigned long long hubs[kHubClasses];   // top-down: rows of that level cut into 4^class slices
     __host__ __device__ void zero() {
+        for (int j = 0; j < kHubClasses; j++) hubs[j] = 0;
         tail = accn = accm = scanned = examined = ntask = nmiss = nmiss_in = dsum_out = dsum_in = heavy = 0;
     }
 };
-constexpr int kCtrWords = 11;
+constexpr int kCtrWords = 16 + kHubClasses;
 
 // Control block of one single-source launch: zeroed by the host
 // (cudaMemsetAsync) before every launch.  The level counters rotate (slot =

@@ -14,9 +14,9 @@
 //              for u in the queue, for v in adj(u): claim v by an atomicOr on
 //              the visited bitmap; the winner writes parent/level and appends
 //              v to the next queue (warp ballot + one atomicAdd per warp).
-//              Frontier vertices of degree > big_deg are cut into edge chunks
+//              Frontier vertices of degree > big_deg are cut into slices
 //              that all warps share after a barrier (load balance on R-MAT
-//              hubs); the rest are gathered warp-cooperatively (a warp prefix
+//              hubs), taken in the order of the targets they hold; the rest are gathered warp-cooperatively (a warp prefix
 //              sum over its 32 vertices' degrees maps lanes onto edges).
 //   bottom-up (Algorithm 2 inner loops; the local search of Algorithm 4):
 //              a warp owns 32 consecutive vertices (one word of the
@@ -49,9 +49,9 @@ namespace bfsk {
 constexpr int kBlock = BFS_BLOCK;  // CSR kernel
 constexpr int kDBlock = 1024;   // DCSC kernel (one CTA per vertex block)
 constexpr int kWarps = 32;      // shared-memory per-warp arrays sized for up to 1024 threads
-constexpr int kChunk = 256;    // edges per top-down chunk task of the allocation-free entry point
+constexpr int kChunk = 256;    // td_chunk of the allocation-free entry point
 constexpr int kDefaultChunk = 128;   // default of options.td_chunk (measured best at R-MAT 26)
-constexpr int kMinChunk = 64;  // smallest chunk task: the task lists are sized for it
+constexpr int kMinChunk = 64;  // smallest options.td_chunk and td_big_degree: the hub lists are sized for them
 constexpr int kStage = 256;    // per-warp shared-memory staging of next-queue entries
 
 // Shared memory that phases of the CSR kernel borrow in turn: the top-down
@@ -70,9 +70,10 @@ constexpr long long kPrefetchNf = 1 << 16;   // top-down levels below this prefe
 constexpr unsigned kFull = 0xffffffffu;
 constexpr size_t kSingleDynSmem = 0;   // the CSR kernel uses static shared memory only
 
-struct Task {
-    long long start;
-    int len;
+// a frontier row that all warps share (top-down)
+struct Hub {
+    long long start;   // its first column index
+    int len;           // its degree
     int u;
 };
 
@@ -110,15 +111,17 @@ struct SingleParams {
     unsigned* front1;
     int* queue0;
     int* queue1;
-    Task* tasks;
-    long long task_cap;
+    // rows shared by all warps, by class j: rows of 4^j to 4^(j+1) - 1 chunks of
+    // td_chunk edges at hubs[hub_off[j]..hub_off[j + 1])
+    Hub* hubs;
+    long long hub_off[kHubClasses + 1];
     Ctrl* ctrl;
     bfs_level_record* rec;
     int rec_cap;
     int root0;     // the root when nroots == 1
     int nroots;    // > 1: roots already copied into queue0[0..nroots)
     int mode, alpha, beta, parent_mode, big_deg;
-    int td_chunk;      // edges per top-down chunk task (>= kMinChunk)
+    int td_chunk;      // edges of a hub row's shortest slice (>= kMinChunk)
     // cluster levels: CTAs per thread-block cluster of the launch (1 = none);
     // cluster 0 runs a top-down level alone while the frontier holds at most
     // clu_nf vertices and clu_mf edges and no vertex of degree above clu_big
@@ -611,6 +614,76 @@ __device__ __forceinline__ WarpStage warp_stage_in(int* buf) {
 __device__ __forceinline__ WarpStage warp_stage() { return warp_stage_in(g_stage[threadIdx.x >> 5]); }
 __device__ __forceinline__ WarpStage warp_stage_dcsc() { return warp_stage_in(g_stage_d[threadIdx.x >> 5]); }
 
+// Heavy rows are cut into slices for all warps.  A row of class j (4^j to
+// 4^(j+1) - 1 chunks of td_chunk edges) has 4^j slices of equal length, and the
+// slices of all rows are taken in the order of their place in the row, 64 windows
+// of it: rows are sorted by id, so with ids spread evenly the grid works on one
+// 64th of the targets at a time, and the claims' scattered stores (parents,
+// level bytes) and reads (bitmap words, degree bytes) meet in L2.  In the order
+// the rows were found instead, a claim's 4-byte parent store is a read and a write
+// of its own DRAM sector: R-MAT 26, a level of 72 M hub edges and 10.7 M claims,
+// 956 us, 609 us in this order.  Nothing depends on the even spread but speed.
+// The order needs no list of slices: from the classes' row counts alone a
+// slice's number gives window, class, row and place (hub_slice).
+constexpr int kHubWinShift = 3;                       // 4^3 windows
+constexpr int kHubWindows = 1 << (2 * kHubWinShift);
+
+__device__ __forceinline__ int hub_class(long long deg, int chunk) {
+    const unsigned nch = (unsigned)((deg + chunk - 1) / chunk);
+    return (31 - __clz((int)nch)) >> 1;
+}
+
+__device__ __forceinline__ long long hub_slices(const LevelCtr& c) {
+    const int lane = lane_id();
+    return warp_sum(lane < kHubClasses ? (long long)c.hubs[lane] << (2 * lane) : 0LL);
+}
+
+// Slice x of the level's hub rows (x < hub_slices, the same in every lane; all
+// lanes call): its column range and row vertex.  Window k holds, for each class j
+// >= 3, slices k 4^(j-3) .. (k+1) 4^(j-3) - 1 of every row, and for j < 3 slice
+// k / 4^(3-j) when that divides.
+__device__ __forceinline__ void hub_slice(const SingleParams& p, const LevelCtr& c, long long x, long long& start,
+                                          int& len, int& u) {
+    const int lane = lane_id();
+    const long long h = lane < kHubClasses ? (long long)c.hubs[lane] : 0LL;
+    const int big = 2 * (lane - kHubWinShift);   // >= 0: log2 of this class's slices per window
+    // slices before window k (a lane's class alone), summed over the classes
+    const long long per = warp_sum(big >= 0 ? h << big : 0LL);
+    const long long h0 = __shfl_sync(kFull, h, 0), h1 = __shfl_sync(kFull, h, 1), h2 = __shfl_sync(kFull, h, 2);
+    auto before = [&](int k) {
+        return per * k + h0 * ((k + 63) >> 6) + h1 * ((k + 15) >> 4) + h2 * ((k + 3) >> 2);
+    };
+    static_assert(kHubWinShift == 3 && kHubWindows == 64, "the windows of classes 0 to 2");
+    int k = 2 * (__popc(__ballot_sync(kFull, before(2 * lane) <= x)) - 1);
+    if (before(k + 1) <= x) k++;
+    long long r = x - before(k);
+    // class: the first whose slices in this window reach past r
+    const long long mine = big >= 0 ? h << big : (k & ((1 << -big) - 1)) == 0 ? h : 0LL;
+    long long incl = mine;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const long long y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int j = __ffs(__ballot_sync(kFull, incl > r)) - 1;
+    r -= __shfl_sync(kFull, incl - mine, j);
+    const unsigned hj = (unsigned)__shfl_sync(kFull, h, j);
+    long long slice;
+    unsigned row;
+    if (j >= kHubWinShift) {
+        slice = ((long long)k << (2 * (j - kHubWinShift))) + (unsigned)r / hj;
+        row = (unsigned)r % hj;
+    } else {
+        slice = k >> (2 * (kHubWinShift - j));
+        row = (unsigned)r;
+    }
+    const int4 raw = __ldcg(reinterpret_cast<const int4*>(p.hubs + p.hub_off[j] + row));
+    const long long lo = ((long long)raw.z * slice) >> (2 * j), hi = ((long long)raw.z * (slice + 1)) >> (2 * j);
+    start = ((long long)(unsigned)raw.x | ((long long)raw.y << 32)) + lo;
+    len = (int)(hi - lo);
+    u = raw.w;
+}
+
 __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long long nf, int* qnext, int snext,
                          bool nodeg, unsigned long long& acc_m, unsigned long long& acc_h) {
     const int lane = lane_id();
@@ -633,26 +706,22 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
         const long long deg = e - s;
         const bool big = deg > p.big_deg;
         const int mydeg = big ? 0 : (int)deg;
-        // heavy rows become edge-chunk tasks; the warp writes each row's chunk
-        // descriptors together
-        unsigned bm = __ballot_sync(kFull, big);
-        while (bm) {
-            const int L = __ffs(bm) - 1;
-            bm &= bm - 1;
-            const long long bs = __shfl_sync(kFull, s, L), be = __shfl_sync(kFull, e, L);
-            const int bu = __shfl_sync(kFull, u, L);
-            const long long nch = (be - bs + p.td_chunk - 1) / p.td_chunk;
-            unsigned long long t0 = 0;
-            if (lane == 0) t0 = atomicAdd(&p.ctrl->lv[snext].ntask, (unsigned long long)nch);
-            t0 = __shfl_sync(kFull, t0, 0);
-            for (long long c = lane; c < nch; c += 32) {
-                const long long ti = (long long)t0 + c;
-                if (ti < p.task_cap) {
-                    Task t;
-                    t.start = bs + c * p.td_chunk;
-                    t.len = (int)min((long long)p.td_chunk, be - t.start);
-                    t.u = bu;
-                    p.tasks[ti] = t;
+        // heavy rows: into the lists, one atomic per class and warp
+        if (__any_sync(kFull, big)) {
+            const int cls = big ? hub_class(deg, p.td_chunk) : -1;
+            const unsigned same = __match_any_sync(kFull, cls);
+            unsigned long long at = 0;
+            if (big && lane == __ffs(same) - 1)
+                at = atomicAdd(&p.ctrl->lv[snext].hubs[cls], (unsigned long long)__popc(same));
+            at = __shfl_sync(kFull, at, __ffs(same) - 1) + __popc(same & lanemask_lt());
+            if (big) {
+                const long long slot = p.hub_off[cls] + (long long)at;
+                if (slot < p.hub_off[cls + 1]) {
+                    Hub h;
+                    h.start = s;
+                    h.len = (int)deg;
+                    h.u = u;
+                    p.hubs[slot] = h;
                 } else {
                     raise_status(&p.ctrl->b, kDevOverflow);
                 }
@@ -681,20 +750,28 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
     acc_h += st.hv;
 }
 
-__device__ void task_phase(const SingleParams& p, int d, long long ntask, int* qnext, int snext, bool nodeg,
-                           unsigned long long& acc_m, unsigned long long& acc_h) {
+__device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int* qnext, int snext, bool nodeg,
+                          unsigned long long& acc_m, unsigned long long& acc_h) {
     const int lane = lane_id();
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
     st.nodeg = nodeg;
-    const long long nt = ntask < p.task_cap ? ntask : p.task_cap;
+    const long long slices = hub_slices(ctr);
+    // few slices: each in 2^sh parts, down to 32 edges, so that a small level is one
+    // short round per warp (R-MAT 26, 93 K edges: 404 slices 51 us, in 16 parts 25 us)
+    int sh = 0;
+    while (sh < 4 && (slices << (sh + 1)) <= 8 * nw) sh++;
+    const long long nt = slices << sh;
     for (long long t = gw; t < nt; t += nw) {
-        const int4 raw = __ldcg(reinterpret_cast<const int4*>(p.tasks + t));
-        const long long start = (long long)(unsigned)raw.x | ((long long)raw.y << 32);
-        const int len = raw.z, u = raw.w;
+        long long start;
+        int len, u;
+        hub_slice(p, ctr, t >> sh, start, len, u);
+        const int i = (int)(t & ((1 << sh) - 1));
+        int k0 = (int)(((long long)len * i) >> sh);
+        len = (int)(((long long)len * (i + 1)) >> sh);
         // four independent edges per lane per step (coalesced across the warp)
-        for (int k0 = 0; k0 < len; k0 += 128) {
+        for (; k0 < len; k0 += 128) {
             int v[4];
             bool act[4];
 #pragma unroll
@@ -707,13 +784,13 @@ __device__ void task_phase(const SingleParams& p, int d, long long ntask, int* q
             unsigned seen[4];
 #pragma unroll
             for (int q = 0; q < 4; q++) seen[q] = act[q] ? __ldcg(p.visited + (v[q] >> 5)) : kFull;
-            bool claimed[4];
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const unsigned bit = 1u << (v[q] & 31);
                 if (!(seen[q] & bit)) seen[q] = atomicOr(p.visited + (v[q] >> 5), bit);
                 else seen[q] = bit;
             }
+            bool claimed[4];
 #pragma unroll
             for (int q = 0; q < 4; q++) claimed[q] = act[q] && !(seen[q] & (1u << (v[q] & 31)));
 #pragma unroll
@@ -730,7 +807,7 @@ __device__ void task_phase(const SingleParams& p, int d, long long ntask, int* q
 // the top-down local discovery).  Bottom-up levels over the id-ordered rows
 // find exactly that parent (their first hit); a top-down claim takes whichever
 // edge wins.  So right after a top-down level its edges are walked once more,
-// the same way (rows, then chunk tasks), and an edge (u, v) into a vertex the
+// the same way (rows, then hub slices), and an edge (u, v) into a vertex the
 // level discovered offers u by atomicMin: the winner's own u stands as the
 // first offer.  The work is that of the level itself, balanced like it,
 // whatever the degrees of the discovered vertices: finding the parents from the
@@ -742,7 +819,7 @@ __device__ __forceinline__ void min_offer(const SingleParams& p, int d, int u, i
     if (get_level(p, v) == d + 1) atomicMin(p.parent + v, u);
 }
 
-__device__ void td_min_pass(const SingleParams& p, int d, const int* q, long long nf, long long ntask) {
+__device__ void td_min_pass(const SingleParams& p, int d, const int* q, long long nf, const LevelCtr& ctr) {
     const int lane = lane_id();
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
     const long long per = nf >= nw * 32 ? 32 : max(1LL, (nf + nw - 1) / nw);
@@ -754,7 +831,7 @@ __device__ void td_min_pass(const SingleParams& p, int d, const int* q, long lon
             u = __ldcg(q + i);
             long long e;
             row_of(p, u, s, e);
-            deg = e - s > p.big_deg ? 0 : (int)(e - s);   // heavier rows: their chunk tasks
+            deg = e - s > p.big_deg ? 0 : (int)(e - s);   // heavier rows: their slices
         }
         const int incl = warp_inclusive_scan(deg);
         const int total = __shfl_sync(kFull, incl, 31);
@@ -773,11 +850,12 @@ __device__ void td_min_pass(const SingleParams& p, int d, const int* q, long lon
             if (k < total) min_offer(p, d, uj, __ldg(p.cols + sj + (k - exj)));
         }
     }
-    const long long nt = ntask < p.task_cap ? ntask : p.task_cap;
+    const long long nt = hub_slices(ctr);
     for (long long t = gw; t < nt; t += nw) {
-        const int4 raw = __ldcg(reinterpret_cast<const int4*>(p.tasks + t));
-        const long long start = (long long)(unsigned)raw.x | ((long long)raw.y << 32);
-        for (int k = lane; k < raw.z; k += 32) min_offer(p, d, raw.w, __ldg(p.cols + start + k));
+        long long start;
+        int len, u;
+        hub_slice(p, ctr, t, start, len, u);
+        for (int k = lane; k < len; k += 32) min_offer(p, d, u, __ldg(p.cols + start + k));
     }
 }
 
@@ -1935,16 +2013,16 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             }
             if (!level_sync(p, snext, s_ctr)) return;
             if (lead) S.t_mid = globaltimer_ns();
-            if (s_ctr.ntask > 0) {
+            if (hub_slices(s_ctr) > 0) {
                 unsigned long long am = 0, ah = 0;
-                task_phase(p, S.d, (long long)s_ctr.ntask, S.qsel ? p.queue0 : p.queue1, snext, p.directed != 0, am, ah);
+                hub_phase(p, S.d, s_ctr, S.qsel ? p.queue0 : p.queue1, snext, p.directed != 0, am, ah);
                 block_add4(ah, am, 0, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm, nullptr, nullptr);
                 if (!level_sync(p, snext, s_ctr)) return;
             }
             if constexpr (kMinId) {
                 if (s_ctr.tail > 0) {
-                    td_min_pass(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, (long long)s_ctr.ntask);
-                    // the next level writes this queue and the task list
+                    td_min_pass(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, s_ctr);
+                    // the next level writes this queue and the hub lists
                     if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
                 }
             }
@@ -2000,6 +2078,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             block_add4(so, si, 0, 0, &c->lv[snext].dsum_out, &c->lv[snext].dsum_in, nullptr, nullptr);
             if (!level_sync(p, snext, s_ctr)) return;
         }
+        const long long slices = dir == TD ? hub_slices(s_ctr) : 0;
         const long long nf_next = (long long)(dir == TD ? s_ctr.tail : s_ctr.accn);
         if (threadIdx.x == 0) {
             const long long macc = (long long)s_ctr.accm;
@@ -2015,7 +2094,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 r.scanned = dir == BU ? (long long)s_ctr.scanned : 0;
                 r.examined = dir == BU ? (long long)s_ctr.examined : S.mf;
                 r.t_ns = (long long)(globaltimer_ns() - S.t_start);
-                r.aux = (long long)s_ctr.ntask;
+                r.aux = dir == TD ? slices : (long long)s_ctr.ntask;
                 r.t_mid_ns = S.t_mid ? (long long)(S.t_mid - S.t_start) : 0;
                 p.rec[S.d] = r;
             }
@@ -2346,7 +2425,7 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
 constexpr long long kStaticMaxN = 1LL << 20;
 constexpr long long kStaticMaxNnz = 1LL << 24;
 constexpr long long kStaticW = kStaticMaxN / 32;
-constexpr long long kStaticTasks = kStaticMaxNnz / kChunk + kStaticMaxNnz / 64 + 1024;   // default chunk
+constexpr long long kStaticTasks = kStaticMaxNnz / kChunk + kStaticMaxNnz / 64 + 1024;   // hub_regions at degree 96, chunk kChunk
 constexpr int kStaticRec = 64;
 constexpr size_t kStaticCtrlOff = 0;
 constexpr size_t kStaticIsoOff = (sizeof(Ctrl) + 255) / 256 * 256;   // control block slot
@@ -2356,7 +2435,7 @@ constexpr size_t kStaticF1Off = kStaticF0Off + 4 * kStaticW;
 constexpr size_t kStaticQ0Off = kStaticF1Off + 4 * kStaticW;
 constexpr size_t kStaticQ1Off = kStaticQ0Off + 4 * (kStaticMaxN + 64);
 constexpr size_t kStaticTaskOff = kStaticQ1Off + 4 * (kStaticMaxN + 64);
-constexpr size_t kStaticRecOff = kStaticTaskOff + sizeof(Task) * kStaticTasks;
+constexpr size_t kStaticRecOff = kStaticTaskOff + sizeof(Hub) * kStaticTasks;
 constexpr size_t kStaticBytes = kStaticRecOff + sizeof(bfs_level_record) * kStaticRec;
 static_assert(kStaticQ1Off % 16 == 0 && kStaticTaskOff % 16 == 0 && kStaticRecOff % 8 == 0, "alignment");
 
@@ -2383,7 +2462,7 @@ namespace bfsrt {
 
 using bfsk::Ctrl;
 using bfsk::SingleParams;
-using bfsk::Task;
+using bfsk::Hub;
 
 // the CSR kernel's variants: any parent over the id-ordered rows, over the hub-first
 // rows, and minimum-id parents (id-ordered rows only); each without and with
@@ -2419,6 +2498,20 @@ static cudaError_t csr_occupancy(int* per_sm) {
     return cudaSuccess;
 }
 
+// Hub lists: rows of degree > big_deg (>= kMinChunk), those of class j >= 1 of degree
+// > (4^j - 1) * td_chunk (>= kMinChunk).  The classes' most rows add up to less than
+// nnz / 64 + nnz / 144 for any such setting.
+static long long hub_capacity(long long nnz) { return nnz / bfsk::kMinChunk + nnz / 64 + 1024; }
+static void hub_regions(SingleParams& p) {
+    long long at = 0;
+    for (int j = 0; j < bfsk::kHubClasses; j++) {
+        p.hub_off[j] = at;
+        const long long least = std::max<long long>(p.big_deg, ((1LL << (2 * j)) - 1) * p.td_chunk) + 1;
+        at += p.nnz / least + 1;
+    }
+    p.hub_off[bfsk::kHubClasses] = at;
+}
+
 bfs_status single_prepare(bfs_graph* g, cudaStream_t s) { return single_prepare_work(g, g->single, s, 0); }
 
 // Work buffers of one single-source search state on graph g; grid > 0 caps the
@@ -2426,8 +2519,7 @@ bfs_status single_prepare(bfs_graph* g, cudaStream_t s) { return single_prepare_
 bfs_status single_prepare_work(bfs_graph* g, SingleWork& w, cudaStream_t s, int grid) {
     if (w.ready) return BFS_OK;
     const long long n = g->n, W = g->W;
-    // chunks of >= kMinChunk edges of vertices of degree > 64: at most nnz/64 + nnz/64 tasks
-    const long long task_cap = g->nnz / bfsk::kMinChunk + g->nnz / 64 + 1024;
+    const long long task_cap = hub_capacity(g->nnz);
     const int rec_cap = 1 << 16;
     struct Item { void** p; size_t bytes; };
     Item items[] = {
@@ -2438,7 +2530,7 @@ bfs_status single_prepare_work(bfs_graph* g, SingleWork& w, cudaStream_t s, int 
         {(void**)&w.queue1, sizeof(int) * (size_t)(n + 32)},
         {(void**)&w.lv8, (size_t)W * 32},   // one byte per vertex, rounded up to whole bitmap words
         {(void**)&w.pfirst, sizeof(unsigned) * (size_t)W},
-        {(void**)&w.tasks, sizeof(Task) * (size_t)task_cap},
+        {(void**)&w.tasks, sizeof(Hub) * (size_t)task_cap},
         {(void**)&w.ctrl, sizeof(Ctrl)},
         {(void**)&w.records, sizeof(bfs_level_record) * (size_t)rec_cap},
     };
@@ -2479,7 +2571,7 @@ void single_release_work(bfs_graph* g, SingleWork& w) {
     mem_of(g, w).release(w.lv8, (size_t)W * 32, nullptr);
     mem_of(g, w).release(w.pfirst, sizeof(unsigned) * (size_t)W, nullptr);
     if (w.level_scratch) mem_of(g, w).release(w.level_scratch, sizeof(int) * (size_t)n, nullptr);
-    mem_of(g, w).release(w.tasks, sizeof(Task) * (size_t)w.task_cap, nullptr);
+    mem_of(g, w).release(w.tasks, sizeof(Hub) * (size_t)w.task_cap, nullptr);
     mem_of(g, w).release(w.ctrl, sizeof(Ctrl), nullptr);
     mem_of(g, w).release(w.records, sizeof(bfs_level_record) * (size_t)w.rec_cap, nullptr);
     DeviceAlloc* keep = w.mem;   // the allocator choice outlives the buffers
@@ -2527,8 +2619,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     p.front1 = w.front1;
     p.queue0 = w.queue0;
     p.queue1 = w.queue1;
-    p.tasks = reinterpret_cast<Task*>(w.tasks);
-    p.task_cap = w.task_cap;
+    p.hubs = reinterpret_cast<Hub*>(w.tasks);
     p.ctrl = reinterpret_cast<Ctrl*>(w.ctrl);
     p.rec = w.records;
     p.rec_cap = w.rec_cap;
@@ -2540,6 +2631,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     p.parent_mode = opt.parent_mode;
     p.big_deg = opt.td_big_degree > 0 ? opt.td_big_degree : 96;
     p.td_chunk = opt.td_chunk > 0 ? opt.td_chunk : bfsk::kDefaultChunk;
+    hub_regions(p);
     p.clu_c = 1;
     p.clu_big = 0;
     p.clu_nf = 0;
@@ -2662,7 +2754,7 @@ bfs_status single_collect(bfs_graph* g, cudaStream_t s, bfs_stats* stats) {
     if (c.b.status == bfsk::kDevTimeout)
         return fail(BFS_ERR_TIMEOUT, "device grid barrier wait ran out of time; outputs are undefined");
     if (c.b.status == bfsk::kDevOverflow)
-        return fail(BFS_ERR_CUDA, "top-down chunk task list overflowed (internal sizing error)");
+        return fail(BFS_ERR_CUDA, "top-down hub list overflowed (internal sizing error)");
     if (stats) {
         stats->num_levels = (int32_t)c.num_levels;
         stats->t_init_ns = c.t_init > c.t_enter ? (int64_t)(c.t_init - c.t_enter) : 0;
@@ -2758,8 +2850,7 @@ extern "C" bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int3
     p.front1 = reinterpret_cast<unsigned*>(b + bfsk::kStaticF1Off);
     p.queue0 = reinterpret_cast<int*>(b + bfsk::kStaticQ0Off);
     p.queue1 = reinterpret_cast<int*>(b + bfsk::kStaticQ1Off);
-    p.tasks = reinterpret_cast<bfsk::Task*>(b + bfsk::kStaticTaskOff);
-    p.task_cap = bfsk::kStaticTasks;
+    p.hubs = reinterpret_cast<bfsk::Hub*>(b + bfsk::kStaticTaskOff);
     p.ctrl = reinterpret_cast<bfsk::Ctrl*>(b + bfsk::kStaticCtrlOff);
     p.rec = reinterpret_cast<bfs_level_record*>(b + bfsk::kStaticRecOff);
     p.rec_cap = bfsk::kStaticRec;
@@ -2771,6 +2862,7 @@ extern "C" bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int3
     p.parent_mode = BFS_PARENT_ANY;
     p.big_deg = 96;
     p.td_chunk = bfsk::kChunk;
+    hub_regions(p);
     p.clu_c = 1;
     p.clu_big = 0;
     p.clu_nf = 0;

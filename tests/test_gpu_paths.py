@@ -110,3 +110,92 @@ def test_bottom_up_chunk_widths(gpu_lib, n, hub):
             for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext", "scanned", "examined"]):
                 assert np.array_equal(info["records"][:, col], getattr(s, name)), (root, mode, name)
     g.close()
+
+
+@pytest.mark.parametrize("shape", ["er", "hubs"])
+def test_large_graph_outputs(gpu_lib, shape):
+    """Graphs whose parent array exceeds what stays in L2 (top-down levels then take their
+    targets by windows), with a ragged last block: claims from short rows and from hubs,
+    first windows, row heads and long rows; both row orders, every direction, several
+    roots, with and without levels."""
+    import torch
+    bfs = gpu_lib
+    n = (1 << 23) + 77
+    if shape == "er":
+        e = graphgen.erdos_renyi(n, 3 * n, seed=4)
+    else:
+        # 40 hubs over overlapping slices of the ids, and a sparse random rest
+        rng = np.random.default_rng(5)
+        ids = rng.permutation(n).astype(np.int32)
+        cut = [ids[i * 150_000:i * 150_000 + 400_000] for i in range(40)]
+        r = graphgen.erdos_renyi(n, n, seed=6)
+        e = graphgen.EdgeList(n, np.concatenate([np.full(400_000, ids[i], np.int32) for i in range(40)] + [r.src]),
+                              np.concatenate(cut + [r.dst]))
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, hub_first=True)
+    level, parent = _buffers(n)
+    root = int(graphgen.pick_roots(e, 1, 3)[0])
+    want = oracle.levels(ref, root)
+    for mode in (bfs.MODE_DO, bfs.MODE_TD_ONLY, bfs.MODE_BU_ONLY):
+        for rows in (bfs.BU_ROWS_BY_ID, bfs.BU_ROWS_HUB_FIRST):
+            o = bfs.options(mode=mode, bu_rows=rows)
+            parent.fill_(-7)
+            g.run(root, parent=parent, level=level, opts=o)
+            assert np.array_equal(level.cpu().numpy(), want), (mode, rows)
+            assert oracle.certify(ref, root, want, parent.cpu().numpy(), labels) == (0, -1), (mode, rows)
+            parent.fill_(-7)
+            g.run(root, parent=parent, opts=o)
+            assert oracle.certify(ref, root, want, parent.cpu().numpy(), labels) == (0, -1), (mode, rows, "no levels")
+    # an output that starts off a 16-byte boundary
+    off = torch.full((n + 1,), -7, dtype=torch.int32, device="cuda")
+    g.run(root, parent=off[1:], level=level)
+    assert oracle.certify(ref, root, want, off[1:].cpu().numpy(), labels) == (0, -1)
+    # several roots: every root its own parent, every other vertex one level below its parent
+    roots = np.unique(graphgen.pick_roots(e, 9, 4))
+    g.run_multiroot(roots, parent=parent, level=level)
+    lv, pa = level.cpu().numpy(), parent.cpu().numpy()
+    assert (lv[roots] == 0).all() and (pa[roots] == roots).all()
+    v = np.flatnonzero(lv > 0)
+    assert np.array_equal(lv[pa[v]], lv[v] - 1) and np.array_equal(pa < 0, lv < 0)
+    for x in v[:: max(1, v.size // 2000)]:
+        assert pa[x] in ref.cols[ref.offsets[x]:ref.offsets[x + 1]]
+    g.close()
+
+
+@pytest.mark.parametrize("big,chunk", [(0, 0), (64, 64), (64, 4096), (300, 200)])
+def test_hub_slices_at_class_edges(gpu_lib, big, chunk):
+    """Top-down rows shared by all warps: degrees just below and at every class of slice
+    counts (1, 4, 16, 64, 256 chunks), alone and many of a class, over overlapping
+    targets."""
+    bfs = gpu_lib
+    n = 60_000
+    c = chunk or 128
+    degs = sorted({int(max(1, min(n // 2, d))) for k in (1, 4, 16, 64, 256) for d in
+                   (c * (k - 1), c * (k - 1) + 1, c * k, c * k + 1)} | {big or 96, (big or 96) + 1} | {70 + i for i in range(40)})
+    rng = np.random.default_rng(big + chunk)
+    hubs = np.arange(1, 1 + len(degs), dtype=np.int32)
+    src, dst = [np.zeros(len(degs), np.int32)], [hubs]
+    for h, d in zip(hubs, degs):
+        t = rng.choice(np.arange(1 + len(degs), n, dtype=np.int32), d, replace=False)
+        src.append(np.full(d, h, np.int32))
+        dst.append(t)
+    perm = rng.permutation(n).astype(np.int32)
+    e = graphgen.EdgeList(n, perm[np.concatenate(src)], perm[np.concatenate(dst)])
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+    level, parent = _buffers(n)
+    root = int(perm[0])
+    want = oracle.levels(ref, root)
+    s = oracle.do_schedule(ref, want, oracle.MODE_TD)
+    for pm in (bfs.PARENT_ANY, bfs.PARENT_MIN_ID):
+        info = g.run(root, parent=parent, level=level, stats=True, record_levels=64,
+                     opts=bfs.options(mode=bfs.MODE_TD_ONLY, parent_mode=pm, td_big_degree=big, td_chunk=chunk))
+        pa = parent.cpu().numpy()
+        assert np.array_equal(level.cpu().numpy(), want)
+        assert oracle.certify(ref, root, want, pa, labels) == (0, -1)
+        assert pm == bfs.PARENT_ANY or np.array_equal(pa, oracle.min_parent(ref, want))
+        for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext"]):
+            assert np.array_equal(info["records"][:, col], getattr(s, name)), name
+    g.close()
