@@ -263,6 +263,19 @@ __device__ __forceinline__ long long deg_from8(const SingleParams& p, int u, uns
     return d8 < 255u ? (long long)d8 : deg_of(p, u);
 }
 
+// out- and in-degree of a directed graph's vertex
+__device__ __forceinline__ long long out_degree(const SingleParams& p, int v) {
+    return deg_from8(p, v, __ldg(p.deg8 + v));
+}
+
+__device__ __forceinline__ long long in_degree(const SingleParams& p, int v) {
+    const unsigned d8 = __ldg(p.deg8_in + v);
+    if (d8 < 255u) return (long long)d8;
+    long long s, e;
+    bu_row_of(p, v, s, e);
+    return e - s;
+}
+
 constexpr unsigned char kLvUnseen = 255;   // not reached (yet)
 constexpr unsigned char kLvDeep = 254;     // depth >= 254: the int32 level holds it
 
@@ -464,7 +477,7 @@ struct WarpStage {
     int* buf;   // kStage entries of this warp's shared-memory slice
     int cnt;    // warp-uniform fill level
     bool pf;    // prefetch the rows of flushed vertices into L2 (small levels)
-    bool nodeg;    // no degrees at the flush (a directed graph sums them after the level)
+    unsigned long long din;   // kDir: this lane's sum of the flushed vertices' in-degrees
     unsigned hv;   // this lane's flushed vertices of degree above the cluster-level cap
 };
 
@@ -491,18 +504,18 @@ __device__ __forceinline__ void flush_degree(const SingleParams& p, int v, bool 
 // in flight together (one by one they would be a chain of dependent DRAM reads).
 constexpr int kFlushBatch = 8;
 
+// kDir (a directed graph): acc_m collects out-degrees (the next frontier's m_f),
+// st.din in-degrees (what m_u loses).
+template <bool kDir>
 __device__ __forceinline__ void flush_entries(const SingleParams& p, WarpStage& st, int* qnext,
                                               unsigned long long base, unsigned long long& acc_m) {
     const int lane = lane_id();
-    if (st.nodeg) {
-        for (int i = lane; i < st.cnt; i += 32) qnext[base + i] = st.buf[i];
-        return;
-    }
     if (!p.deg8 || st.pf) {
         for (int i = lane; i < st.cnt; i += 32) {
             const int v = st.buf[i];
             qnext[base + i] = v;
             flush_degree(p, v, st.pf, acc_m, st.hv);
+            if constexpr (kDir) st.din += (unsigned long long)in_degree(p, v);
         }
         return;
     }
@@ -522,10 +535,12 @@ __device__ __forceinline__ void flush_entries(const SingleParams& p, WarpStage& 
             const long long dg = d8[k] < 255u ? (long long)d8[k] : deg_of(p, vs[k]);
             acc_m += (unsigned long long)dg;
             st.hv += dg > (long long)p.clu_big;
+            if constexpr (kDir) st.din += (unsigned long long)in_degree(p, vs[k]);
         }
     }
 }
 
+template <bool kDir>
 __device__ __forceinline__ void stage_flush(const SingleParams& p, WarpStage& st, int* qnext,
                                             unsigned long long* tail, unsigned long long& acc_m) {
     if (st.cnt == 0) return;
@@ -533,7 +548,7 @@ __device__ __forceinline__ void stage_flush(const SingleParams& p, WarpStage& st
     unsigned long long base = 0;
     if (lane_id() == 0) base = atomicAdd(tail, (unsigned long long)st.cnt);
     base = __shfl_sync(kFull, base, 0);
-    flush_entries(p, st, qnext, base, acc_m);
+    flush_entries<kDir>(p, st, qnext, base, acc_m);
     __syncwarp();
     st.cnt = 0;
 }
@@ -542,6 +557,7 @@ __device__ __forceinline__ void stage_flush(const SingleParams& p, WarpStage& st
 // with one atomicAdd per CTA (a block scan of the warps' counts).  On small
 // levels most warps hold a few entries each, and one queue-tail atomic per
 // warp would serialise thousands of arrivals on one word.  All threads call.
+template <bool kDir>
 __device__ void block_flush(const SingleParams& p, WarpStage& st, int* qnext, unsigned long long* tail,
                             unsigned long long& acc_m) {
     __shared__ int s_wcnt[kWarps];
@@ -560,12 +576,13 @@ __device__ void block_flush(const SingleParams& p, WarpStage& st, int* qnext, un
     }
     __syncthreads();
     const unsigned long long base = s_bbase + (unsigned long long)s_wcnt[wib];
-    flush_entries(p, st, qnext, base, acc_m);
+    flush_entries<kDir>(p, st, qnext, base, acc_m);
     __syncwarp();
     st.cnt = 0;
 }
 
 // Record the claims of one warp step: winners write parent/level and stage v.
+template <bool kDir>
 __device__ __forceinline__ void td_stage(const SingleParams& p, int d, int u, int v, bool claimed, WarpStage& st,
                                          int* qnext, unsigned long long* tail, unsigned long long& acc_m) {
     const unsigned cm = __ballot_sync(kFull, claimed);
@@ -576,13 +593,14 @@ __device__ __forceinline__ void td_stage(const SingleParams& p, int d, int u, in
             set_level(p, v, d + 1);
         }
         st.cnt += __popc(cm);
-        if (st.cnt > kStage - 32) stage_flush(p, st, qnext, tail, acc_m);
+        if (st.cnt > kStage - 32) stage_flush<kDir>(p, st, qnext, tail, acc_m);
     }
 }
 
 // Visit edge (u, v) for the whole warp (every lane calls; `act` masks): claim
 // v with an atomicOr on the visited bitmap; the winner records parent/level
 // and stages v for the next queue.
+template <bool kDir>
 __device__ __forceinline__ void td_visit(const SingleParams& p, int d, int u, int v, bool act, WarpStage& st,
                                          int* qnext, unsigned long long* tail, unsigned long long& acc_m) {
     bool claimed = false;
@@ -598,7 +616,7 @@ __device__ __forceinline__ void td_visit(const SingleParams& p, int d, int u, in
         claimed = !(atomicOr(wp, bit) & bit);
 #endif
     }
-    td_stage(p, d, u, v, claimed, st, qnext, tail, acc_m);
+    td_stage<kDir>(p, d, u, v, claimed, st, qnext, tail, acc_m);
 }
 
 __device__ __forceinline__ WarpStage warp_stage_in(int* buf) {
@@ -606,7 +624,7 @@ __device__ __forceinline__ WarpStage warp_stage_in(int* buf) {
     st.buf = buf;
     st.cnt = 0;
     st.pf = false;
-    st.nodeg = false;
+    st.din = 0;
     st.hv = 0;
     return st;
 }
@@ -684,14 +702,14 @@ __device__ __forceinline__ void hub_slice(const SingleParams& p, const LevelCtr&
     u = raw.w;
 }
 
+template <bool kDir>
 __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long long nf, int* qnext, int snext,
-                         bool nodeg, unsigned long long& acc_m, unsigned long long& acc_h) {
+                         unsigned long long& acc_m, unsigned long long& acc_h, unsigned long long& acc_in) {
     const int lane = lane_id();
     const long long gw = spread_warp(), nw = gthreads() >> 5;
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
-    st.nodeg = nodeg;
-    st.pf = !nodeg && nf < kPrefetchNf;
+    st.pf = nf < kPrefetchNf;
     // A small frontier is spread over every warp (fewer vertices per warp, so
     // each warp's edges take one gather round instead of several dependent ones).
     const long long per = nf >= nw * 32 ? 32 : max(1LL, (nf + nw - 1) / nw);
@@ -743,20 +761,21 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
             const int uj = __shfl_sync(kFull, u, j);
             const bool act = k < total;
             const int v = act ? __ldg(p.cols + sj + (k - exj)) : 0;
-            td_visit(p, d, uj, v, act, st, qnext, tail, acc_m);
+            td_visit<kDir>(p, d, uj, v, act, st, qnext, tail, acc_m);
         }
     }
-    block_flush(p, st, qnext, tail, acc_m);
+    block_flush<kDir>(p, st, qnext, tail, acc_m);
     acc_h += st.hv;
+    acc_in += st.din;
 }
 
-__device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int* qnext, int snext, bool nodeg,
-                          unsigned long long& acc_m, unsigned long long& acc_h) {
+template <bool kDir>
+__device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int* qnext, int snext,
+                          unsigned long long& acc_m, unsigned long long& acc_h, unsigned long long& acc_in) {
     const int lane = lane_id();
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
-    st.nodeg = nodeg;
     const long long slices = hub_slices(ctr);
     // few slices: each in 2^sh parts, down to 32 edges, so that a small level is one
     // short round per warp (R-MAT 26, 93 K edges: 404 slices 51 us, in 16 parts 25 us)
@@ -794,11 +813,12 @@ __device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int
 #pragma unroll
             for (int q = 0; q < 4; q++) claimed[q] = act[q] && !(seen[q] & (1u << (v[q] & 31)));
 #pragma unroll
-            for (int q = 0; q < 4; q++) td_stage(p, d, u, v[q], claimed[q], st, qnext, tail, acc_m);
+            for (int q = 0; q < 4; q++) td_stage<kDir>(p, d, u, v[q], claimed[q], st, qnext, tail, acc_m);
         }
     }
-    block_flush(p, st, qnext, tail, acc_m);
+    block_flush<kDir>(p, st, qnext, tail, acc_m);
     acc_h += st.hv;
+    acc_in += st.din;
 }
 
 // parent_mode MIN_ID: every reached v other than a root takes the smallest
@@ -902,45 +922,6 @@ __device__ void min_parent_rows(const SingleParams& p, const unsigned* lv) {
                     if (lane == 0) p.parent[base + L] = pu;
                     break;
                 }
-            }
-        }
-    }
-}
-
-// A directed graph's new frontier, after its level: the sum of its out-degrees
-// (m_f of the direction rule) and of its in-degrees (what m_u, the in-degree
-// sum of the unreached vertices, loses).  The frontier is the queue q[0..nq)
-// after a top-down level (q non-null), else the bitmap f.
-__device__ __forceinline__ long long out_degree(const SingleParams& p, int v) {
-    const unsigned d8 = __ldg(p.deg8 + v);
-    return d8 < 255u ? (long long)d8 : deg_of(p, v);
-}
-
-__device__ __forceinline__ long long in_degree(const SingleParams& p, int v) {
-    const unsigned d8 = __ldg(p.deg8_in + v);
-    if (d8 < 255u) return (long long)d8;
-    long long s, e;
-    bu_row_of(p, v, s, e);
-    return e - s;
-}
-
-__device__ void frontier_degree_sums(const SingleParams& p, const int* q, long long nq, const unsigned* f,
-                                     unsigned long long& sum_out, unsigned long long& sum_in) {
-    const long long tid = gtid(), nth = gthreads();
-    if (q) {
-        for (long long i = tid; i < nq; i += nth) {
-            const int v = __ldcg(q + i);
-            sum_out += (unsigned long long)out_degree(p, v);
-            sum_in += (unsigned long long)in_degree(p, v);
-        }
-    } else {
-        for (long long w = tid; w < p.W; w += nth) {
-            unsigned x = __ldcg(f + w);
-            while (x) {
-                const int v = (int)(w * 32 + __ffs(x) - 1);
-                x &= x - 1;
-                sum_out += (unsigned long long)out_degree(p, v);
-                sum_in += (unsigned long long)in_degree(p, v);
             }
         }
     }
@@ -1075,9 +1056,10 @@ __device__ __forceinline__ int bu_chunk_words(long long W, long long nwarps) {
 // whose row continues past the window without a hit goes on the long list
 // (phase B).  Found vertices are collected per word in shared memory and
 // written as whole next-frontier / completed words (the warp owns its words).
+template <bool kDir>
 __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, unsigned* fnext, int* longlist,
                            unsigned long long* longcnt, unsigned long long& acc_n, unsigned long long& acc_m,
-                           unsigned long long& acc_sc, unsigned long long& acc_ex) {
+                           unsigned long long& acc_sc, unsigned long long& acc_ex, unsigned long long& acc_out) {
     __shared__ unsigned s_next[kBlock / 32][32];
     const int lane = lane_id(), wib = threadIdx.x >> 5;
     unsigned short* list = g_list[wib];
@@ -1109,6 +1091,8 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
         if (u0 >= 0) {
             bu_row_of_stream(p, u0, s0, e0);
         }
+        unsigned o0 = 0, o1 = 0;   // kDir: out-degree bytes, read with the windows
+        if (kDir && u0 >= 0) o0 = __ldg(p.deg8 + u0);
         int4 xa0 = z4, xb0 = z4;
         if (u0 >= 0 && e0 > s0) {
             const int4* src = reinterpret_cast<const int4*>(p.cols_bu + (s0 & ~3LL));
@@ -1128,6 +1112,7 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
                 bu_row_of_stream(p, u2, s2, e2);
             }
             // round r+1: window
+            if (kDir && u1 >= 0) o1 = __ldg(p.deg8 + u1);
             int4 xa1 = z4, xb1 = z4;
             if (u1 >= 0 && e1 > s1) {
                 const int4* src = reinterpret_cast<const int4*>(p.cols_bu + (s1 & ~3LL));
@@ -1156,6 +1141,7 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
                     const int t = __ffs(hb) - 1;
                     acc_ex += (unsigned long long)(rb + t - s0 + 1);
                     acc_m += (unsigned long long)(e0 - s0);
+                    if constexpr (kDir) acc_out += (unsigned long long)deg_from8(p, u0, o0);
                     if (p.parent) p.parent[u0] = pick(ids, t);
                     set_level(p, u0, d + 1);
                     atomicOr(&s_next[wib][(u0 >> 5) - wbase], 1u << (u0 & 31));
@@ -1174,6 +1160,7 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
             u0 = u1;
             s0 = s1;
             e0 = e1;
+            o0 = o1;
             xa0 = xa1;
             xb0 = xb1;
             u1 = u2;
@@ -1463,9 +1450,10 @@ __device__ void bu_misses(const SingleParams& p, int d, const unsigned* fcur, un
 // atomicOr.
 // With count_left, acc_m receives the degrees of the searchers left unvisited
 // (the hub-first sweep's accounting); otherwise those of the ones found.
+template <bool kDir>
 __device__ void bu_phase_b(const SingleParams& p, int d, const unsigned* fcur, unsigned* fnext, const int* longlist,
                            long long nlong, int skip, bool count_left, unsigned long long& acc_n,
-                           unsigned long long& acc_m, unsigned long long& acc_ex) {
+                           unsigned long long& acc_m, unsigned long long& acc_ex, unsigned long long& acc_out) {
     const int lane = lane_id(), grp = lane >> 2, gl = lane & 3;
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
     for (long long base = gw * 8; base < nlong; base += nw * 8) {
@@ -1515,6 +1503,7 @@ __device__ void bu_phase_b(const SingleParams& p, int d, const unsigned* fcur, u
             if (hitpos >= 0) {
                 acc_ex += (unsigned long long)(hitpos - s0 + 1);
                 if (!count_left) acc_m += (unsigned long long)(e0 - s0);
+                if constexpr (kDir) acc_out += (unsigned long long)out_degree(p, u);
                 acc_n += 1;
                 if (p.parent) p.parent[u] = pv;
                 set_level(p, u, d + 1);
@@ -1915,10 +1904,12 @@ struct LoopState {
 // kMinId: the launch also makes the parents the minimum-id ones (parent_mode
 // MIN_ID with both arrays there).  kHub: bottom-up steps scan the hub-first rows
 // (p.first is there).  kClu: the launch is in clusters and runs cluster levels.
+// kDir: a directed graph (accm: out-degrees found top-down, in-degrees bottom-up;
+// the other sum in dsum_in, dsum_out).
 // Variants, so that the passes of one take no registers from another (all in
 // one kernel: 24 to 290 bytes of spills per thread; apart: none to 36 without
 // cluster levels).
-template <bool kMinId, bool kHub, bool kClu>
+template <bool kMinId, bool kHub, bool kClu, bool kDir>
 __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(SingleParams p) {
     Ctrl* c = p.ctrl;
     __shared__ unsigned s_clu_lv[kMinId && kClu ? 8 : 1];   // level bytes that cluster levels discovered
@@ -1945,7 +1936,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
         S.reached = p.nroots;
         S.mf = (long long)s_ctr.accm;
         long long rin = (long long)s_ctr.accm;
-        if (p.directed) {
+        if constexpr (kDir) {
             // m_u sums in-degrees: the edges a bottom-up step could still examine
             if (p.nroots == 1) {
                 long long s0, e0;
@@ -2012,18 +2003,19 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             {
-                unsigned long long am = 0, ah = 0;
-                // a directed graph sums the new frontier's degrees after the level
-                td_phase(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, S.qsel ? p.queue0 : p.queue1, snext,
-                         p.directed != 0, am, ah);
-                block_add4(ah, am, 0, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm, nullptr, nullptr);
+                unsigned long long am = 0, ah = 0, ai = 0;
+                td_phase<kDir>(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, S.qsel ? p.queue0 : p.queue1, snext, am, ah,
+                               ai);
+                block_add4(ah, am, ai, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm,
+                           &c->lv[snext].dsum_in, nullptr);
             }
             if (!level_sync(p, snext, s_ctr)) return;
             if (lead) S.t_mid = globaltimer_ns();
             if (hub_slices(s_ctr) > 0) {
-                unsigned long long am = 0, ah = 0;
-                hub_phase(p, S.d, s_ctr, S.qsel ? p.queue0 : p.queue1, snext, p.directed != 0, am, ah);
-                block_add4(ah, am, 0, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm, nullptr, nullptr);
+                unsigned long long am = 0, ah = 0, ai = 0;
+                hub_phase<kDir>(p, S.d, s_ctr, S.qsel ? p.queue0 : p.queue1, snext, am, ah, ai);
+                block_add4(ah, am, ai, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm,
+                           &c->lv[snext].dsum_in, nullptr);
                 if (!level_sync(p, snext, s_ctr)) return;
             }
             if constexpr (kMinId) {
@@ -2044,16 +2036,17 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             // bottom-up levels (a preceding queue -> bitmap conversion ended at the
             // barrier above): one holds the long list, the other the miss list
             {
-                unsigned long long an = 0, am = 0, asc = 0, aex = 0;
+                unsigned long long an = 0, am = 0, asc = 0, aex = 0, ao = 0;
                 if constexpr (kHub)
                     bu_compact(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
                                S.qsel ? p.queue1 : p.queue0, &c->lv[snext].nmiss, &c->lv[snext].nmiss_in,
                                S.qsel ? p.queue0 : p.queue1, &c->lv[snext].ntask, an, am, asc, aex);
                 else
-                    bu_phase_a(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
-                               S.qsel ? p.queue0 : p.queue1, &c->lv[snext].ntask, an, am, asc, aex);
+                    bu_phase_a<kDir>(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                               S.qsel ? p.queue0 : p.queue1, &c->lv[snext].ntask, an, am, asc, aex, ao);
                 block_add4(an, am, asc, aex, &c->lv[snext].accn, &c->lv[snext].accm, &c->lv[snext].scanned,
                            &c->lv[snext].examined);
+                if constexpr (kDir) block_add4(ao, 0, 0, 0, &c->lv[snext].dsum_out, nullptr, nullptr, nullptr);
             }
             if (!level_sync(p, snext, s_ctr)) return;
             if (lead) S.t_mid = globaltimer_ns();
@@ -2068,28 +2061,19 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 }
             }
             if (s_ctr.ntask > 0) {
-                unsigned long long bn = 0, bm = 0, bex = 0;
-                bu_phase_b(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
-                           S.qsel ? p.queue0 : p.queue1, (long long)s_ctr.ntask, kHub ? kHead : kWin, kHub, bn, bm, bex);
-                block_add4(bn, bm, 0, bex, &c->lv[snext].accn, &c->lv[snext].accm, nullptr, &c->lv[snext].examined);
+                unsigned long long bn = 0, bm = 0, bex = 0, bo = 0;
+                bu_phase_b<kDir>(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                           S.qsel ? p.queue0 : p.queue1, (long long)s_ctr.ntask, kHub ? kHead : kWin, kHub, bn, bm, bex, bo);
+                block_add4(bn, bm, bo, bex, &c->lv[snext].accn, &c->lv[snext].accm, &c->lv[snext].dsum_out,
+                           &c->lv[snext].examined);
                 if (!level_sync(p, snext, s_ctr)) return;
             }
-        }
-        // the new frontier: a queue (the one written) after a top-down level, else a bitmap
-        if (p.directed) {
-            unsigned long long so = 0, si = 0;
-            if (dir == TD)
-                frontier_degree_sums(p, S.qsel ? p.queue0 : p.queue1, (long long)s_ctr.tail, nullptr, so, si);
-            else
-                frontier_degree_sums(p, nullptr, 0, S.bsel ? p.front0 : p.front1, so, si);
-            block_add4(so, si, 0, 0, &c->lv[snext].dsum_out, &c->lv[snext].dsum_in, nullptr, nullptr);
-            if (!level_sync(p, snext, s_ctr)) return;
         }
         const long long slices = dir == TD ? hub_slices(s_ctr) : 0;
         const long long nf_next = (long long)(dir == TD ? s_ctr.tail : s_ctr.accn);
         if (threadIdx.x == 0) {
             const long long macc = (long long)s_ctr.accm;
-            const long long mf_next = p.directed ? (long long)s_ctr.dsum_out : (kHub && dir == BU) ? S.mu - macc : macc;
+            const long long mf_next = dir == TD ? macc : kDir ? (long long)s_ctr.dsum_out : kHub ? S.mu - macc : macc;
             if (lead && S.d < p.rec_cap) {
                 bfs_level_record r;
                 r.dir = dir;
@@ -2108,7 +2092,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             if (nf_next > 0) {
                 S.reached = S.reached + nf_next;
                 // what the unreached lose: in-degrees (undirected: both sums coincide)
-                S.mu = S.mu - (p.directed ? (long long)s_ctr.dsum_in : mf_next);
+                S.mu = S.mu - (!kDir ? mf_next : dir == TD ? (long long)s_ctr.dsum_in : macc);
                 S.nf = nf_next;
                 S.mf = mf_next;
                 if (dir == TD) S.qsel = S.qsel ^ 1;
@@ -2226,11 +2210,11 @@ __device__ void td_dcsc_phase(const SingleParams& p, int d, const int* qcur, lon
                     if (p.level) p.level[u] = d + 1;
                 }
                 st.cnt += __popc(cm);
-                if (st.cnt > kStage - 32) stage_flush(p, st, qnext, tail, acc_m);
+                if (st.cnt > kStage - 32) stage_flush<false>(p, st, qnext, tail, acc_m);
             }
         }
     }
-    stage_flush(p, st, qnext, tail, acc_m);
+    stage_flush<false>(p, st, qnext, tail, acc_m);
     __syncthreads();
     for (long long w = threadIdx.x; w < nbw; w += blockDim.x) p.visited[wbase + w] = s_own[w];
 }
@@ -2472,21 +2456,23 @@ using bfsk::SingleParams;
 using bfsk::Hub;
 
 // the CSR kernel's variants: any parent over the id-ordered rows, over the hub-first
-// rows, and minimum-id parents (id-ordered rows only); each without and with
-// cluster levels
-enum CsrVariant { kCsrId, kCsrHub, kCsrMin, kCsrVariants };
+// rows, and minimum-id parents (id-ordered rows only), each without and with
+// cluster levels; and the two that a directed graph has
+enum CsrVariant { kCsrId, kCsrHub, kCsrMin, kCsrDirId, kCsrDirMin, kCsrVariants };
 static const void* csr_kernel(int variant, bool clu) {
     using namespace bfsk;
     switch (variant) {
         case kCsrHub:
-            return clu ? (const void*)bfs_single_kernel<false, true, true>
-                       : (const void*)bfs_single_kernel<false, true, false>;
+            return clu ? (const void*)bfs_single_kernel<false, true, true, false>
+                       : (const void*)bfs_single_kernel<false, true, false, false>;
         case kCsrMin:
-            return clu ? (const void*)bfs_single_kernel<true, false, true>
-                       : (const void*)bfs_single_kernel<true, false, false>;
+            return clu ? (const void*)bfs_single_kernel<true, false, true, false>
+                       : (const void*)bfs_single_kernel<true, false, false, false>;
+        case kCsrDirId: return (const void*)bfs_single_kernel<false, false, false, true>;
+        case kCsrDirMin: return (const void*)bfs_single_kernel<true, false, false, true>;
         default:
-            return clu ? (const void*)bfs_single_kernel<false, false, true>
-                       : (const void*)bfs_single_kernel<false, false, false>;
+            return clu ? (const void*)bfs_single_kernel<false, false, true, false>
+                       : (const void*)bfs_single_kernel<false, false, false, false>;
     }
 }
 
@@ -2701,7 +2687,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
             cfg.attrs = at;
             cfg.numAttrs = 1;
             int ncl = INT_MAX;
-            for (int m = 0; m < kCsrVariants; m++) {
+            for (int m : {kCsrId, kCsrHub, kCsrMin}) {
                 int k = 0;
                 BFS_CUDA_TRY(cudaFuncSetAttribute(csr_kernel(m, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
                 BFS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&k, csr_kernel(m, true), &cfg));
@@ -2723,7 +2709,8 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         p.clu_nf = (long long)C * (bfsk::kCluCap / 2);
         p.clu_mf = (long long)C * bfsk::kCluEdgesPerCta;
     }
-    const int variant = opt.parent_mode == BFS_PARENT_MIN_ID && parent ? kCsrMin : p.first ? kCsrHub : kCsrId;
+    const bool min_id = opt.parent_mode == BFS_PARENT_MIN_ID && parent;
+    const int variant = g->directed ? (min_id ? kCsrDirMin : kCsrDirId) : min_id ? kCsrMin : p.first ? kCsrHub : kCsrId;
     void* args[] = {&p};
     BFS_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(Ctrl), s));
     if (k > 1) BFS_CUDA_TRY(cudaMemcpyAsync(w.queue0, roots_host, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, s));
