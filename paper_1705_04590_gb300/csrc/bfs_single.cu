@@ -58,7 +58,10 @@ constexpr int kStage = 256;    // per-warp shared-memory staging of next-queue e
 // staging slices, and bottom-up phase A's searcher lists, whose two halves are
 // the frontier buffers of the cluster levels.
 __shared__ __align__(16) int g_stage[kBlock / 32][kStage];
-__shared__ __align__(16) int g_stage_d[kDBlock / 32][kStage];   // the DCSC kernel's (more warps per CTA)
+// the DCSC kernel's slices (more warps, and two vertex bitmaps beside them): staging,
+// then a list of columns
+constexpr int kDStage = 128, kDList = 64;
+__shared__ __align__(16) int g_stage_d[kDBlock / 32][kDStage + kDList];
 __shared__ __align__(16) unsigned short g_list[kBlock / 32][1024];
 constexpr long long kPrefetchNf = 1 << 16;   // top-down levels below this prefetch the next rows
 #ifndef BFS_TD_CHECK
@@ -139,6 +142,7 @@ struct SingleParams {
     int nb;            // p blocks
     long long B;       // vertices per block (multiple of 32)
     long long Bw;      // words per block
+    long long dcsc_stream;   // (frontier vertices x p) from which a top-down level streams JC
 };
 
 constexpr int TD = 0, BU = 1;
@@ -2135,6 +2139,50 @@ __device__ __forceinline__ long long block_words(const SingleParams& p, int b) {
     return w1 > w0 ? w1 - w0 : 0;
 }
 
+// Claim the rows of the lanes' columns (column k of a lane at IR entries cs..ce;
+// all lanes call): the warp gathers them edge by edge.
+__device__ __forceinline__ void dcsc_claim(const SingleParams& p, int d, int k, long long cs, long long ce,
+                                           unsigned* s_own, const unsigned* s_old, bool min_id, WarpStage& st,
+                                           int* qnext, unsigned long long* tail, unsigned long long& acc_m) {
+    const int b = blockIdx.x, lane = lane_id();
+    const int mydeg = (int)(ce - cs);
+    const int incl = warp_inclusive_scan(mydeg);
+    const int total = __shfl_sync(kFull, incl, 31);
+    const int excl = incl - mydeg;
+    for (int k0 = 0; k0 < total; k0 += 32) {
+        const int kk = k0 + lane;
+        int j = 0;
+#pragma unroll
+        for (int step = 16; step >= 1; step >>= 1) {
+            const int c = __shfl_sync(kFull, incl, j + step - 1);
+            if (c <= kk) j += step;
+        }
+        const long long cj = __shfl_sync(kFull, cs, j);
+        const int exj = __shfl_sync(kFull, excl, j);
+        const int kj = __shfl_sync(kFull, k, j);
+        bool claimed = false;
+        int u = 0;
+        if (kk < total) {
+            const int ul = __ldg(p.ir + cj + (kk - exj));
+            const unsigned bit = 1u << (ul & 31);
+            if (!(s_own[ul >> 5] & bit)) claimed = !(atomicOr(s_own + (ul >> 5), bit) & bit);
+            u = (int)((long long)b * p.B + ul);
+            if (min_id && !(s_old[ul >> 5] & bit))
+                atomicMin(reinterpret_cast<unsigned*>(p.parent) + u, (unsigned)kj);
+        }
+        const unsigned cm = __ballot_sync(kFull, claimed);
+        if (cm) {
+            if (claimed) {
+                st.buf[st.cnt + __popc(cm & lanemask_lt())] = u;
+                if (p.parent && !min_id) p.parent[u] = kj;
+                if (p.level) p.level[u] = d + 1;
+            }
+            st.cnt += __popc(cm);
+            if (st.cnt > kDStage - 32) stage_flush<false>(p, st, qnext, tail, acc_m);
+        }
+    }
+}
+
 // Top-down on tiles (b, *) (Algorithm 3's local discovery, t = A_bj * f_j):
 // every CTA reads the whole frontier queue, finds each frontier vertex k's
 // column in its tile (b, block(k)) by binary search over JC, and claims the
@@ -2177,47 +2225,136 @@ __device__ void td_dcsc_phase(const SingleParams& p, int d, const int* qcur, lon
                 ce = __ldg(p.cp + lo + 1);
             }
         }
-        const int mydeg = (int)(ce - cs);
-        const int incl = warp_inclusive_scan(mydeg);
-        const int total = __shfl_sync(kFull, incl, 31);
-        const int excl = incl - mydeg;
-        for (int k0 = 0; k0 < total; k0 += 32) {
-            const int kk = k0 + lane;
-            int j = 0;
-#pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const int c = __shfl_sync(kFull, incl, j + step - 1);
-                if (c <= kk) j += step;
-            }
-            const long long cj = __shfl_sync(kFull, cs, j);
-            const int exj = __shfl_sync(kFull, excl, j);
-            const int kj = __shfl_sync(kFull, k, j);
-            bool claimed = false;
-            int u = 0;
-            if (kk < total) {
-                const int ul = __ldg(p.ir + cj + (kk - exj));
-                const unsigned bit = 1u << (ul & 31);
-                if (!(s_own[ul >> 5] & bit)) claimed = !(atomicOr(s_own + (ul >> 5), bit) & bit);
-                u = (int)((long long)b * p.B + ul);
-                if (min_id && !(s_old[ul >> 5] & bit))
-                    atomicMin(reinterpret_cast<unsigned*>(p.parent) + u, (unsigned)kj);
-            }
-            const unsigned cm = __ballot_sync(kFull, claimed);
-            if (cm) {
-                if (claimed) {
-                    st.buf[st.cnt + __popc(cm & lanemask_lt())] = u;
-                    if (p.parent && !min_id) p.parent[u] = kj;
-                    if (p.level) p.level[u] = d + 1;
-                }
-                st.cnt += __popc(cm);
-                if (st.cnt > kStage - 32) stage_flush<false>(p, st, qnext, tail, acc_m);
-            }
-        }
+        dcsc_claim(p, d, k, cs, ce, s_own, s_old, min_id, st, qnext, tail, acc_m);
     }
     stage_flush<false>(p, st, qnext, tail, acc_m);
     __syncthreads();
     for (long long w = threadIdx.x; w < nbw; w += blockDim.x) p.visited[wbase + w] = s_own[w];
 }
+
+// A CTA's tiles as units of at most kUnit column entries for its warps, whatever
+// the tiles' sizes: pref[t] units lie in the tiles before the t-th.  Taken tile by
+// tile by the whole CTA instead, a tile's few entries per thread (2 at R-MAT 22)
+// leave each of the 152 tiles a chain of dependent reads of its own.
+constexpr int kUnit = 512;
+
+// the unit counts of `nb` tiles, tile t at tile_ptr[first + t * step]; every thread calls
+__device__ void tile_units(const SingleParams& p, long long first, long long step, int* pref) {
+    if (threadIdx.x == 0) pref[0] = 0;
+    for (int t = threadIdx.x; t < p.nb; t += blockDim.x) {
+        const long long at = first + t * step;
+        pref[t + 1] = (int)((__ldg(p.tile_ptr + at + 1) - __ldg(p.tile_ptr + at) + kUnit - 1) / kUnit);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        int run = 0;
+        for (int t0 = 0; t0 < p.nb; t0 += 32) {
+            const int t = t0 + lane_id();
+            const int incl = warp_inclusive_scan(t < p.nb ? pref[t + 1] : 0);
+            if (t < p.nb) pref[t + 1] = run + incl;
+            run += __shfl_sync(kFull, incl, 31);
+        }
+    }
+    __syncthreads();
+}
+
+// unit `unit`'s tile and its range of column entries (the same in every lane)
+__device__ __forceinline__ int tile_unit(const SingleParams& p, long long first, long long step, const int* pref,
+                                         int unit, long long& lo, long long& hi) {
+    int t = 0, n = p.nb;
+    while (n > 1) {
+        const int h = n >> 1;
+        if (pref[t + h] <= unit) t += h;
+        n -= h;
+    }
+    const long long at = first + t * step;
+    lo = __ldg(p.tile_ptr + at) + (long long)(unit - pref[t]) * kUnit;
+    hi = min(__ldg(p.tile_ptr + at + 1), lo + kUnit);
+    return t;
+}
+
+// Frontier bit v of a tile's segment.  A warp stays in a tile for a unit, so the
+// segment (3 KB at R-MAT 22) is worth its place in L1; the grid barrier before the
+// level dropped what L1 held of it.
+__device__ __forceinline__ bool seg_bit(const unsigned* fseg, int v) {
+    return (__ldca(fseg + (v >> 5)) >> (v & 31)) & 1u;
+}
+
+// Top-down on a large frontier: every column of the tiles (b, *) is tested
+// against the frontier's bitmap, one stream over JC, where the search for each
+// frontier vertex's column in every tile is a chain of a dozen dependent reads
+// (R-MAT 22, 134 K vertices: 465 us that way, 164 us so).
+__device__ void td_dcsc_stream(const SingleParams& p, int d, const unsigned* f, int* qnext, int snext, unsigned* s_own,
+                               unsigned* s_old, const int* pref, unsigned long long& acc_m) {
+    const int b = blockIdx.x, lane = lane_id(), wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
+    const long long nbw = block_words(p, b), wbase = (long long)b * p.Bw;
+    const bool min_id = p.parent_mode == BFS_PARENT_MIN_ID && p.parent;
+    for (long long w = threadIdx.x; w < nbw; w += blockDim.x) {
+        const unsigned x = __ldcg(p.visited + wbase + w);
+        s_own[w] = x;
+        if (min_id) s_old[w] = x;
+    }
+    __syncthreads();
+    unsigned long long* tail = &p.ctrl->lv[snext].tail;
+    WarpStage st = warp_stage_dcsc();
+    int* list = g_stage_d[wib] + kDStage;   // columns found, unit-relative
+    const long long first = (long long)b * p.nb;
+    for (int unit = wib; unit < pref[p.nb]; unit += nwb) {
+        long long lo, hi;
+        const int j = tile_unit(p, first, 1, pref, unit, lo, hi);
+        const unsigned* fseg = f + (long long)j * p.Bw;
+        int np = 0;
+        // the list's last `n` columns (all lanes call)
+        auto claim = [&](int n) {
+            __syncwarp();
+            int k = -1;
+            long long cs = 0, ce = 0;
+            if (lane < n) {
+                const long long x = lo + list[np - n + lane];
+                k = (int)((long long)j * p.B + __ldg(p.jc + x));
+                cs = __ldg(p.cp + x);
+                ce = __ldg(p.cp + x + 1);
+            }
+            np -= n;
+            __syncwarp();
+            dcsc_claim(p, d, k, cs, ce, s_own, s_old, min_id, st, qnext, tail, acc_m);
+        };
+        for (long long x0 = lo; x0 < hi; x0 += 128) {
+            int kl[4];
+            unsigned in = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const long long x = x0 + q * 32 + lane;
+                kl[q] = x < hi ? __ldg(p.jc + x) : -1;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (kl[q] >= 0 && seg_bit(fseg, kl[q])) in |= 1u << q;
+            // the columns of frontier vertices, 32 at a time
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const unsigned m = __ballot_sync(kFull, (in >> q) & 1u);
+                if ((in >> q) & 1u) list[np + __popc(m & lanemask_lt())] = (int)(x0 - lo) + q * 32 + lane;
+                np += __popc(m);
+                if (np >= 32) claim(32);
+            }
+        }
+        claim(np);
+    }
+    stage_flush<false>(p, st, qnext, tail, acc_m);
+    __syncthreads();
+    for (long long w = threadIdx.x; w < nbw; w += blockDim.x) p.visited[wbase + w] = s_own[w];
+}
+
+// column u of tile (i, blockIdx.x) has row v in the frontier
+__device__ __forceinline__ void dcsc_found(const SingleParams& p, int d, int i, int ul, int vl, unsigned* s_own) {
+    const long long u = (long long)blockIdx.x * p.B + ul;
+    if (p.parent) p.parent[u] = (int)((long long)i * p.B + vl);
+    if (p.level) p.level[u] = d + 1;
+    atomicOr(s_own + (ul >> 5), 1u << (ul & 31));
+}
+constexpr int kOwnSteps = 2;     // entries of a column that its own lane tests
+constexpr int kGroupSteps = 16;  // steps of four more by four lanes, before the whole warp takes it
 
 // Bottom-up on tiles (*, b) (Algorithm 4's sub-steps without messages): the
 // CTA owning block b walks the p tiles of its column of the grid; each
@@ -2227,10 +2364,10 @@ __device__ void td_dcsc_phase(const SingleParams& p, int d, const int* qcur, lon
 // level.  With minimum-id parents the tiles run 0..p-1 with the frontier
 // segment of block i staged in shared memory and a CTA barrier between tiles
 // (so a searcher stops at its first frontier neighbour in id order); with any
-// parent the tile order rotates with b, the segment is probed in L2, and tiles
-// follow one another without barriers.
+// parent the warps take units of the tiles (`pref`) side by side and the segment is
+// probed in L2.
 __device__ void bu_dcsc_phase(const SingleParams& p, int d, const unsigned* fcur, unsigned* fnext, unsigned* s_own,
-                              unsigned* s_seg, unsigned long long& acc_n, unsigned long long& acc_m,
+                              unsigned* s_seg, const int* pref, unsigned long long& acc_n, unsigned long long& acc_m,
                               unsigned long long& acc_sc, unsigned long long& acc_ex) {
     const int b = blockIdx.x;
     const long long nbw = block_words(p, b), wbase = (long long)b * p.Bw;
@@ -2240,39 +2377,124 @@ __device__ void bu_dcsc_phase(const SingleParams& p, int d, const unsigned* fcur
         acc_sc += (unsigned long long)__popc(~x);
     }
     if (p.parent_mode != BFS_PARENT_MIN_ID) {
-        // any parent will do: tiles in rotated order with no staging and no barrier
-        // between them (the frontier segment is probed in L2), four column entries per
-        // thread in flight.  A searcher found in two tiles at once gets either parent.
-        for (int t = 0; t < p.nb; t++) {
-            const int i = (b + t) % p.nb;
+        // any parent will do: units of the tiles to the warps, no staging and no barrier
+        // between tiles (the frontier segment is probed in L2), four column entries per
+        // lane in flight at every step.  A searcher found in two tiles at once gets
+        // either parent.
+        __syncthreads();
+        const int lane = lane_id(), wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
+        int* list = g_stage_d[wib];   // columns of a step that go on past their lane's entries
+        for (int unit = wib; unit < pref[p.nb]; unit += nwb) {
+            long long lo, hi;
+            const int i = tile_unit(p, b, p.nb, pref, unit, lo, hi);
             const unsigned* fseg = fcur + (long long)i * p.Bw;
-            const long long tt = (long long)i * p.nb + b;
-            const long long lo = __ldg(p.tile_ptr + tt), hi = __ldg(p.tile_ptr + tt + 1);
-            for (long long x0 = lo + threadIdx.x; x0 < hi; x0 += 4LL * blockDim.x) {
-                int ul[4];
+            int nx[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) nx[k] = lo + k * 32 + lane < hi ? __ldg(p.jc + lo + k * 32 + lane) : -1;
+            for (long long x0 = lo; x0 < hi; x0 += 128) {
+                int ul[4], vl[4], left[4];
+                long long e[4];
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
-                    const long long x = x0 + (long long)k * blockDim.x;
-                    ul[k] = x < hi ? __ldg(p.jc + x) : -1;
+                    ul[k] = nx[k];
+                    const long long x = x0 + 128 + k * 32 + lane;
+                    nx[k] = x < hi ? __ldg(p.jc + x) : -1;
                 }
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
-                    if (ul[k] < 0 || ((s_own[ul[k] >> 5] >> (ul[k] & 31)) & 1u)) continue;
-                    const long long x = x0 + (long long)k * blockDim.x;
-                    const long long e0 = __ldg(p.cp + x), e1 = __ldg(p.cp + x + 1);
-                    for (long long e = e0; e < e1; e++) {
-                        const int vl = __ldg(p.ir + e);
-                        if ((__ldcg(fseg + (vl >> 5)) >> (vl & 31)) & 1u) {
-                            const long long u = (long long)b * p.B + ul[k];
-                            if (p.parent) p.parent[u] = (int)((long long)i * p.B + vl);
-                            if (p.level) p.level[u] = d + 1;
-                            atomicOr(s_own + (ul[k] >> 5), 1u << (ul[k] & 31));
-                            acc_ex += (unsigned long long)(e - e0 + 1);
-                            break;
-                        }
-                        if (e + 1 == e1) acc_ex += (unsigned long long)(e1 - e0);
+                    left[k] = 0;
+                    e[k] = 0;
+                    if (ul[k] >= 0 && !((s_own[ul[k] >> 5] >> (ul[k] & 31)) & 1u)) {
+                        const long long x = x0 + k * 32 + lane;
+                        e[k] = __ldg(p.cp + x);
+                        left[k] = (int)(__ldg(p.cp + x + 1) - e[k]);
                     }
                 }
+                // a column's first entries by its own lane
+#pragma unroll 1
+                for (int step = 0; step < kOwnSteps && __any_sync(kFull, left[0] | left[1] | left[2] | left[3]); step++) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) vl[k] = left[k] ? __ldg(p.ir + e[k] + step) : 0;
+                    bool in[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) in[k] = left[k] && seg_bit(fseg, vl[k]);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        if (!left[k]) continue;
+                        left[k]--;
+                        if (in[k]) {
+                            dcsc_found(p, d, i, ul[k], vl[k], s_own);
+                            left[k] = 0;
+                        }
+                        if (!left[k]) acc_ex += (unsigned long long)(step + 1);
+                    }
+                }
+                // longer columns: eight at a time, four lanes each
+                int np = 0;
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const unsigned m = __ballot_sync(kFull, left[k] > 0);
+                    if (left[k] > 0) list[np + __popc(m & lanemask_lt())] = (int)(x0 - lo) + k * 32 + lane;
+                    np += __popc(m);
+                }
+                __syncwarp();
+                const int grp = lane >> 2, gl = lane & 3;
+                for (int r0 = 0; r0 < np; r0 += 8) {
+                    const bool has = r0 + grp < np;
+                    long long ea = 0, e1 = 0, e0 = 0;
+                    int u = 0;
+                    if (has) {
+                        const long long x = lo + list[r0 + grp];
+                        u = __ldg(p.jc + x);
+                        e0 = __ldg(p.cp + x);
+                        e1 = __ldg(p.cp + x + 1);
+                        ea = e0 + kOwnSteps;
+                    }
+                    bool live = has;
+                    for (int step = 0; step < kGroupSteps && __any_sync(kFull, live); step++) {
+                        int v = 0;
+                        bool in = false;
+                        if (live && ea + gl < e1) {
+                            v = __ldg(p.ir + ea + gl);
+                            in = seg_bit(fseg, v);
+                        }
+                        const unsigned gm = (__ballot_sync(kFull, in) >> (grp * 4)) & 0xFu;
+                        if (live) {
+                            if (gm) {
+                                const int h = __ffs(gm) - 1;
+                                if (gl == h) dcsc_found(p, d, i, u, v, s_own);
+                                if (gl == 0) acc_ex += (unsigned long long)(ea + h + 1 - e0);
+                                live = false;
+                            } else if (ea + 4 >= e1) {
+                                if (gl == 0) acc_ex += (unsigned long long)(e1 - e0);
+                                live = false;
+                            }
+                            ea += 4;
+                        }
+                    }
+                    // what is left of a hub's column: the whole warp
+                    unsigned lm = __ballot_sync(kFull, live && gl == 0);
+                    while (lm) {
+                        const int L = __ffs(lm) - 1;
+                        lm &= lm - 1;
+                        long long q = __shfl_sync(kFull, ea, L);
+                        const long long q0 = __shfl_sync(kFull, e0, L), q1 = __shfl_sync(kFull, e1, L);
+                        const int uu = __shfl_sync(kFull, u, L);
+                        unsigned m = 0;
+                        for (; q < q1 && !m; q += 32) {
+                            int v = 0;
+                            bool in = false;
+                            if (q + lane < q1) {
+                                v = __ldg(p.ir + q + lane);
+                                in = seg_bit(fseg, v);
+                            }
+                            m = __ballot_sync(kFull, in);
+                            if (m && lane == __ffs(m) - 1) dcsc_found(p, d, i, uu, v, s_own);
+                        }
+                        if (lane == 0) acc_ex += (unsigned long long)(m ? q - 32 + __ffs(m) - q0 : q1 - q0);
+                    }
+                }
+                __syncwarp();
             }
         }
     }
@@ -2324,6 +2546,10 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
     extern __shared__ unsigned dyn[];
     unsigned* s_own = dyn;
     unsigned* s_seg = dyn + p.Bw;
+    int* s_urow = reinterpret_cast<int*>(dyn + 2 * p.Bw);   // units of the tiles (b, *), top-down
+    int* s_ucol = s_urow + p.nb + 1;                        // ... and of (*, b), bottom-up
+    tile_units(p, (long long)blockIdx.x * p.nb, 1, s_urow);
+    tile_units(p, blockIdx.x, p.nb, s_ucol);
     Ctrl* c = p.ctrl;
     __shared__ LevelCtr s_ctr;   // the last completed level's counters
     init_phase(p);
@@ -2358,7 +2584,18 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             unsigned long long am = 0;
-            td_dcsc_phase(p, d, qcur, nf, qnext, snext, s_own, s_seg, am);
+            if (nf * p.nb >= p.dcsc_stream) {
+                // the frontier's bitmap goes into the idle one (a bottom-up level overwrites it whole)
+                unsigned* f = fnext;
+                const long long nbw = block_words(p, blockIdx.x), wbase = (long long)blockIdx.x * p.Bw;
+                for (long long w = threadIdx.x; w < nbw; w += blockDim.x) f[wbase + w] = 0u;
+                if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+                queue_to_bitmap(p, qcur, nf, f);
+                if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+                td_dcsc_stream(p, d, f, qnext, snext, s_own, s_seg, s_urow, am);
+            } else {
+                td_dcsc_phase(p, d, qcur, nf, qnext, snext, s_own, s_seg, am);
+            }
             block_add4(0, am, 0, 0, nullptr, &c->lv[snext].accm, nullptr, nullptr);
             if (!level_sync(p, snext, s_ctr)) return;
             nf_next = (long long)s_ctr.tail;
@@ -2369,7 +2606,7 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             unsigned long long an = 0, am = 0, asc = 0, aex = 0;
-            bu_dcsc_phase(p, d, fcur, fnext, s_own, s_seg, an, am, asc, aex);
+            bu_dcsc_phase(p, d, fcur, fnext, s_own, s_seg, s_ucol, an, am, asc, aex);
             block_add4(an, am, asc, aex, &c->lv[snext].accn, &c->lv[snext].accm, &c->lv[snext].scanned, &c->lv[snext].examined);
             if (!level_sync(p, snext, s_ctr)) return;
             nf_next = (long long)s_ctr.accn;
@@ -2490,6 +2727,11 @@ static cudaError_t csr_occupancy(int* per_sm) {
     }
     return cudaSuccess;
 }
+
+// A column search in a tile costs about as much as kDcscStream entries of the JC
+// stream (R-MAT 22: a level of 13 K vertices x 152 tiles 70 us by searches, of 134 K
+// 465 us; the stream 90 to 165 us for frontiers of up to a few hundred thousand).
+constexpr long long kDcscStream = 16;
 
 // Hub lists: rows of degree > big_deg (>= kMinChunk), those of class j >= 1 of degree
 // > (4^j - 1) * td_chunk (>= kMinChunk).  The classes' most rows add up to less than
@@ -2640,6 +2882,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     p.nb = 0;
     p.B = 0;
     p.Bw = 0;
+    p.dcsc_stream = 0;
     const bool dcsc = opt.layout == BFS_LAYOUT_DCSC_TILED;
     int grid = w.grid, block = w.block;
     if (opt.ctas_per_sm > 0 && (long long)opt.ctas_per_sm * g->sm_count < grid) {
@@ -2656,7 +2899,8 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
         p.nb = D.num_blocks;
         p.B = D.block_size;
         p.Bw = D.block_size / 32;
-        dyn = sizeof(unsigned) * 2 * (size_t)p.Bw;
+        p.dcsc_stream = D.nzc / kDcscStream + 1;
+        dyn = sizeof(unsigned) * 2 * (size_t)p.Bw + sizeof(int) * 2 * (size_t)(p.nb + 1);
         BFS_CUDA_TRY(cudaFuncSetAttribute(bfsk::bfs_dcsc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         int occ = 0;
         BFS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bfsk::bfs_dcsc_kernel, bfsk::kDBlock, dyn));

@@ -199,3 +199,40 @@ def test_hub_slices_at_class_edges(gpu_lib, big, chunk):
         for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext"]):
             assert np.array_equal(info["records"][:, col], getattr(s, name)), name
     g.close()
+
+
+@pytest.mark.parametrize("shape", ["hub", "er", "tiny", "union"])
+@pytest.mark.parametrize("min_id", [False, True])
+def test_dcsc_streams_and_long_columns(gpu_lib, shape, min_id):
+    """Tiles whose columns run past a lane's, a group's and a warp's share of them, tiles of
+    several units, empty tiles, frontiers on both sides of the streaming rule."""
+    bfs = gpu_lib
+    rng = np.random.default_rng(11)
+    if shape == "hub":
+        n = 20_000
+        h = rng.integers(0, n, 6)
+        e = graphgen.EdgeList(n, np.concatenate([np.repeat(h, 9000), rng.integers(0, n, 30_000)]).astype(np.int32),
+                              np.concatenate([rng.integers(0, n, 54_000), rng.integers(0, n, 30_000)]).astype(np.int32))
+    elif shape == "er":
+        e = graphgen.erdos_renyi(150_001, 1_500_000, seed=3)
+    elif shape == "tiny":
+        e = graphgen.random_small(65, 400, 2)
+    else:
+        e, _ = graphgen.disjoint_union([graphgen.complete(60), graphgen.path(9000), graphgen.star(3000)])
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, dcsc=True)
+    level, parent = _buffers(e.n)
+    for root in graphgen.pick_roots(e, 3, 1).tolist():
+        want = oracle.levels(ref, root)
+        for mode in (bfs.MODE_DO, bfs.MODE_TD_ONLY, bfs.MODE_BU_ONLY):
+            if mode == bfs.MODE_BU_ONLY and want.max() > 2000:
+                continue
+            g.run(root, parent=parent, level=level,
+                  opts=bfs.options(mode=mode, layout=bfs.LAYOUT_DCSC_TILED,
+                                   parent_mode=bfs.PARENT_MIN_ID if min_id else bfs.PARENT_ANY))
+            pa = parent.cpu().numpy()
+            assert np.array_equal(level.cpu().numpy(), want), (root, mode)
+            assert oracle.certify(ref, root, want, pa, labels) == (0, -1), (root, mode)
+            assert not min_id or np.array_equal(pa, oracle.min_parent(ref, want)), (root, mode)
+    g.close()
