@@ -130,6 +130,7 @@ struct SingleParams {
     // clu_nf vertices and clu_mf edges and no vertex of degree above clu_big
     // (0 when off: the top-down flushes then count no heavy vertices)
     int clu_c, clu_big;
+    int clu_d;         // lanes per frontier entry on graphs of degree <= 4 or 8 (clu_expand_short), else 0
     long long clu_nf, clu_mf;
     unsigned long long seed;
     unsigned long long timeout_ns;
@@ -1574,9 +1575,17 @@ __device__ __forceinline__ unsigned clu_nranks() {
 // shared-memory (local and remote) writes before it against reads after it.
 // The aligned form (the warp executes it together, as after the __syncwarp)
 // keeps the kernel's register allocation intact; the unaligned form does not.
-__device__ __forceinline__ void clu_sync() {
+__device__ __forceinline__ void clu_arrive() {
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void clu_await() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void clu_sync() {
+    clu_arrive();
+    clu_await();
 }
 // the shared::cluster address of `local` in CTA `rank` of this cluster
 __device__ __forceinline__ unsigned clu_map(const void* local, unsigned rank) {
@@ -1597,6 +1606,15 @@ __device__ __forceinline__ void clu_st64(unsigned addr, unsigned long long x) {
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(x) : "memory");
 }
 
+// A vertex's outputs are written when it is expanded, from its entry, and not when
+// it is claimed: the cluster barrier's release waits for the stores before it, and
+// here they are most of a level old.  par < 0: the grid wrote them.
+__device__ __forceinline__ void clu_outputs(const SingleParams& p, int v, int par, int lev) {
+    if (par < 0) return;
+    if (p.parent) p.parent[v] = par;
+    set_level(p, v, lev);
+}
+
 // Per-CTA summaries of a frontier, pushed by each CTA into every CTA of the
 // cluster: [parity][rank] = {entries | heavy << 15 | spilled << 32, degree sum}.
 __shared__ unsigned long long g_csum[2][kCluMaxC][2];
@@ -1607,30 +1625,133 @@ struct CluState {
     bool done;
 };
 
+// Expand level L of a frontier whose degrees are at most kD (4 or 8), in place of
+// clu_expand: kD lanes per entry, which they read themselves, so that neither a
+// scan of degrees nor a search for each lane's edge stands before the column
+// reads.  While the CTAs' shares are even enough each expands its own entries (a
+// plain shared-memory read); else they are numbered CTA by CTA and shared out
+// again.  A level of a few hundred vertices is a chain of dependent steps, and a
+// third of it was instructions around the reads (torus of 512^2: 4.6 us a level,
+// 3.7 us so; of 4096^2: 27.1 ms a search, 22.4 ms).
+template <int kD>
+__device__ void clu_expand_short(const SingleParams& p, int L, int C, int r, int mine, int nf, const CluEntry* cur,
+                                 CluEntry* next, int* s_lcnt, unsigned long long& acc_m, unsigned& acc_h) {
+    constexpr int kPer = 32 / kD;   // entries of a warp's round
+    const int lane = lane_id(), nwb = blockDim.x >> 5, wib = threadIdx.x >> 5;
+    const int most = (int)__reduce_max_sync(kFull, (unsigned)mine);
+    // own entries: at most one round of every warp, or a quarter over the average
+    const int clog = 31 - __clz(C);   // C is a power of two
+    const bool own = most <= max(nwb * kPer, (nf + (nf >> 2)) >> clog);
+    const int upto = own ? 0 : warp_inclusive_scan(mine);
+    const int n = own ? __shfl_sync(kFull, mine, r) : nf;
+    const int w0 = own ? wib : r * nwb + wib, nw = own ? nwb : C * nwb;
+    for (int s0 = w0; s0 * kPer < n; s0 += 4 * nw) {
+        long long row[4];
+        int deg[4], u[4], par[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int i = (s0 + q * nw) * kPer + lane / kD;
+            deg[q] = 0;
+            u[q] = 0;
+            par[q] = -1;
+            row[q] = 0;
+            if (own) {
+                if (i < n) {
+                    const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(cur + i);
+                    row[q] = (long long)(e.x & ((1ull << kCluDegShift) - 1ull));
+                    deg[q] = (int)(e.x >> kCluDegShift);
+                    u[q] = (int)(unsigned)e.y;
+                    par[q] = (int)(unsigned)(e.y >> 32);
+                }
+            } else {
+                int o = 0;
+#pragma unroll
+                for (int step = kCluMaxC / 2; step >= 1; step >>= 1)
+                    if (__shfl_sync(kFull, upto, o + step - 1) <= i) o += step;
+                const int at = i - __shfl_sync(kFull, upto - mine, o);
+                if (i < n && at < kCluCap) clu_ld_entry(clu_map(cur + at, (unsigned)o), row[q], deg[q], u[q], par[q]);
+            }
+        }
+        // columns, then claims, then the claimed rows' offsets, each four in flight
+        // together; the edge back to a vertex's parent is known visited and skipped
+        int v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) v[q] = lane % kD < deg[q] ? __ldg(p.cols + row[q] + lane % kD) : -1;
+        // the entries' outputs, a lane of each group one of the four
+        {
+            const int q = lane % kD;
+            const int uu = q == 0 ? u[0] : q == 1 ? u[1] : q == 2 ? u[2] : u[3];
+            const int pp = q == 0 ? par[0] : q == 1 ? par[1] : q == 2 ? par[2] : par[3];
+            if (q < 4) clu_outputs(p, uu, pp, L);
+        }
+        unsigned old[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            old[q] = kFull;
+            if (v[q] >= 0 && v[q] != par[q]) old[q] = atomicOr(p.visited + (v[q] >> 5), 1u << (v[q] & 31));
+        }
+        bool cl[4];
+        unsigned m[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            cl[q] = !((old[q] >> (v[q] & 31)) & 1u);
+            m[q] = __ballot_sync(kFull, cl[q]);
+        }
+        long long rs[4], re[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            rs[q] = re[q] = 0;
+            if (cl[q]) row_of(p, v[q], rs[q], re[q]);
+        }
+        const int c0 = __popc(m[0]), c1 = c0 + __popc(m[1]), c2 = c1 + __popc(m[2]), c3 = c2 + __popc(m[3]);
+        if (c3 == 0) continue;
+        int pos = 0;
+        if (lane == 0) pos = atomicAdd(s_lcnt, c3);
+        pos = __shfl_sync(kFull, pos, 0);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (!cl[q]) continue;
+            const int at = pos + (q == 0 ? 0 : q == 1 ? c0 : q == 2 ? c1 : c2) + __popc(m[q] & lanemask_lt());
+            const long long dg = re[q] - rs[q];
+            acc_m += (unsigned long long)dg;
+            acc_h |= dg > (long long)p.clu_big;
+            if (dg > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.cols + rs[q]));
+            if (at < kCluCap) {
+                CluEntry e;
+                e.row = clu_row(rs[q], dg);
+                e.v = v[q];
+                e.par = u[q];
+                next[at] = e;
+            } else {
+                p.queue0[atomicAdd(&p.ctrl->clu_spill, 1ull)] = v[q];
+                clu_outputs(p, v[q], u[q], L + 1);
+            }
+        }
+    }
+}
+
 // Expand level L of the cluster's frontier (entries in `cur` of every CTA,
 // counts in g_csum[b]) into this CTA's `next` buffer.  Entries past the
 // buffer spill to the front of queue0 (the level after is then the grid's).
-__device__ void clu_expand(const SingleParams& p, int L, int C, int r, int b, long long nf, const CluEntry* cur,
+__device__ void clu_expand(const SingleParams& p, int L, int C, int r, int mine, long long nf, const CluEntry* cur,
                            CluEntry* next, int* s_lcnt, unsigned long long& acc_m, unsigned& acc_h) {
     const int lane = lane_id(), nwb = blockDim.x >> 5, wib = threadIdx.x >> 5;
     const long long cw = (long long)r * nwb + wib, ncw = (long long)C * nwb;
     const long long per = nf >= ncw * 32 ? 32 : max(1LL, (nf + ncw - 1) / ncw);
+    // the entries are numbered CTA by CTA: lane q holds the entries up to CTA q's end
+    const int upto = warp_inclusive_scan(mine);
     for (long long base = cw * per; base < nf; base += ncw * per) {
         const long long i = base + lane;
         int u = 0, deg = 0, pu = -1;
         long long s = 0;
-        if (lane < per && i < nf) {
-            // owner CTA of entry i (the entries are numbered CTA by CTA)
-            int q = 0;
-            long long acc = 0;
-            while (q < C - 1) {
-                const long long c = (long long)(g_csum[b][q][0] & kCluCntMask);
-                if (i < acc + c) break;
-                acc += c;
-                q++;
-            }
-            if (i - acc < kCluCap) clu_ld_entry(clu_map(cur + (i - acc), (unsigned)q), s, deg, u, pu);
-        }
+        // owner CTA of entry i
+        int q = 0;
+#pragma unroll
+        for (int step = kCluMaxC / 2; step >= 1; step >>= 1)
+            if (__shfl_sync(kFull, upto, q + step - 1) <= i) q += step;
+        const int at = (int)i - __shfl_sync(kFull, upto - mine, q);
+        if (lane < per && i < nf && at < kCluCap) clu_ld_entry(clu_map(cur + at, (unsigned)q), s, deg, u, pu);
+        clu_outputs(p, u, pu, L);
         const int incl = warp_inclusive_scan(deg);
         const int total = __shfl_sync(kFull, incl, 31);
         const int excl = incl - deg;
@@ -1657,12 +1778,17 @@ __device__ void clu_expand(const SingleParams& p, int L, int C, int r, int b, lo
                 v[q4] = act[q4] ? __ldg(p.cols + sj + (k - exj)) : 0;
                 act[q4] = act[q4] && v[q4] != pj;
             }
-            bool cl[4];
+            // (issued together and tested after: a test right behind its atomic would
+            // make each wait for the one before)
+            unsigned old[4];
 #pragma unroll
             for (int q4 = 0; q4 < 4; q4++) {
-                const unsigned bit = 1u << (v[q4] & 31);
-                cl[q4] = act[q4] && !(atomicOr(p.visited + (v[q4] >> 5), bit) & bit);
+                old[q4] = kFull;
+                if (act[q4]) old[q4] = atomicOr(p.visited + (v[q4] >> 5), 1u << (v[q4] & 31));
             }
+            bool cl[4];
+#pragma unroll
+            for (int q4 = 0; q4 < 4; q4++) cl[q4] = !((old[q4] >> (v[q4] & 31)) & 1u);
             long long rs[4], re[4];
 #pragma unroll
             for (int q4 = 0; q4 < 4; q4++) {
@@ -1670,19 +1796,17 @@ __device__ void clu_expand(const SingleParams& p, int L, int C, int r, int b, lo
                 re[q4] = 0;
                 if (cl[q4]) row_of(p, v[q4], rs[q4], re[q4]);
             }
-            const int mine = (int)cl[0] + (int)cl[1] + (int)cl[2] + (int)cl[3];
-            const int inc2 = warp_inclusive_scan(mine);
+            const int ncl = (int)cl[0] + (int)cl[1] + (int)cl[2] + (int)cl[3];
+            const int inc2 = warp_inclusive_scan(ncl);
             const int tot2 = __shfl_sync(kFull, inc2, 31);
             if (tot2 == 0) continue;
             int pos = 0;
             if (lane == 0) pos = atomicAdd(s_lcnt, tot2);
-            pos = __shfl_sync(kFull, pos, 0) + inc2 - mine;
+            pos = __shfl_sync(kFull, pos, 0) + inc2 - ncl;
 #pragma unroll
             for (int q4 = 0; q4 < 4; q4++) {
                 if (!cl[q4]) continue;
                 const int vv = v[q4];
-                if (p.parent) p.parent[vv] = uu[q4];
-                set_level(p, vv, L + 1);
                 const long long dg = re[q4] - rs[q4];
                 acc_m += (unsigned long long)dg;
                 acc_h |= dg > (long long)p.clu_big;
@@ -1696,6 +1820,7 @@ __device__ void clu_expand(const SingleParams& p, int L, int C, int r, int b, lo
                 } else {
                     const unsigned long long sp = atomicAdd(&p.ctrl->clu_spill, 1ull);
                     p.queue0[sp] = vv;
+                    clu_outputs(p, vv, uu[q4], L + 1);
                 }
                 pos++;
             }
@@ -1712,7 +1837,8 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
                                long long mu0, long long reached0, unsigned long long epi, uint64_t t_start,
                                CluState& out) {
     __shared__ int s_lcnt, s_lh;
-    __shared__ unsigned long long s_lm;
+    __shared__ unsigned s_lm;                // degree sum of the CTA's claims,
+    __shared__ unsigned long long s_lbig;    // ... and of the warps that met a large degree
     Ctrl* c = p.ctrl;
     const int C = p.clu_c, r = (int)clu_rank(), tid = threadIdx.x, nth = blockDim.x;
     const int lane = lane_id(), wib = tid >> 5;
@@ -1741,37 +1867,49 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
             s_lcnt = 0;
             s_lh = 0;
             s_lm = 0;
+            s_lbig = 0;
         }
     }
     clu_sync();
     int L = d0, b = 0;
-    long long mu = mu0, reached = reached0, pnf = 0, pmf = 0;
+    long long mu = mu0, reached = reached0;
+    // the record of the level before, written while the CTAs wait for one another
+    // (the lead thread's clock and stores would otherwise hold up every level)
+    long long pnf = 0, pmf = 0, pnext = 0, pmnext = 0;
+    uint64_t t_end = 0;
+    auto record = [&](int level) {
+        if (!lead || level < d0 || level >= p.rec_cap) return;
+        bfs_level_record rec;
+        rec.dir = TD;
+        rec.misses = 0;
+        rec.nf = pnf;
+        rec.mf = pmf;
+        rec.nnext = pnext;
+        rec.mnext = pmnext;
+        rec.scanned = 0;
+        rec.examined = pmf;
+        rec.t_ns = (long long)(t_end - t_start);
+        rec.aux = -1;   // a cluster level
+        rec.t_mid_ns = 0;
+        p.rec[level] = rec;
+    };
     while (true) {
-        long long nf = 0, mf = 0, spill = 0;
-        bool heavy = false;
-        for (int q = 0; q < C; q++) {
-            const unsigned long long w0 = g_csum[b][q][0];
-            nf += (long long)(w0 & kCluCntMask) + (long long)(w0 >> 32);
-            spill += (long long)(w0 >> 32);
-            heavy |= ((w0 >> 15) & 1ull) != 0;
-            mf += (long long)g_csum[b][q][1];
+        // the CTAs' summaries, a lane each
+        const unsigned long long w0 = lane < C ? g_csum[b][lane][0] : 0ull, w1 = lane < C ? g_csum[b][lane][1] : 0ull;
+        const int mine = (int)(w0 & kCluCntMask);
+        // entries (at most 2^14 in all) and, above them, CTAs with a heavy vertex
+        const unsigned ch = __reduce_add_sync(kFull, (unsigned)(w0 & 0xFFFFull));
+        const bool heavy = (ch >> 15) != 0;
+        long long nf = (long long)(ch & (unsigned)kCluCntMask), spill = 0, mf;
+        if (__any_sync(kFull, (w0 >> 32) != 0)) {
+            spill = (long long)__reduce_add_sync(kFull, (unsigned)(w0 >> 32));
+            nf += spill;
         }
+        if (!__any_sync(kFull, (w1 >> 24) != 0)) mf = (long long)__reduce_add_sync(kFull, (unsigned)w1);
+        else mf = (long long)warp_sum(w1);
         if (L > d0) {
-            if (lead && L - 1 < p.rec_cap) {
-                bfs_level_record rec;
-                rec.dir = TD;
-                rec.misses = 0;
-                rec.nf = pnf;
-                rec.mf = pmf;
-                rec.nnext = nf;
-                rec.mnext = mf;
-                rec.scanned = 0;
-                rec.examined = pmf;
-                rec.t_ns = (long long)(globaltimer_ns() - t_start);
-                rec.aux = -1;   // a cluster level
-                rec.t_mid_ns = 0;
-                p.rec[L - 1] = rec;
-            }
+            pnext = nf;
+            pmnext = mf;
             if (nf > 0) {
                 reached += nf;
                 mu -= mf;
@@ -1781,13 +1919,17 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
         const bool leave = done || spill > 0 || heavy || nf > p.clu_nf || mf > p.clu_mf ||
                            decide_dir(p, TD, nf, mf, mu, L) != TD;
         if (leave) {
+            record(L - 1);
             if (!done) {
                 // the frontier back to queue0: spilled entries first, then CTA by CTA
                 long long pre = spill;
                 for (int q = 0; q < r; q++) pre += (long long)(g_csum[b][q][0] & kCluCntMask);
-                const int mine = (int)(g_csum[b][r][0] & kCluCntMask);
+                const int mine = (int)(g_csum[b][r][0] & kCluCntMask);   // (this CTA's)
                 const CluEntry* cur = b ? buf1 : buf0;
-                for (int i = tid; i < mine; i += nth) p.queue0[pre + i] = cur[i].v;
+                for (int i = tid; i < mine; i += nth) {
+                    p.queue0[pre + i] = cur[i].v;
+                    clu_outputs(p, cur[i].v, cur[i].par, L);
+                }
             }
             out.d = done ? L - 1 : L;
             out.nf = nf;
@@ -1816,17 +1958,29 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
                                : "memory");
         unsigned long long am = 0;
         unsigned ah = 0;
-        clu_expand(p, L, C, r, b, nf, b ? buf1 : buf0, b ? buf0 : buf1, &s_lcnt, am, ah);
-        am = warp_sum(am);
-        const bool hw = __any_sync(kFull, ah != 0);
-        if (lane == 0) {
-            if (am) atomicAdd(&s_lm, am);
-            if (hw) s_lh = 1;
+        if (p.clu_d == 4)
+            clu_expand_short<4>(p, L, C, r, mine, (int)nf, b ? buf1 : buf0, b ? buf0 : buf1, &s_lcnt, am, ah);
+        else if (p.clu_d == 8)
+            clu_expand_short<8>(p, L, C, r, mine, (int)nf, b ? buf1 : buf0, b ? buf0 : buf1, &s_lcnt, am, ah);
+        else
+            clu_expand(p, L, C, r, mine, nf, b ? buf1 : buf0, b ? buf0 : buf1, &s_lcnt, am, ah);
+        if (__any_sync(kFull, am != 0)) {
+            const bool hw = __any_sync(kFull, ah != 0);
+            if (!__any_sync(kFull, (am >> 20) != 0)) {
+                const unsigned sum = __reduce_add_sync(kFull, (unsigned)am);   // under 2^25, a CTA's under 2^29
+                if (lane == 0) atomicAdd(&s_lm, sum);
+            } else {
+                am = warp_sum(am);
+                if (lane == 0) atomicAdd(&s_lbig, am);
+            }
+            if (lane == 0) {
+                if (hw) s_lh = 1;
+            }
         }
         __syncthreads();
         if (wib == 0) {
             const int lc = s_lcnt;
-            const unsigned long long lm = s_lm;
+            const unsigned long long lm = (unsigned long long)s_lm + s_lbig;
             const int lh = s_lh;
             const int cnt = lc < kCluCap ? lc : kCluCap;
             const unsigned long long w0 = (unsigned long long)cnt | ((unsigned long long)(lh ? 1 : 0) << 15) |
@@ -1840,11 +1994,15 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
                 s_lcnt = 0;
                 s_lh = 0;
                 s_lm = 0;
+                s_lbig = 0;
             }
         }
-        clu_sync();
+        clu_arrive();
+        record(L - 1);
         pnf = nf;
         pmf = mf;
+        if (lead) t_end = globaltimer_ns();
+        clu_await();
         L++;
         b ^= 1;
     }
@@ -2869,6 +3027,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     hub_regions(p);
     p.clu_c = 1;
     p.clu_big = 0;
+    p.clu_d = 0;
     p.clu_nf = 0;
     p.clu_mf = 0;
     p.seed = opt.seed;
@@ -2950,6 +3109,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     if (C > 1) {
         p.clu_c = C;
         p.clu_big = bfsk::kCluBig;
+        p.clu_d = g->max_degree <= 4 ? 4 : g->max_degree <= 8 ? 8 : 0;
         p.clu_nf = (long long)C * (bfsk::kCluCap / 2);
         p.clu_mf = (long long)C * bfsk::kCluEdgesPerCta;
     }
@@ -3103,6 +3263,7 @@ extern "C" bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int3
     hub_regions(p);
     p.clu_c = 1;
     p.clu_big = 0;
+    p.clu_d = 0;
     p.clu_nf = 0;
     p.clu_mf = 0;
     p.timeout_ns = 10000ull * 1000000ull;

@@ -236,3 +236,58 @@ def test_dcsc_streams_and_long_columns(gpu_lib, shape, min_id):
             assert oracle.certify(ref, root, want, pa, labels) == (0, -1), (root, mode)
             assert not min_id or np.array_equal(pa, oracle.min_parent(ref, want)), (root, mode)
     g.close()
+
+
+def _mesh(w, h, diag, seed):
+    """A w x h grid without wrap-around (degree <= 4; <= 8 with `diag`), ids shuffled."""
+    ids = np.random.default_rng(seed).permutation(w * h).astype(np.int32).reshape(h, w)
+    pairs = [(ids[:, :-1], ids[:, 1:]), (ids[:-1], ids[1:])]
+    if diag:
+        pairs += [(ids[:-1, :-1], ids[1:, 1:]), (ids[:-1, 1:], ids[1:, :-1])]
+    return graphgen.EdgeList(w * h, np.concatenate([a.ravel() for a, _ in pairs]),
+                             np.concatenate([b.ravel() for _, b in pairs]))
+
+
+@pytest.mark.parametrize("shape", ["mesh4", "mesh8", "narrow", "tree", "path"])
+@pytest.mark.parametrize("min_id", [False, True])
+def test_cluster_levels_of_short_rows(gpu_lib, shape, min_id):
+    """Cluster levels with 4 and 8 lanes per entry and past them: frontiers from one vertex to
+    more than a CTA's even share, uneven shares, frontiers that outgrow the cluster (a
+    binary tree doubles to the grid's), depths past the byte staging, several roots."""
+    bfs = gpu_lib
+    rng = np.random.default_rng(4)
+    if shape == "tree":
+        n = (1 << 15) - 1
+        ids = rng.permutation(n).astype(np.int32)
+        e = graphgen.EdgeList(n, ids[(np.arange(1, n) - 1) // 2], ids[1:])
+    else:
+        e = {"mesh4": lambda: _mesh(300, 210, False, 1), "mesh8": lambda: _mesh(180, 190, True, 2),
+             "narrow": lambda: _mesh(3, 900, True, 3), "path": lambda: graphgen.path(600)}[shape]()
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+    level, parent = _buffers(e.n)
+    pm = bfs.PARENT_MIN_ID if min_id else bfs.PARENT_ANY
+    for root in graphgen.pick_roots(e, 3, 6).tolist():
+        want = oracle.levels(ref, root)
+        for mode, omode in ((bfs.MODE_DO, oracle.MODE_DO), (bfs.MODE_TD_ONLY, oracle.MODE_TD)):
+            for c in (0, 2, 8):
+                parent.fill_(-7)
+                info = g.run(root, parent=parent, level=level, stats=True, record_levels=2048,
+                             opts=bfs.options(mode=mode, parent_mode=pm, cluster_size=c))
+                pa = parent.cpu().numpy()
+                assert np.array_equal(level.cpu().numpy(), want), (root, mode, c)
+                assert oracle.certify(ref, root, want, pa, labels) == (0, -1), (root, mode, c)
+                assert not min_id or np.array_equal(pa, oracle.min_parent(ref, want)), (root, mode, c)
+                s = oracle.do_schedule(ref, want, omode)
+                for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext", "scanned", "examined"]):
+                    assert np.array_equal(info["records"][:, col], getattr(s, name)), (root, mode, c, name)
+                assert (np.diff(info["records"][:, 7]) >= 0).all()
+    roots = np.unique(graphgen.pick_roots(e, 40, 7))
+    g.run_multiroot(roots, parent=parent, level=level, opts=bfs.options(parent_mode=pm))
+    lv, pa = level.cpu().numpy(), parent.cpu().numpy()
+    want = np.min(np.stack([np.where(x < 0, 1 << 30, x) for x in (oracle.levels(ref, int(r)) for r in roots)]), axis=0)
+    assert np.array_equal(lv, np.where(want == 1 << 30, -1, want))
+    v = np.flatnonzero(lv > 0)
+    assert np.array_equal(lv[pa[v]], lv[v] - 1) and np.array_equal(pa[roots], roots)
+    g.close()
