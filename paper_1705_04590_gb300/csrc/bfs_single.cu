@@ -47,6 +47,7 @@ namespace bfsk {
 #define BFS_BLOCK 512
 #endif
 constexpr int kBlock = BFS_BLOCK;  // CSR kernel
+constexpr long long kSmallN = 1LL << 18;   // graphs up to this size launch one CTA per SM
 constexpr int kDBlock = 1024;   // DCSC kernel (one CTA per vertex block)
 constexpr int kWarps = 32;      // shared-memory per-warp arrays sized for up to 1024 threads
 constexpr int kChunk = 256;    // td_chunk of the allocation-free entry point
@@ -503,22 +504,19 @@ __device__ __forceinline__ void flush_degree(const SingleParams& p, int v, bool 
     if (pf && re > rs) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.cols + rs));
 }
 
-// Write st.buf[0..cnt) to qnext[base..] and add their degrees (the next
-// frontier's m_f, read here in batches rather than on the claim path) to acc_m:
-// a lane takes up to kFlushBatch entries per step and has all their degree bytes
-// in flight together (one by one they would be a chain of dependent DRAM reads).
+// The degrees of st.buf[0..cnt) (the next frontier's m_f, read here in batches
+// rather than on the claim path) into acc_m: a lane takes up to kFlushBatch
+// entries per step and has all their degree bytes in flight together (one by one
+// they would be a chain of dependent DRAM reads).  kDir (a directed graph): acc_m
+// collects out-degrees, st.din in-degrees (what m_u loses).
 constexpr int kFlushBatch = 8;
 
-// kDir (a directed graph): acc_m collects out-degrees (the next frontier's m_f),
-// st.din in-degrees (what m_u loses).
 template <bool kDir>
-__device__ __forceinline__ void flush_entries(const SingleParams& p, WarpStage& st, int* qnext,
-                                              unsigned long long base, unsigned long long& acc_m) {
+__device__ __forceinline__ void flush_degrees(const SingleParams& p, WarpStage& st, unsigned long long& acc_m) {
     const int lane = lane_id();
     if (!p.deg8 || st.pf) {
         for (int i = lane; i < st.cnt; i += 32) {
             const int v = st.buf[i];
-            qnext[base + i] = v;
             flush_degree(p, v, st.pf, acc_m, st.hv);
             if constexpr (kDir) st.din += (unsigned long long)in_degree(p, v);
         }
@@ -536,13 +534,19 @@ __device__ __forceinline__ void flush_entries(const SingleParams& p, WarpStage& 
 #pragma unroll
         for (int k = 0; k < kFlushBatch; k++) {
             if (vs[k] < 0) continue;
-            qnext[base + i0 + k * 32 + lane] = vs[k];
             const long long dg = d8[k] < 255u ? (long long)d8[k] : deg_of(p, vs[k]);
             acc_m += (unsigned long long)dg;
             st.hv += dg > (long long)p.clu_big;
             if constexpr (kDir) st.din += (unsigned long long)in_degree(p, vs[k]);
         }
     }
+}
+
+// st.buf[0..cnt) to qnext[base..]; the staging is empty after it
+__device__ __forceinline__ void flush_store(WarpStage& st, int* qnext, unsigned long long base) {
+    for (int i = lane_id(); i < st.cnt; i += 32) qnext[base + i] = st.buf[i];
+    __syncwarp();
+    st.cnt = 0;
 }
 
 template <bool kDir>
@@ -552,16 +556,16 @@ __device__ __forceinline__ void stage_flush(const SingleParams& p, WarpStage& st
     __syncwarp();
     unsigned long long base = 0;
     if (lane_id() == 0) base = atomicAdd(tail, (unsigned long long)st.cnt);
-    base = __shfl_sync(kFull, base, 0);
-    flush_entries<kDir>(p, st, qnext, base, acc_m);
-    __syncwarp();
-    st.cnt = 0;
+    flush_degrees<kDir>(p, st, acc_m);   // while the atomic is under way
+    flush_store(st, qnext, __shfl_sync(kFull, base, 0));
 }
 
 // End of a top-down phase: every warp's remaining staged entries are appended
 // with one atomicAdd per CTA (a block scan of the warps' counts).  On small
 // levels most warps hold a few entries each, and one queue-tail atomic per
-// warp would serialise thousands of arrivals on one word.  All threads call.
+// warp would serialise thousands of arrivals on one word.  The entries' degrees
+// are read while that atomic is under way (0.6 us each, one behind the other
+// otherwise).  All threads call.
 template <bool kDir>
 __device__ void block_flush(const SingleParams& p, WarpStage& st, int* qnext, unsigned long long* tail,
                             unsigned long long& acc_m) {
@@ -577,13 +581,13 @@ __device__ void block_flush(const SingleParams& p, WarpStage& st, int* qnext, un
         unsigned long long b = 0;
         if (lane == 0 && total) b = atomicAdd(tail, (unsigned long long)total);
         if (lane < nwb) s_wcnt[lane] = incl - c;
+        flush_degrees<kDir>(p, st, acc_m);
         if (lane == 0) s_bbase = b;
+    } else {
+        flush_degrees<kDir>(p, st, acc_m);
     }
     __syncthreads();
-    const unsigned long long base = s_bbase + (unsigned long long)s_wcnt[wib];
-    flush_entries<kDir>(p, st, qnext, base, acc_m);
-    __syncwarp();
-    st.cnt = 0;
+    flush_store(st, qnext, s_bbase + (unsigned long long)s_wcnt[wib]);
 }
 
 // Record the claims of one warp step: winners write parent/level and stage v.
@@ -3046,6 +3050,14 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     int grid = w.grid, block = w.block;
     if (opt.ctas_per_sm > 0 && (long long)opt.ctas_per_sm * g->sm_count < grid) {
         grid = opt.ctas_per_sm * g->sm_count;
+        p.expected = (unsigned)grid + extra;
+    }
+    // a small graph's levels are the chain of their reads and barriers, not work to
+    // spread: one CTA per SM halves the arrivals of a barrier (R-MAT 12: 50.6 us with
+    // 304 CTAs, 47.8 with 152, 49.2 with 8; R-MAT 18: 81.0, 77.6 and 161; R-MAT 20 is
+    // even at 107 / 108)
+    if (g->n <= bfsk::kSmallN && grid > g->sm_count) {
+        grid = g->sm_count;
         p.expected = (unsigned)grid + extra;
     }
     size_t dyn = bfsk::kSingleDynSmem;
