@@ -590,8 +590,14 @@ __device__ void block_flush(const SingleParams& p, WarpStage& st, int* qnext, un
     flush_store(st, qnext, s_bbase + (unsigned long long)s_wcnt[wib]);
 }
 
-// Record the claims of one warp step: winners write parent/level and stage v.
-template <bool kDir>
+// Record the claims of one warp step: winners write their parent and stage v.
+// The level waits for the next step (a top-down level that reads v from the queue,
+// or the bottom-up sweep that comes past it: mark_chunk) unless kNow: the level bytes, the
+// parents and the degree bytes of a large level's claims together overflow L2, and
+// every scattered store is then a DRAM access (Erdos-Renyi, 40 M vertices, 11.4 M
+// claims: 754 us with both stores, 412 without the level's, 295 without the
+// parent's).
+template <bool kDir, bool kNow>
 __device__ __forceinline__ void td_stage(const SingleParams& p, int d, int u, int v, bool claimed, WarpStage& st,
                                          int* qnext, unsigned long long* tail, unsigned long long& acc_m) {
     const unsigned cm = __ballot_sync(kFull, claimed);
@@ -599,7 +605,7 @@ __device__ __forceinline__ void td_stage(const SingleParams& p, int d, int u, in
         if (claimed) {
             st.buf[st.cnt + __popc(cm & lanemask_lt())] = v;
             if (p.parent) p.parent[v] = u;
-            set_level(p, v, d + 1);
+            if constexpr (kNow) set_level(p, v, d + 1);
         }
         st.cnt += __popc(cm);
         if (st.cnt > kStage - 32) stage_flush<kDir>(p, st, qnext, tail, acc_m);
@@ -609,7 +615,7 @@ __device__ __forceinline__ void td_stage(const SingleParams& p, int d, int u, in
 // Visit edge (u, v) for the whole warp (every lane calls; `act` masks): claim
 // v with an atomicOr on the visited bitmap; the winner records parent/level
 // and stages v for the next queue.
-template <bool kDir>
+template <bool kDir, bool kNow>
 __device__ __forceinline__ void td_visit(const SingleParams& p, int d, int u, int v, bool act, WarpStage& st,
                                          int* qnext, unsigned long long* tail, unsigned long long& acc_m) {
     bool claimed = false;
@@ -625,7 +631,7 @@ __device__ __forceinline__ void td_visit(const SingleParams& p, int d, int u, in
         claimed = !(atomicOr(wp, bit) & bit);
 #endif
     }
-    td_stage<kDir>(p, d, u, v, claimed, st, qnext, tail, acc_m);
+    td_stage<kDir, kNow>(p, d, u, v, claimed, st, qnext, tail, acc_m);
 }
 
 __device__ __forceinline__ WarpStage warp_stage_in(int* buf) {
@@ -711,9 +717,9 @@ __device__ __forceinline__ void hub_slice(const SingleParams& p, const LevelCtr&
     u = raw.w;
 }
 
-template <bool kDir>
+template <bool kDir, bool kNow>
 __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long long nf, int* qnext, int snext,
-                         unsigned long long& acc_m, unsigned long long& acc_h, unsigned long long& acc_in) {
+                         bool mark, unsigned long long& acc_m, unsigned long long& acc_h, unsigned long long& acc_in) {
     const int lane = lane_id();
     const long long gw = spread_warp(), nw = gthreads() >> 5;
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
@@ -729,6 +735,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
         if (lane < per && i < nf) {
             u = __ldcg(qcur + i);
             row_of(p, u, s, e);
+            if (mark) set_level(p, u, d);   // a top-down level found it
         }
         const long long deg = e - s;
         const bool big = deg > p.big_deg;
@@ -770,7 +777,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
             const int uj = __shfl_sync(kFull, u, j);
             const bool act = k < total;
             const int v = act ? __ldg(p.cols + sj + (k - exj)) : 0;
-            td_visit<kDir>(p, d, uj, v, act, st, qnext, tail, acc_m);
+            td_visit<kDir, kNow>(p, d, uj, v, act, st, qnext, tail, acc_m);
         }
     }
     block_flush<kDir>(p, st, qnext, tail, acc_m);
@@ -778,7 +785,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
     acc_in += st.din;
 }
 
-template <bool kDir>
+template <bool kDir, bool kNow>
 __device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int* qnext, int snext,
                           unsigned long long& acc_m, unsigned long long& acc_h, unsigned long long& acc_in) {
     const int lane = lane_id();
@@ -822,7 +829,7 @@ __device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int
 #pragma unroll
             for (int q = 0; q < 4; q++) claimed[q] = act[q] && !(seen[q] & (1u << (v[q] & 31)));
 #pragma unroll
-            for (int q = 0; q < 4; q++) td_stage<kDir>(p, d, u, v[q], claimed[q], st, qnext, tail, acc_m);
+            for (int q = 0; q < 4; q++) td_stage<kDir, kNow>(p, d, u, v[q], claimed[q], st, qnext, tail, acc_m);
         }
     }
     block_flush<kDir>(p, st, qnext, tail, acc_m);
@@ -938,11 +945,13 @@ __device__ void min_parent_rows(const SingleParams& p, const unsigned* lv) {
 
 // ------------------------------------------------------------------ conversions
 
-__device__ void queue_to_bitmap(const SingleParams& p, const int* q, long long nf, unsigned* f) {
+// (mark: the level that filled the queue left its vertices' levels, d, to this step)
+__device__ void queue_to_bitmap(const SingleParams& p, const int* q, long long nf, unsigned* f, int d, bool mark) {
     const long long tid = gtid(), nth = gthreads();
     for (long long i = tid; i < nf; i += nth) {
         const int v = __ldcg(q + i);
         atomicOr(f + (v >> 5), 1u << (v & 31));
+        if (mark) set_level(p, v, d);
     }
 }
 
@@ -1297,7 +1306,31 @@ __device__ __forceinline__ void chunk_misses(const SingleParams& p, int d, const
     st.cnt = 0;
 }
 
-__device__ void bu_compact(const SingleParams& p, int d, const unsigned* fcur, unsigned* fnext, int* misslist,
+// The sweep after a large top-down level writes the levels that it left: those of
+// the chunk's frontier vertices (this lane's word of the frontier in `fw`), listed
+// so that a store covers neighbouring vertices.  In the queue's order, with the
+// conversion to a bitmap, 10.7 M of them took 90 us (R-MAT 26; here 11), but the
+// sweep reads every word for it: 10 us a search of R-MAT 24 whose 43 K are written
+// with the conversion in one.
+constexpr long long kMarkSweep = 64;   // from n / this many vertices on
+__device__ __forceinline__ void mark_chunk(const SingleParams& p, int d, unsigned fw, unsigned short* list,
+                                           long long wbase) {
+    const int lane = lane_id();
+    const int cnt = __popc(fw);
+    const int incl = warp_inclusive_scan(cnt);
+    const int T = __shfl_sync(kFull, incl, 31);
+    if (T == 0) return;
+    int at = incl - cnt;
+    while (fw) {
+        list[at++] = (unsigned short)(lane * 32 + __ffs(fw) - 1);
+        fw &= fw - 1;
+    }
+    __syncwarp();
+    for (int k = lane; k < T; k += 32) set_level(p, (int)(wbase * 32 + list[k]), d);
+    __syncwarp();
+}
+
+__device__ void bu_compact(const SingleParams& p, int d, bool mark, const unsigned* fcur, unsigned* fnext, int* misslist,
                            unsigned long long* misscnt, unsigned long long* misscnt_inline, int* longlist,
                            unsigned long long* longcnt,
                            unsigned long long& acc_n, unsigned long long& acc_left, unsigned long long& acc_sc,
@@ -1317,6 +1350,7 @@ __device__ void bu_compact(const SingleParams& p, int d, const unsigned* fcur, u
         const long long w = wbase + lane;
         const bool own = lane < cwords && w < p.W;
         const unsigned cw = own ? __ldcg(p.visited + w) : kFull;
+        if (mark) mark_chunk(p, d, own ? __ldcg(fcur + w) : 0u, list, wbase);
         unsigned todo = ~cw;
         const int cnt = __popc(todo);
         const int incl = warp_inclusive_scan(cnt);
@@ -1856,6 +1890,7 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
             const int u = __ldcg(qcur + i);
             long long rs, re;
             row_of(p, u, rs, re);
+            set_level(p, u, d0);   // the grid's claim left it
             CluEntry e;
             e.row = clu_row(rs, re - rs);
             e.v = u;
@@ -2123,6 +2158,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
     }
     // cluster levels only in a launch whose clusters have the size the parameters name
     const bool clu_on = kClu && p.clu_c > 1 && clu_nranks() == (unsigned)p.clu_c;
+    constexpr bool kNow = kMinId;   // the offers after a level look for its level bytes
     while (true) {
         __syncthreads();   // S is settled
         const int dir = decide_dir(p, S.prev, S.nf, S.mf, S.mu, S.d);
@@ -2170,8 +2206,8 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             }
             {
                 unsigned long long am = 0, ah = 0, ai = 0;
-                td_phase<kDir>(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, S.qsel ? p.queue0 : p.queue1, snext, am, ah,
-                               ai);
+                td_phase<kDir, kNow>(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, S.qsel ? p.queue0 : p.queue1, snext,
+                                     !kNow && S.prev == TD && S.d > 0, am, ah, ai);
                 block_add4(ah, am, ai, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm,
                            &c->lv[snext].dsum_in, nullptr);
             }
@@ -2179,7 +2215,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             if (lead) S.t_mid = globaltimer_ns();
             if (hub_slices(s_ctr) > 0) {
                 unsigned long long am = 0, ah = 0, ai = 0;
-                hub_phase<kDir>(p, S.d, s_ctr, S.qsel ? p.queue0 : p.queue1, snext, am, ah, ai);
+                hub_phase<kDir, kNow>(p, S.d, s_ctr, S.qsel ? p.queue0 : p.queue1, snext, am, ah, ai);
                 block_add4(ah, am, ai, 0, clu_on ? &c->lv[snext].heavy : nullptr, &c->lv[snext].accm,
                            &c->lv[snext].dsum_in, nullptr);
                 if (!level_sync(p, snext, s_ctr)) return;
@@ -2192,8 +2228,14 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 }
             }
         } else {
+            // levels that a top-down level left: a large frontier's in the sweep over the
+            // hub-first rows, others with the conversion (in the id-ordered rows' sweep it
+            // costs that loop registers: R-MAT 24 1734 -> 1852 us)
+            const bool left = !kNow && S.prev == TD && S.d > 0;
+            const bool in_sweep = kHub && S.nf * kMarkSweep >= p.n;
             if (S.prev == TD) {
-                queue_to_bitmap(p, S.qsel ? p.queue1 : p.queue0, S.nf, S.bsel ? p.front1 : p.front0);
+                queue_to_bitmap(p, S.qsel ? p.queue1 : p.queue0, S.nf, S.bsel ? p.front1 : p.front0, S.d,
+                                left && !in_sweep);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             // over the hub-first rows accm collects the degrees of the searchers left
@@ -2204,7 +2246,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             {
                 unsigned long long an = 0, am = 0, asc = 0, aex = 0, ao = 0;
                 if constexpr (kHub)
-                    bu_compact(p, S.d, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
+                    bu_compact(p, S.d, left && in_sweep, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
                                S.qsel ? p.queue1 : p.queue0, &c->lv[snext].nmiss, &c->lv[snext].nmiss_in,
                                S.qsel ? p.queue0 : p.queue1, &c->lv[snext].ntask, an, am, asc, aex);
                 else
@@ -2752,7 +2794,7 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
                 const long long nbw = block_words(p, blockIdx.x), wbase = (long long)blockIdx.x * p.Bw;
                 for (long long w = threadIdx.x; w < nbw; w += blockDim.x) f[wbase + w] = 0u;
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-                queue_to_bitmap(p, qcur, nf, f);
+                queue_to_bitmap(p, qcur, nf, f, d, false);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
                 td_dcsc_stream(p, d, f, qnext, snext, s_own, s_seg, s_urow, am);
             } else {
@@ -2764,7 +2806,7 @@ __global__ void __launch_bounds__(kDBlock, 1) bfs_dcsc_kernel(SingleParams p) {
             qsel ^= 1;
         } else {
             if (prev == TD) {
-                queue_to_bitmap(p, qcur, nf, fcur);
+                queue_to_bitmap(p, qcur, nf, fcur, d, false);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             unsigned long long an = 0, am = 0, asc = 0, aex = 0;
