@@ -38,8 +38,8 @@ namespace bfsk {
 constexpr int kMBlock = 512;
 constexpr int kMChunk = 512;      // edges per top-down chunk task
 constexpr int kMBigDeg = 256;     // rows above this become chunk tasks (the task lists are sized for it)
-constexpr int kPullChunk = 1024;  // ids per chunk task of a long row (pulls, parents)
-constexpr int kPullSteps = 16;    // 16-id steps a 4-lane group pulls before the rest of the row becomes tasks
+constexpr int kPullChunk = 512;   // ids per chunk task of a long row (pulls, parents)
+constexpr int kPullSteps = 4;     // 16-id steps a 4-lane group pulls before the rest of the row becomes tasks
 constexpr int kPlaneMax = 15;     // largest level + 1 that the four planes hold
 constexpr unsigned kMFull = 0xffffffffu;
 
@@ -138,16 +138,21 @@ __device__ __forceinline__ void m_append(MStage& st, int* q, unsigned long long*
     }
 }
 
-// Push lane bits along edge (v -> u); record u the first time its next mask
+// Push the lane bits nb[q] to u[q] (-1: none), four edges per lane: the seen masks
+// in flight together, then the atomics; u is recorded the first time its next mask
 // becomes nonzero.  All lanes call.
-__device__ __forceinline__ void ms_push(const MultiParams& p, unsigned long long f, int u, bool act, MStage& st,
-                                        int* tq, unsigned long long* tlen) {
-    bool first = false;
-    if (act) {
-        const unsigned long long nb = f & ~ldcg64(p.seen + u);
-        if (nb) first = atomicOr(p.next + u, nb) == 0ull;
+__device__ __forceinline__ void ms_push4(const MultiParams& p, unsigned long long (&nb)[4], const int (&u)[4],
+                                         MStage& st, int* tq, unsigned long long* tlen) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) nb[q] = u[q] >= 0 ? nb[q] & ~ldcg64(p.seen + u[q]) : 0ull;
+    unsigned long long old[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        old[q] = 1ull;
+        if (nb[q]) old[q] = atomicOr(p.next + u[q], nb[q]);
     }
-    m_append(st, tq, tlen, first, u);
+#pragma unroll
+    for (int q = 0; q < 4; q++) m_append(st, tq, tlen, old[q] == 0ull, u[q]);
 }
 
 // Top-down push over the frontier queue (warp-balanced gather; heavy rows
@@ -206,20 +211,25 @@ __device__ void ms_td_phase(const MultiParams& p, MCtrl* c, int slot, const int*
         const int incl = warp_inclusive_scan(mydeg);
         const int total = __shfl_sync(kMFull, incl, 31);
         const int excl = incl - mydeg;
-        for (int k0 = 0; k0 < total; k0 += 32) {
-            const int k = k0 + lane;
-            int j = 0;
+        // four edges per lane per step: the ids, the seen masks, the pushes
+        for (int k0 = 0; k0 < total; k0 += 128) {
+            int u[4];
+            unsigned long long nb[4];
 #pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const int cc = __shfl_sync(kMFull, incl, j + step - 1);
-                if (cc <= k) j += step;
+            for (int q = 0; q < 4; q++) {
+                const int k = k0 + q * 32 + lane;
+                int j = 0;
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1) {
+                    const int cc = __shfl_sync(kMFull, incl, j + step - 1);
+                    if (cc <= k) j += step;
+                }
+                const long long sj = __shfl_sync(kMFull, s, j);
+                const int exj = __shfl_sync(kMFull, excl, j);
+                nb[q] = __shfl_sync(kMFull, f, j);
+                u[q] = k < total ? __ldg(p.cols + sj + (k - exj)) : -1;
             }
-            const long long sj = __shfl_sync(kMFull, s, j);
-            const int exj = __shfl_sync(kMFull, excl, j);
-            const unsigned long long fj = __shfl_sync(kMFull, f, j);
-            const bool act = k < total;
-            const int u = act ? __ldg(p.cols + sj + (k - exj)) : 0;
-            ms_push(p, fj, u, act, st, tq, tlen);
+            ms_push4(p, nb, u, st, tq, tlen);
         }
     }
     m_block_flush(st, tq, tlen);
@@ -245,12 +255,8 @@ __device__ void ms_tasks_phase(const MultiParams& p, MCtrl* c, int slot, int* tq
                 u[q] = k < len ? __ldg(p.cols + start + k) : -1;
             }
 #pragma unroll
-            for (int q = 0; q < 4; q++) nb[q] = u[q] >= 0 ? f & ~ldcg64(p.seen + u[q]) : 0ull;
-            bool first[4];
-#pragma unroll
-            for (int q = 0; q < 4; q++) first[q] = nb[q] && atomicOr(p.next + u[q], nb[q]) == 0ull;
-#pragma unroll
-            for (int q = 0; q < 4; q++) m_append(st, tq, tlen, first[q], u[q]);
+            for (int q = 0; q < 4; q++) nb[q] = f;
+            ms_push4(p, nb, u, st, tq, tlen);
         }
     }
     m_block_flush(st, tq, tlen);
@@ -260,7 +266,9 @@ __device__ void ms_tasks_phase(const MultiParams& p, MCtrl* c, int slot, int* tq
 // frontier masks of its first 8 neighbours.  Rows with lanes still missing then
 // go on in groups of 4 lanes, 8 rows per warp at a time, 16 neighbours a step
 // until every missing lane is covered; a row that is not done after kPullSteps
-// steps becomes chunk tasks of kPullChunk ids for all warps (ms_bu_tasks_phase).
+// steps becomes chunk tasks of kPullChunk ids for all warps (ms_bu_tasks_phase):
+// few steps here, as a group's are a chain (with 16 steps the groups of the level
+// that reads most of R-MAT 22 took 469 us for 30 M ids, the tasks 276 for 100 M).
 // Bound by dependent reads (ids, then masks): one row at a time per warp left
 // two thirds of the cycles waiting at the level's barrier for the warps whose
 // vertices had long rows (R-MAT 20, 64 roots).
@@ -306,7 +314,32 @@ __device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned l
             const unsigned long long mL = __shfl_sync(kMFull, miss, L);
             unsigned long long aL = __shfl_sync(kMFull, acc, L);
             bool live = has;
-            for (int step = 0; step < kPullSteps && __any_sync(kMFull, live); step++) {
+            // (a row that finds the task list full goes on here)
+            for (int step = 0; __any_sync(kMFull, live); step++) {
+                if (step == kPullSteps) {
+                    if (live && gl == 0) {
+                        const long long nch = (qe - q + kPullChunk - 1) / kPullChunk;
+                        const unsigned long long t0 = atomicAdd(&c->ntask[slot], (unsigned long long)nch);
+                        if ((long long)t0 + nch <= p.task_cap) {
+                            for (long long k = 0; k < nch; k++) {
+                                MTask t;
+                                t.start = q + k * kPullChunk;
+                                t.len = (int)min((long long)kPullChunk, qe - t.start);
+                                t.v = (int)(base + L);
+                                p.tasks[t0 + k] = t;
+                            }
+                            live = false;
+                        } else {
+                            // what was reserved past the room left: tasks with nothing in them
+                            MTask t;
+                            t.start = 0;
+                            t.len = 0;
+                            t.v = (int)(base + L);
+                            for (long long k = (long long)t0; k < p.task_cap; k++) p.tasks[k] = t;
+                        }
+                    }
+                    live = __shfl_sync(kMFull, live, lane & ~3);
+                }
                 unsigned long long x = 0;
                 const long long q4 = q + 4 * gl;   // a multiple of 4: the window was aligned
                 if (live && q4 < qe) {
@@ -324,25 +357,7 @@ __device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned l
                     live = (aL & mL) != mL && q < qe;
                 }
             }
-            if (has && gl == 0) {
-                s_acc[wib][L] = aL;
-                if (live) {
-                    const long long nch = (qe - q + kPullChunk - 1) / kPullChunk;
-                    const unsigned long long t0 = atomicAdd(&c->ntask[slot], (unsigned long long)nch);
-                    for (long long k = 0; k < nch; k++) {
-                        const long long ti = (long long)t0 + k;
-                        if (ti >= p.task_cap) {
-                            raise_status(&c->b, kDevOverflow);
-                            break;
-                        }
-                        MTask t;
-                        t.start = q + k * kPullChunk;
-                        t.len = (int)min((long long)kPullChunk, qe - t.start);
-                        t.v = (int)(base + L);
-                        p.tasks[ti] = t;
-                    }
-                }
-            }
+            if (has && gl == 0) s_acc[wib][L] = aL;
         }
         __syncwarp();
         if (more) acc = s_acc[wib][lane];
@@ -423,64 +438,90 @@ __device__ void ms_apply_phase(const MultiParams& p, MCtrl* c, int slot, int ite
     if (tid == 0) c->accn[slot] = (unsigned long long)tlen;
 }
 
-// Apply after a bottom-up level, over all vertices (that level swept them all
-// anyway): the same updates as ms_apply_phase, old frontier bits dropped in
-// the same pass, and the new frontier listed in queue nq.
+// Apply over all vertices: after a bottom-up level (which swept them all anyway),
+// and after a top-down level that touched a large share of them: the same updates
+// as ms_apply_phase, old frontier bits dropped in the same pass, and the new
+// frontier listed in queue nq (null after a top-down level: the touched queue is
+// that list).  Four vertices per lane are in flight; read by read, one vertex at a
+// time, a nearly empty level took 95 us of latency at R-MAT 22.  Vertex by vertex in
+// the touched queue's order the masks, planes and offsets (112 bytes a vertex) are
+// random DRAM accesses: 918 K vertices of 4.2 M took 358 us.  In order, with few pull
+// steps and four pushes in flight, R-MAT 22 with 64 roots went from 1843 to 1576 us
+// (2217 to 2026 and 2274 to 2112 on other seeds).
+constexpr int kApplyAll = 16;   // touched vertices from n / this many on are applied in order
+
 __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int iter, unsigned long long active,
                                    const LaneSmem& L, bool direct, int* nq, unsigned long long* nlen) {
-    const long long tid = m_gtid(), nth = m_gthreads();
+    const int lane = lane_id();
+    const long long gw = m_gtid() >> 5, nw = m_gthreads() >> 5;
     MStage st = m_stage();
     unsigned long long an = 0, am = 0, adone = 0, found = 0;
-    for (long long base = tid - lane_id(); base < p.n; base += nth) {
-        const long long v = base + lane_id();
-        unsigned long long x = 0;
-        if (v < p.n) {
-            x = ldcg64(p.next + v);
-            if (x) {
-                p.next[v] = 0ull;
-                const unsigned long long s = ldcg64(p.seen + v);
-                p.seen[v] = s | x;
-                p.front[v] = x;
-                found |= x;
-                if (!direct) ms_set_planes(p, v, x, iter + 2);
-                const long long deg = __ldg(p.off + v + 1) - __ldg(p.off + v);
-                an += 1;
-                am += (unsigned long long)deg;
-                if ((s & active) != active && ((s | x) & active) == active) adone += (unsigned long long)deg;
-            } else if (ldcg64(p.front + v)) {
-                p.front[v] = 0ull;
+    for (long long base = gw * 128; base < p.n; base += nw * 128) {
+        unsigned long long x[4], f[4], s[4];
+        long long deg[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const long long v = base + k * 32 + lane;
+            x[k] = v < p.n ? ldcg64(p.next + v) : 0ull;
+            f[k] = v < p.n ? ldcg64(p.front + v) : 0ull;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const long long v = base + k * 32 + lane;
+            s[k] = 0;
+            deg[k] = 0;
+            if (x[k]) {
+                s[k] = ldcg64(p.seen + v);
+                deg[k] = __ldg(p.off + v + 1) - __ldg(p.off + v);
             }
         }
-        // level rows: the warp walks the lanes any of its 32 vertices gained, one
-        // lane at a time, so each store instruction writes consecutive vertices of
-        // one row (a lane-by-lane walk per thread would scatter every store)
-        unsigned long long ub = direct ? warp_or64(x) : 0ull;
-        while (ub) {
-            const int i2 = __ffsll((long long)ub) - 1;
-            ub &= ub - 1;
-            if ((x >> i2) & 1ull) L.rows[i2][v] = iter + 1 - L.start[i2];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const long long v = base + k * 32 + lane;
+            if (x[k]) {
+                p.next[v] = 0ull;
+                p.seen[v] = s[k] | x[k];
+                p.front[v] = x[k];
+                found |= x[k];
+                if (!direct) ms_set_planes(p, v, x[k], iter + 2);
+                an += 1;
+                am += (unsigned long long)deg[k];
+                if ((s[k] & active) != active && ((s[k] | x[k]) & active) == active) adone += (unsigned long long)deg[k];
+            } else if (f[k]) {
+                p.front[v] = 0ull;
+            }
+            // level rows written as it goes: the warp walks the lanes any of its 32
+            // vertices gained, one lane at a time, so each store instruction writes
+            // consecutive vertices of one row (a lane-by-lane walk per thread would
+            // scatter every store)
+            unsigned long long ub = direct ? warp_or64(x[k]) : 0ull;
+            while (ub) {
+                const int i2 = __ffsll((long long)ub) - 1;
+                ub &= ub - 1;
+                if ((x[k] >> i2) & 1ull) L.rows[i2][v] = iter + 1 - L.start[i2];
+            }
+            if (nq) m_append(st, nq, nlen, x[k] != 0ull, (int)v);
         }
-        m_append(st, nq, nlen, x != 0ull, (int)v);
     }
-    m_block_flush(st, nq, nlen);
+    if (nq) m_block_flush(st, nq, nlen);
     found = warp_or64(found);
-    if (lane_id() == 0 && found) atomicOr(&c->found[slot], found);
+    if (lane == 0 && found) atomicOr(&c->found[slot], found);
     block_add4(an, am, adone, 0, &c->accn[slot], &c->accm[slot], &c->mdone[slot], nullptr);
 }
 
 // Clear the three masks and both queue counters (grid-stride).
-__device__ void ms_clear_phase(const MultiParams& p) {
+__device__ void ms_clear_words(unsigned long long* a, long long cnt) {
     const long long tid = m_gtid(), nth = m_gthreads();
-    for (long long v = tid; v < p.n; v += nth) {
-        p.seen[v] = 0ull;
-        p.front[v] = 0ull;
-        p.next[v] = 0ull;
-        if (p.planes) {
-            const ulonglong2 z = make_ulonglong2(0ull, 0ull);
-            reinterpret_cast<ulonglong2*>(p.planes)[2 * v] = z;
-            reinterpret_cast<ulonglong2*>(p.planes)[2 * v + 1] = z;
-        }
-    }
+    const ulonglong2 z = make_ulonglong2(0ull, 0ull);
+    for (long long i = tid; i < cnt / 2; i += nth) reinterpret_cast<ulonglong2*>(a)[i] = z;
+    if ((cnt & 1) && tid == 0) a[cnt - 1] = 0ull;
+}
+
+__device__ void ms_clear_phase(const MultiParams& p) {
+    ms_clear_words(p.seen, p.n);
+    ms_clear_words(p.front, p.n);
+    ms_clear_words(p.next, p.n);
+    if (p.planes) ms_clear_words(p.planes, 4 * p.n);
 }
 
 // The level rows from the planes, every active lane's row whole: a warp takes
@@ -606,7 +647,11 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
                 ms_tasks_phase(p, c, slot, tq, tlen);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
-            ms_apply_phase(p, c, slot, it, active, L, direct, tq, (long long)ld_relaxed64(tlen));
+            const long long touched = (long long)ld_relaxed64(tlen);
+            if (touched * kApplyAll >= p.n)
+                ms_apply_all_phase(p, c, slot, it, active, L, direct, nullptr, nullptr);
+            else
+                ms_apply_phase(p, c, slot, it, active, L, direct, tq, touched);
         } else {
             ms_bu_phase(p, c, slot, active);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
@@ -865,7 +910,11 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_serve_kernel(MultiParams p, in
                 ms_tasks_phase(p, c, slot, tq, tlen);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
-            ms_apply_phase(p, c, slot, it, active, L, true, tq, (long long)ld_relaxed64(tlen));
+            const long long touched = (long long)ld_relaxed64(tlen);
+            if (touched * kApplyAll >= p.n)
+                ms_apply_all_phase(p, c, slot, it, active, L, true, nullptr, nullptr);
+            else
+                ms_apply_phase(p, c, slot, it, active, L, true, tq, touched);
         } else {
             ms_bu_phase(p, c, slot, active);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;

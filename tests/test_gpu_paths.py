@@ -55,7 +55,7 @@ def test_min_parents_of_top_down_levels(gpu_lib, shape, layout, cluster):
 
 
 @pytest.mark.parametrize("k", [1, 7, 64, 70])
-@pytest.mark.parametrize("shape", ["rmat", "star", "hubs", "path14", "path15", "path16", "comb", "er"])
+@pytest.mark.parametrize("shape", ["rmat", "star", "hubs", "path14", "path15", "path16", "comb", "er", "deg120"])
 def test_multi_rows_and_parents(gpu_lib, shape, k):
     """Batches whose levels end just inside and just past the level planes (depth 14 / 15),
     whose rows are longer than a group pulls before they become tasks, that do not fill
@@ -67,6 +67,8 @@ def test_multi_rows_and_parents(gpu_lib, shape, k):
          "hubs": lambda: graphgen.EdgeList(3002, np.repeat(np.array([17, 2900], np.int32), 3002),
                                            np.tile(rng.permutation(3002).astype(np.int32), 2)),
          "path14": lambda: graphgen.path(15), "path15": lambda: graphgen.path(16), "path16": lambda: graphgen.path(17),
+         # more rows past a group's steps than the list of chunk tasks holds
+         "deg120": lambda: graphgen.erdos_renyi(6000, 360_000, seed=7),
          "comb": lambda: _comb(40, 300), "er": lambda: graphgen.erdos_renyi(3333, 9000, seed=2)}[shape]()
     ref = oracle.build_csr(e.n, e.src, e.dst)
     g = bfs.Graph.from_edges(e.src, e.dst, e.n, hub_first=True)
