@@ -1485,6 +1485,11 @@ __device__ void bu_misses(const SingleParams& p, int d, const unsigned* fcur, un
     long_flush(lst, longlist, longcnt);
 }
 
+// 16-id steps of a 4-lane group before the whole warp takes what is left of the row,
+// 128 ids a step: a group with a long row otherwise keeps its warp's other seven
+// waiting (256 R-MAT graphs in one: 1.7 M long rows 446 us, 263 us so)
+constexpr int kLongSteps = 8;
+
 // Bottom-up, phase B: the long list.  Groups of 4 lanes take one searcher
 // each (8 per warp); a group reads 16 ids per step (one int4 per lane, in row
 // order) and stops at the first frontier neighbour: the lowest lane of the
@@ -1499,19 +1504,20 @@ __device__ void bu_phase_b(const SingleParams& p, int d, const unsigned* fcur, u
                            unsigned long long& acc_m, unsigned long long& acc_ex, unsigned long long& acc_out) {
     const int lane = lane_id(), grp = lane >> 2, gl = lane & 3;
     const long long gw = gtid() >> 5, nw = gthreads() >> 5;
+    int un = gw * 8 + grp < nlong ? __ldcg(longlist + gw * 8 + grp) : -1;   // the next round's row
     for (long long base = gw * 8; base < nlong; base += nw * 8) {
-        const long long i = base + grp;
-        int u = -1;
+        const int u = un;
         long long s0 = 0, e0 = 0, pos = 0;
-        if (i < nlong) {
-            u = __ldcg(longlist + i);
+        const long long i = base + nw * 8 + grp;
+        if (u >= 0) {
             bu_row_of(p, u, s0, e0);
             pos = ((s0 + skip) & ~3LL) + 4 * gl;
         }
+        un = i < nlong ? __ldcg(longlist + i) : -1;
         long long hitpos = -1;
         int pv = -1;
         bool live = u >= 0;
-        while (__any_sync(kFull, live)) {
+        for (int step = 0; step < kLongSteps && __any_sync(kFull, live); step++) {
             unsigned hb = 0;
             int4 x = make_int4(0, 0, 0, 0);
             if (live && pos < e0) {
@@ -1541,6 +1547,42 @@ __device__ void bu_phase_b(const SingleParams& p, int d, const unsigned* fcur, u
                 }
             }
             pos += 16;
+        }
+        // a row past its steps: the whole warp, 128 ids at a time
+        unsigned rest = __ballot_sync(kFull, live && gl == 0);
+        while (rest) {
+            const int L = __ffs(rest) - 1;
+            rest &= rest - 1;
+            const long long re = __shfl_sync(kFull, e0, L);
+            long long q = __shfl_sync(kFull, pos, L);   // lane L is its group's first
+            long long hp = -1;
+            int hv = -1;
+            for (; q < re && hp < 0; q += 128) {
+                const long long q4 = q + 4 * lane;
+                unsigned hb = 0;
+                int4 x = make_int4(0, 0, 0, 0);
+                if (q4 < re) {
+                    x = ld_stream4(reinterpret_cast<const int4*>(p.cols_bu + q4));
+                    const int ids[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int t = 0; t < 4; t++)
+                        if (q4 + t < re && in_frontier(fcur, ids[t])) hb |= 1u << t;
+                }
+                const unsigned any = __ballot_sync(kFull, hb != 0);
+                const int t_own = hb ? __ffs(hb) - 1 : 0;
+                const int v_own = (t_own == 0) ? x.x : (t_own == 1) ? x.y : (t_own == 2) ? x.z : x.w;
+                const int first = any ? __ffs(any) - 1 : 0;
+                const int t_src = __shfl_sync(kFull, t_own, first);
+                const int v_src = __shfl_sync(kFull, v_own, first);
+                if (any) {
+                    hp = q + 4 * first + t_src;
+                    hv = v_src;
+                }
+            }
+            if (lane == L) {
+                hitpos = hp;
+                pv = hv;
+            }
         }
         if (u >= 0 && gl == 0) {
             if (hitpos >= 0) {
