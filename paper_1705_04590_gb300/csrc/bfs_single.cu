@@ -119,6 +119,7 @@ struct SingleParams {
     // td_chunk edges at hubs[hub_off[j]..hub_off[j + 1])
     Hub* hubs;
     long long hub_off[kHubClasses + 1];
+    long long hub_win_slices;   // up to so many slices are taken by windows (hub_order)
     Ctrl* ctrl;
     bfs_level_record* rec;
     int rec_cap;
@@ -648,18 +649,22 @@ __device__ __forceinline__ WarpStage warp_stage() { return warp_stage_in(g_stage
 __device__ __forceinline__ WarpStage warp_stage_dcsc() { return warp_stage_in(g_stage_d[threadIdx.x >> 5]); }
 
 // Heavy rows are cut into slices for all warps.  A row of class j (4^j to
-// 4^(j+1) - 1 chunks of td_chunk edges) has 4^j slices of equal length, and the
-// slices of all rows are taken in the order of their place in the row, 64 windows
-// of it: rows are sorted by id, so with ids spread evenly the grid works on one
-// 64th of the targets at a time, and the claims' scattered stores (parents,
-// level bytes) and reads (bitmap words, degree bytes) meet in L2.  In the order
-// the rows were found instead, a claim's 4-byte parent store is a read and a write
-// of its own DRAM sector: R-MAT 26, a level of 72 M hub edges and 10.7 M claims,
-// 956 us, 609 us in this order.  Nothing depends on the even spread but speed.
-// The order needs no list of slices: from the classes' row counts alone a
-// slice's number gives window, class, row and place (hub_slice).
-constexpr int kHubWinShift = 3;                       // 4^3 windows
-constexpr int kHubWindows = 1 << (2 * kHubWinShift);
+// 4^(j+1) - 1 chunks of td_chunk edges) has 4^j slices of equal length, taken class
+// by class and row by row, or, on a large graph, in the order of their place in the
+// row, by 64 windows of it: rows are sorted by id, so with ids spread evenly the grid
+// then works on one window of the targets at a time, and the claims' scattered
+// stores (parents) and reads (bitmap words, degree bytes) meet in L2, where row by
+// row a claim's 4-byte parent store is a read and a write of its own DRAM sector
+// (R-MAT 26, levels of 42 and 138 M hub edges with 8.3 and 14.2 M claims: 467 and
+// 959 us row by row, 347 and 899 by windows).  Below 2^25 vertices the arrays stay in
+// L2 anyway, and a grid in one window claims the same bitmap words at once (R-MAT 21
+// and 24, top-down levels of 10^7 and 10^8 hub edges: 372 and 1741 us row by row, 428
+// and 1924 by windows); past two slices per td_chunk vertices, the claims are so many
+// that every order meets the same sectors (R-MAT 26, 10^9 edges: even).  Nothing
+// depends on the even spread but speed.  Neither order needs a list of slices: from
+// the classes' row counts alone a slice's number gives its row and place (hub_slice).
+constexpr int kHubWin = 3;
+constexpr long long kHubWinN = 1LL << 25;
 
 __device__ __forceinline__ int hub_class(long long deg, int chunk) {
     const unsigned nch = (unsigned)((deg + chunk - 1) / chunk);
@@ -671,44 +676,72 @@ __device__ __forceinline__ long long hub_slices(const LevelCtr& c) {
     return warp_sum(lane < kHubClasses ? (long long)c.hubs[lane] << (2 * lane) : 0LL);
 }
 
+// The order of a level's slices: what hub_slice needs of the counts, read and summed
+// once per phase (in every slice's path instead: R-MAT 21 top-down only 576 us, 544).
+struct HubOrder {
+    long long h, mine, upto;   // lane j's class: rows, slices, slices up to and with it
+    int win;                   // log4 of the windows
+};
+
+__device__ __forceinline__ HubOrder hub_order(const SingleParams& p, const LevelCtr& c, long long slices) {
+    const int lane = lane_id();
+    HubOrder o;
+    o.h = lane < kHubClasses ? (long long)c.hubs[lane] : 0LL;
+    o.mine = o.h << 2 * (lane < kHubClasses ? lane : 0);
+    o.upto = o.mine;
+#pragma unroll
+    for (int s = 1; s < 16; s <<= 1) {
+        const long long y = __shfl_up_sync(kFull, o.upto, s);
+        if (lane >= s) o.upto += y;
+    }
+    o.win = slices <= p.hub_win_slices ? kHubWin : 0;
+    return o;
+}
+
 // Slice x of the level's hub rows (x < hub_slices, the same in every lane; all
-// lanes call): its column range and row vertex.  Window k holds, for each class j
-// >= 3, slices k 4^(j-3) .. (k+1) 4^(j-3) - 1 of every row, and for j < 3 slice
-// k / 4^(3-j) when that divides.
-__device__ __forceinline__ void hub_slice(const SingleParams& p, const LevelCtr& c, long long x, long long& start,
+// lanes call): its column range and row vertex.  Without windows: class by class,
+// row by row.  With 4^W windows, window k holds, for each class j >= W, slices
+// k 4^(j-W) .. (k+1) 4^(j-W) - 1 of every row, and for j < W slice k / 4^(W-j) when
+// that divides.
+__device__ __forceinline__ void hub_slice(const SingleParams& p, const HubOrder& o, long long x, long long& start,
                                           int& len, int& u) {
     const int lane = lane_id();
-    const long long h = lane < kHubClasses ? (long long)c.hubs[lane] : 0LL;
-    const int big = 2 * (lane - kHubWinShift);   // >= 0: log2 of this class's slices per window
-    // slices before window k (a lane's class alone), summed over the classes
-    const long long per = warp_sum(big >= 0 ? h << big : 0LL);
-    const long long h0 = __shfl_sync(kFull, h, 0), h1 = __shfl_sync(kFull, h, 1), h2 = __shfl_sync(kFull, h, 2);
-    auto before = [&](int k) {
-        return per * k + h0 * ((k + 63) >> 6) + h1 * ((k + 15) >> 4) + h2 * ((k + 3) >> 2);
-    };
-    static_assert(kHubWinShift == 3 && kHubWindows == 64, "the windows of classes 0 to 2");
-    int k = 2 * (__popc(__ballot_sync(kFull, before(2 * lane) <= x)) - 1);
-    if (before(k + 1) <= x) k++;
-    long long r = x - before(k);
-    // class: the first whose slices in this window reach past r
-    const long long mine = big >= 0 ? h << big : (k & ((1 << -big) - 1)) == 0 ? h : 0LL;
-    long long incl = mine;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-        const long long y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int j = __ffs(__ballot_sync(kFull, incl > r)) - 1;
-    r -= __shfl_sync(kFull, incl - mine, j);
-    const unsigned hj = (unsigned)__shfl_sync(kFull, h, j);
-    long long slice;
-    unsigned row;
-    if (j >= kHubWinShift) {
-        slice = ((long long)k << (2 * (j - kHubWinShift))) + (unsigned)r / hj;
-        row = (unsigned)r % hj;
+    constexpr int W = kHubWin;
+    int j;
+    long long slice, row;
+    if (o.win == 0) {
+        j = __ffs(__ballot_sync(kFull, o.upto > x)) - 1;
+        const long long r = x - __shfl_sync(kFull, o.upto - o.mine, j);
+        row = r >> (2 * j);
+        slice = r & ((1LL << 2 * j) - 1);
     } else {
-        slice = k >> (2 * (kHubWinShift - j));
-        row = (unsigned)r;
+        const int big = 2 * (lane - W);   // >= 0: log2 of this class's slices per row and window
+        const long long per = warp_sum(big >= 0 ? o.h << big : 0LL);
+        const long long h0 = __shfl_sync(kFull, o.h, 0), h1 = __shfl_sync(kFull, o.h, 1),
+                        h2 = __shfl_sync(kFull, o.h, 2);
+        auto before = [&](int k) { return per * k + h0 * ((k + 63) >> 6) + h1 * ((k + 15) >> 4) + h2 * ((k + 3) >> 2); };
+        static_assert(W == 3, "slices before window k: classes 0, 1 and 2 have one every 64, 16 and 4 windows");
+        int k = 2 * (__popc(__ballot_sync(kFull, before(2 * lane) <= x)) - 1);
+        if (before(k + 1) <= x) k++;
+        long long r = x - before(k);
+        // class: the first whose slices in this window reach past r
+        const long long here = big >= 0 ? o.h << big : (k & ((1 << -big) - 1)) == 0 ? o.h : 0LL;
+        long long incl = here;
+#pragma unroll
+        for (int s = 1; s < 16; s <<= 1) {
+            const long long y = __shfl_up_sync(kFull, incl, s);
+            if (lane >= s) incl += y;
+        }
+        j = __ffs(__ballot_sync(kFull, incl > r)) - 1;
+        r -= __shfl_sync(kFull, incl - here, j);
+        if (j >= W) {
+            const int sl = 2 * (j - W);
+            row = r >> sl;
+            slice = ((long long)k << sl) + (r & ((1LL << sl) - 1));
+        } else {
+            row = r;
+            slice = k >> (2 * (W - j));
+        }
     }
     const int4 raw = __ldcg(reinterpret_cast<const int4*>(p.hubs + p.hub_off[j] + row));
     const long long lo = ((long long)raw.z * slice) >> (2 * j), hi = ((long long)raw.z * (slice + 1)) >> (2 * j);
@@ -789,19 +822,23 @@ template <bool kDir, bool kNow>
 __device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int* qnext, int snext,
                           unsigned long long& acc_m, unsigned long long& acc_h, unsigned long long& acc_in) {
     const int lane = lane_id();
-    const long long gw = gtid() >> 5, nw = gthreads() >> 5;
+    const long long gw = spread_warp(), nw = gthreads() >> 5;
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
     const long long slices = hub_slices(ctr);
     // few slices: each in 2^sh parts, down to 32 edges, so that a small level is one
-    // short round per warp (R-MAT 26, 93 K edges: 404 slices 51 us, in 16 parts 25 us)
+    // short round or two per warp (R-MAT 26, 93 K edges: 404 slices 51 us, in 16 parts
+    // 25 us).  More parts than two per warp cost more steps than they even out (R-MAT
+    // 22, 92 hubs: 37 us with up to 8 a warp, 25 with 2; a level of 80 K slices: 490
+    // us whole, 502 in quarters)
     int sh = 0;
-    while (sh < 4 && (slices << (sh + 1)) <= 8 * nw) sh++;
+    while (sh < 4 && (slices << (sh + 1)) <= 2 * nw) sh++;
     const long long nt = slices << sh;
+    const HubOrder ord = hub_order(p, ctr, slices);
     for (long long t = gw; t < nt; t += nw) {
         long long start;
         int len, u;
-        hub_slice(p, ctr, t >> sh, start, len, u);
+        hub_slice(p, ord, t >> sh, start, len, u);
         const int i = (int)(t & ((1 << sh) - 1));
         int k0 = (int)(((long long)len * i) >> sh);
         len = (int)(((long long)len * (i + 1)) >> sh);
@@ -887,10 +924,11 @@ __device__ void td_min_pass(const SingleParams& p, int d, const int* q, long lon
         }
     }
     const long long nt = hub_slices(ctr);
+    const HubOrder ord = hub_order(p, ctr, nt);
     for (long long t = gw; t < nt; t += nw) {
         long long start;
         int len, u;
-        hub_slice(p, ctr, t, start, len, u);
+        hub_slice(p, ord, t, start, len, u);
         for (int k = lane; k < len; k += 32) min_offer(p, d, u, __ldg(p.cols + start + k));
     }
 }
@@ -2991,6 +3029,7 @@ static void hub_regions(SingleParams& p) {
         at += p.nnz / least + 1;
     }
     p.hub_off[bfsk::kHubClasses] = at;
+    p.hub_win_slices = p.n >= bfsk::kHubWinN ? 2 * p.n / p.td_chunk : 0;
 }
 
 bfs_status single_prepare(bfs_graph* g, cudaStream_t s) { return single_prepare_work(g, g->single, s, 0); }
@@ -3139,8 +3178,9 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     // a small graph's levels are the chain of their reads and barriers, not work to
     // spread: one CTA per SM halves the arrivals of a barrier (R-MAT 12: 50.6 us with
     // 304 CTAs, 47.8 with 152, 49.2 with 8; R-MAT 18: 81.0, 77.6 and 161; R-MAT 20 is
-    // even at 107 / 108)
-    if (g->n <= bfsk::kSmallN && grid > g->sm_count) {
+    // even at 107 / 108).  A search that stays top-down reads every edge with scattered
+    // claims, and has those to spread (R-MAT 17: 140 us with 152, 134 with 304)
+    if (g->n <= bfsk::kSmallN && opt.mode != BFS_MODE_TD_ONLY && grid > g->sm_count) {
         grid = g->sm_count;
         p.expected = (unsigned)grid + extra;
     }

@@ -293,3 +293,47 @@ def test_cluster_levels_of_short_rows(gpu_lib, shape, min_id):
     v = np.flatnonzero(lv > 0)
     assert np.array_equal(lv[pa[v]], lv[v] - 1) and np.array_equal(pa[roots], roots)
     g.close()
+
+
+@pytest.mark.parametrize("chunk", [64, 128, 4096])
+def test_hub_slices_by_windows(gpu_lib, chunk):
+    """A graph of 2^25 vertices and some, whose heavy rows are taken by windows of the
+    targets: degrees at every class of slice counts below, at and above the 64 windows.
+    One root, the hubs, their targets: levels, smallest parents and counts are known."""
+    bfs = gpu_lib
+    n = (1 << 25) + 3
+    degs = [d for k in (1, 4, 16, 64, 256, 1024) for d in (chunk * (k - 1) + 1, chunk * k, chunk * k + 1)]
+    degs = [d for d in degs if d < n // 16] + [97] * 70 + [4 * chunk + 5] * 70
+    rng = np.random.default_rng(chunk)
+    ids = rng.permutation(n).astype(np.int32)
+    root, hubs, rest = ids[0], ids[1:1 + len(degs)], ids[1 + len(degs):]
+    src, dst = [np.full(hubs.size, root)], [hubs]
+    for h, d in zip(hubs, degs):
+        src.append(np.full(d, h))
+        dst.append(rng.choice(rest[:2_000_000] if d < 1000 else rest, d, replace=False) if d < 100_000 else
+                   rest[rng.integers(0, rest.size - d):][:d])
+    want_parent = np.full(n, n, np.int32)
+    for s, t in zip(src, dst):
+        np.minimum.at(want_parent, t, s)
+    level = np.where(want_parent < n, 2, -1).astype(np.int32)
+    level[hubs], level[root] = 1, 0
+    want_parent[want_parent == n] = -1
+    want_parent[root], want_parent[hubs] = root, root
+    g = bfs.Graph.from_edges(np.concatenate(src), np.concatenate(dst), n)
+    lv, pa = _buffers(n)
+    edges = sum(degs)
+    for pm in (bfs.PARENT_ANY, bfs.PARENT_MIN_ID):
+        info = g.run(int(root), parent=pa, level=lv, stats=True, record_levels=8,
+                     opts=bfs.options(mode=bfs.MODE_TD_ONLY, parent_mode=pm, td_chunk=chunk))
+        assert np.array_equal(lv.cpu().numpy(), level)
+        p = pa.cpu().numpy()
+        two = np.flatnonzero(level == 2)
+        assert (level[p[two]] == 1).all() and np.array_equal(p < 0, level < 0)
+        if pm == bfs.PARENT_MIN_ID:
+            assert np.array_equal(p, want_parent)
+        else:   # each parent is a hub with that edge
+            key = np.sort(np.concatenate([np.full(t.size, s, np.int64) * n + t for s, t in zip(src[1:], dst[1:])]))
+            k = p[two].astype(np.int64) * n + two
+            assert (key[np.searchsorted(key, k)] == k).all()
+        assert info["records"][1, 2] == edges + hubs.size and info["records"][1, 3] == two.size
+    g.close()
