@@ -100,15 +100,17 @@ typedef struct {
     int32_t alpha;         /* >= 1 */
     int32_t beta;          /* >= 1 */
     int32_t parent_mode;   /* BFS_PARENT_* */
-    int32_t td_big_degree; /* top-down: frontier vertices above this degree are split into edge chunks
-                              shared by all warps (0 = tuned default) */
+    int32_t td_big_degree; /* top-down: frontier vertices above this degree are cut into slices
+                              shared by all warps (0 = tuned default 96; bfs_run_multi cuts above
+                              max(this, 256)) */
     int64_t timeout_ms;    /* limit of every device-side wait; 0 = default 10000 */
     uint64_t seed;         /* BFS_MODE_RANDOM only */
     int32_t bu_rows;       /* order in which bottom-up steps scan a row: BFS_BU_ROWS_BY_ID (stored order,
                               the paper's) or BFS_BU_ROWS_HUB_FIRST (needs BFS_FLAG_BUILD_HUB_FIRST, the
                               CSR layout and BFS_PARENT_ANY).  Levels are the same; the bottom-up
                               examination counts and the parents chosen follow the order */
-    int32_t td_chunk;      /* top-down: edges per chunk task of a vertex above td_big_degree, 64..4096
+    int32_t td_chunk;      /* top-down: a vertex above td_big_degree whose row has 4^j to 4^(j+1) - 1
+                              chunks of this many edges is cut into 4^j slices, 64..4096
                               (0 = tuned default 128) */
     int32_t ctas_per_sm;   /* CTAs per SM of the persistent single-source launch, 1 .. the resident
                               maximum (0 = the maximum); fewer means fewer arrivals per grid barrier */
@@ -140,7 +142,8 @@ typedef struct {
     int64_t examined;     /* top-down: m_f; bottom-up: sum over searching vertices of the 1-based
                              position of the first frontier neighbour in sorted order, or the degree */
     int64_t t_ns;         /* device time from the end of initialisation to the end of this level */
-    int64_t aux;          /* top-down: edge-chunk tasks, or -1 for a level thread-block cluster 0 ran
+    int64_t aux;          /* top-down: td_chunk-edge chunks of the rows above td_big_degree (they
+                             are searched in slices), or -1 for a level thread-block cluster 0 ran
                              alone (options.cluster_size); bottom-up: searchers continued past their
                              first window (id-ordered rows) or row head (hub-first rows): the long list */
     int64_t t_mid_ns;     /* device time at the level's first internal barrier (0 if none) */
@@ -332,8 +335,11 @@ bfs_status bfs_run_multiroot(bfs_graph* g, const int32_t* roots_host, int32_t k,
  * advanced together, one fused persistent launch per 64 roots.
  * level_dev: device int32[k][n] row-major (row i = search from roots_host[i]).
  * parent_dev: NULL, or int32[k][n]: for each reached v != root the minimum-id
- * neighbour one level closer (BFS_PARENT_MIN_ID semantics).  Asynchronous
- * on `stream`.  Errors: INVALID, OOM, CUDA.
+ * neighbour one level closer (BFS_PARENT_MIN_ID semantics).  The first call
+ * allocates its work buffers, about 64 bytes a vertex (half of it four planes that
+ * hold the lanes' levels by bits, which the rows are written from at the end;
+ * where they cannot be had, the search writes the rows as it goes, with the
+ * same results).  Asynchronous on `stream`.  Errors: INVALID, OOM, CUDA.
  */
 bfs_status bfs_run_multi(bfs_graph* g, const int32_t* roots_host, int32_t k, int32_t* level_dev,
                          int32_t* parent_dev, const bfs_options* opt, void* stream);

@@ -43,7 +43,7 @@ struct __align__(256) LevelCtr {
     unsigned long long accm;       // degree sum of the frontier
     unsigned long long scanned;    // bottom-up searchers of the level producing it
     unsigned long long examined;   // serial early-exit examinations of that level
-    unsigned long long ntask;      // bottom-up: length of that level's long list
+    unsigned long long ntask;      // top-down: td_chunk-edge chunks of the heavy rows; bottom-up: length of the long list
     unsigned long long nmiss;      // bottom-up first-probe misses left to phase B (miss-list length)
     unsigned long long nmiss_in;   // ... resolved by their chunk's warp in phase A
     unsigned long long dsum_out;   // directed graphs: out-degree sum of the frontier

@@ -12,11 +12,12 @@
 //              bottom-up -> top-down when n_f * beta < n.
 //   top-down  (Algorithm 1 inner loops; the local discovery of Algorithm 3):
 //              for u in the queue, for v in adj(u): claim v by an atomicOr on
-//              the visited bitmap; the winner writes parent/level and appends
-//              v to the next queue (warp ballot + one atomicAdd per warp).
+//              the visited bitmap; the winner writes the parent and appends
+//              v to the next queue (staged per warp in shared memory); the level
+//              byte is written where the next step reads that queue.
 //              Frontier vertices of degree > big_deg are cut into slices
 //              that all warps share after a barrier (load balance on R-MAT
-//              hubs), taken in the order of the targets they hold; the rest are gathered warp-cooperatively (a warp prefix
+//              hubs); the rest are gathered warp-cooperatively (a warp prefix
 //              sum over its 32 vertices' degrees maps lanes onto edges).
 //   bottom-up (Algorithm 2 inner loops; the local search of Algorithm 4):
 //              a warp owns 32 consecutive vertices (one word of the
@@ -793,6 +794,9 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
                     raise_status(&p.ctrl->b, kDevOverflow);
                 }
             }
+            // the record's aux: chunks, whatever the slices
+            const int nch = warp_sum(big ? (int)((unsigned)(deg + p.td_chunk - 1) / (unsigned)p.td_chunk) : 0);
+            if (lane == 0) atomicAdd(&p.ctrl->lv[snext].ntask, (unsigned long long)nch);
         }
         const int incl = warp_inclusive_scan(mydeg);
         const int total = __shfl_sync(kFull, incl, 31);
@@ -2357,7 +2361,6 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 if (!level_sync(p, snext, s_ctr)) return;
             }
         }
-        const long long slices = dir == TD ? hub_slices(s_ctr) : 0;
         const long long nf_next = (long long)(dir == TD ? s_ctr.tail : s_ctr.accn);
         if (threadIdx.x == 0) {
             const long long macc = (long long)s_ctr.accm;
@@ -2373,7 +2376,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 r.scanned = dir == BU ? (long long)s_ctr.scanned : 0;
                 r.examined = dir == BU ? (long long)s_ctr.examined : S.mf;
                 r.t_ns = (long long)(globaltimer_ns() - S.t_start);
-                r.aux = dir == TD ? slices : (long long)s_ctr.ntask;
+                r.aux = (long long)s_ctr.ntask;
                 r.t_mid_ns = S.t_mid ? (long long)(S.t_mid - S.t_start) : 0;
                 p.rec[S.d] = r;
             }
@@ -3180,7 +3183,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     // 304 CTAs, 47.8 with 152, 49.2 with 8; R-MAT 18: 81.0, 77.6 and 161; R-MAT 20 is
     // even at 107 / 108).  A search that stays top-down reads every edge with scattered
     // claims, and has those to spread (R-MAT 17: 140 us with 152, 134 with 304)
-    if (g->n <= bfsk::kSmallN && opt.mode != BFS_MODE_TD_ONLY && grid > g->sm_count) {
+    if (g->n <= bfsk::kSmallN && opt.mode != BFS_MODE_TD_ONLY && opt.ctas_per_sm <= 0 && grid > g->sm_count) {
         grid = g->sm_count;
         p.expected = (unsigned)grid + extra;
     }

@@ -336,4 +336,32 @@ def test_hub_slices_by_windows(gpu_lib, chunk):
             k = p[two].astype(np.int64) * n + two
             assert (key[np.searchsorted(key, k)] == k).all()
         assert info["records"][1, 2] == edges + hubs.size and info["records"][1, 3] == two.size
+        assert info["records"][1, 8] == sum(-(-(d + 1) // chunk) for d in degs if d + 1 > 96)   # chunks of heavy rows
+    g.close()
+
+
+def test_multi_without_room_for_planes(gpu_lib, monkeypatch):
+    """The batched search where the allocator refuses the level planes."""
+    import torch
+    bfs = gpu_lib
+    e = graphgen.rmat(12, seed=6)
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+    roots = [int(r) for r in graphgen.pick_roots(e, 40, 5)]
+    level, parent = _buffers(e.n, len(roots))
+    alloc, refused = torch.cuda.caching_allocator_alloc, []
+
+    def short_of_memory(nbytes, *rest):
+        if nbytes == 32 * e.n:
+            refused.append(nbytes)
+            raise torch.cuda.OutOfMemoryError("no room")
+        return alloc(nbytes, *rest)
+
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", short_of_memory)
+    g.run_multi(roots, level, parent=parent)
+    g.sync()
+    assert refused
+    want = [oracle.levels(ref, r) for r in roots]
+    assert np.array_equal(level.cpu().numpy().reshape(-1, e.n), np.stack(want))
+    assert np.array_equal(parent.cpu().numpy().reshape(-1, e.n), np.stack([oracle.min_parent(ref, w) for w in want]))
     g.close()
