@@ -59,8 +59,9 @@ struct __align__(256) LevelCtr {
 constexpr int kCtrWords = 16 + kHubClasses;
 
 // Control block of one single-source launch: zeroed by the host
-// (cudaMemsetAsync) before every launch.  The level counters rotate (slot =
-// level % 3).
+// (cudaMemsetAsync) before every launch.  The level counters rotate through the
+// levels that the whole grid runs: while a level collects in one slot, the
+// frontier's own may still be being read and the third is cleared.
 struct Ctrl {
     BarrierState b;
     LevelCtr lv[3];

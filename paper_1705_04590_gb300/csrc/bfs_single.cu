@@ -151,6 +151,8 @@ struct SingleParams {
 
 constexpr int TD = 0, BU = 1;
 
+__device__ __forceinline__ int next_slot(int slot) { return slot == 2 ? 0 : slot + 1; }
+
 // the grid barrier, then the counters of level slot `slot` into the CTA's copy
 __device__ __forceinline__ bool level_sync(const SingleParams& p, int slot, LevelCtr& ctr) {
     return grid_sync_read(&p.ctrl->b, p.expected, p.timeout_ns, &p.ctrl->lv[slot], &ctr, kCtrWords);
@@ -2061,8 +2063,8 @@ __device__ void cluster_levels(const SingleParams& p, const int* qcur, int d0, l
             out.reached = reached;
             out.done = done;
             if (lead) {
-                // the grid resumes at level L with every per-level counter slot clear
-                for (int k = 0; k < 3; k++) c->lv[k].zero();
+                // (the level counters are the grid's: a CTA may still be copying the slot that
+                // the barrier before the episode completed, so none is touched here)
                 c->clu_spill = 0;
                 c->clu_d = out.d;
                 c->clu_nf = nf;
@@ -2184,6 +2186,11 @@ struct LoopState {
     unsigned long long epi;          // cluster episodes so far
     int d, prev, qsel, bsel;         // level; last direction; which queue / bitmap holds the frontier
     int no_clu;                      // the level a cluster episode just handed back (the grid takes it)
+    // counter slot of the frontier.  It moves on with the grid's levels alone: a cluster
+    // episode uses and writes none, so after it the next slot is clear, as the last grid
+    // level left it, and the slot that a late CTA is still copying after a barrier is
+    // written only past another barrier, which that CTA has to reach
+    int slot;
 };
 
 // kMinId: the launch also makes the parents the minimum-id ones (parent_mode
@@ -2238,6 +2245,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
         S.bsel = 0;
         S.epi = 0;
         S.no_clu = -1;
+        S.slot = 0;
         S.t_start = lead ? globaltimer_ns() : 0;
     }
     // cluster levels only in a launch whose clusters have the size the parameters name
@@ -2277,15 +2285,15 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
             continue;
         }
         // the level's counters collect in lv[snext]; the slot after it is cleared
-        const int snext = (S.d + 1) % 3;
+        const int snext = next_slot(S.slot);
         if (lead) {
-            c->lv[(S.d + 2) % 3].zero();
+            c->lv[next_slot(snext)].zero();
             S.t_mid = 0;
         }
         if (dir == TD) {
             if (S.prev == BU) {
                 bitmap_to_queue(p, S.bsel ? p.front1 : p.front0, S.bsel ? p.front0 : p.front1,
-                                S.qsel ? p.queue1 : p.queue0, &c->lv[S.d % 3].tail);
+                                S.qsel ? p.queue1 : p.queue0, &c->lv[S.slot].tail);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
             {
@@ -2390,6 +2398,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 else S.bsel = S.bsel ^ 1;
                 S.prev = dir;
                 S.d = S.d + 1;
+                S.slot = snext;
             }
         }
         if (nf_next == 0) break;

@@ -365,3 +365,68 @@ def test_multi_without_room_for_planes(gpu_lib, monkeypatch):
     assert np.array_equal(level.cpu().numpy().reshape(-1, e.n), np.stack(want))
     assert np.array_equal(parent.cpu().numpy().reshape(-1, e.n), np.stack([oracle.min_parent(ref, w) for w in want]))
     g.close()
+
+
+@pytest.mark.parametrize("min_id", [False, True])
+@pytest.mark.parametrize("cluster", [2, 16])
+def test_cluster_episodes_of_one_level(gpu_lib, cluster, min_id):
+    """Cluster episodes that end at once, after which the other CTAs may still be on their
+    way out of the barrier before: components of a few vertices (the search ends in the
+    episode that starts it) and chains of brooms (a path, then a fan that outgrows the
+    cluster, again and again: the grid and the cluster take turns, from every counter slot),
+    one search right behind the other and from several roots."""
+    import torch
+    bfs = gpu_lib
+    src, dst, n = [], [], 0
+    tiny = []
+    for k in range(60):            # an edge, a path of three, a star of 20
+        tiny.append(n)
+        for a, b in ([(0, 1)], [(0, 1), (1, 2)], [(0, j) for j in range(1, 21)])[k % 3]:
+            src.append([n + a]); dst.append([n + b])
+        n += (2, 3, 21)[k % 3]
+    start = n
+    for j in range(7):             # handle of j % 4 + 1 vertices, then 100 x 100 leaves, then the next
+        h = np.arange(n, n + j % 4 + 2)
+        src.append(h[:-1]); dst.append(h[1:])
+        mid = np.arange(h[-1] + 1, h[-1] + 101)
+        leaf = np.arange(mid[-1] + 1, mid[-1] + 1 + 10_000)
+        src += [np.full(100, h[-1]), np.repeat(mid, 100)]
+        dst += [mid, leaf]
+        n = int(leaf[-1]) + 1
+        src.append([int(leaf[j])]); dst.append([n])
+    n += 1
+    ids = np.random.default_rng(6).permutation(n).astype(np.int32)
+    e = graphgen.EdgeList(n, ids[np.concatenate(src)], ids[np.concatenate(dst)])
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+    o = bfs.options(mode=bfs.MODE_TD_ONLY, cluster_size=cluster, timeout_ms=2000,
+                    parent_mode=bfs.PARENT_MIN_ID if min_id else bfs.PARENT_ANY)
+    roots = [int(ids[r]) for r in [start, n - 1] + tiny[:6]]
+    want = {r: oracle.levels(ref, r) for r in roots}
+    sched = {r: oracle.do_schedule(ref, want[r], oracle.MODE_TD) for r in roots}
+    level, parent = _buffers(n)
+    for r in roots:
+        for _ in range(5):
+            info = g.run(r, parent=parent, level=level, opts=o, stats=True, record_levels=64)
+            pa = parent.cpu().numpy()
+            assert np.array_equal(level.cpu().numpy(), want[r]), r
+            assert oracle.certify(ref, r, want[r], pa, labels) == (0, -1), r
+            assert not min_id or np.array_equal(pa, oracle.min_parent(ref, want[r])), r
+            for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext"]):
+                assert np.array_equal(info["records"][:, col], getattr(sched[r], name)), (r, name)
+            clu = info["records"][:, 8] == -1
+            assert clu.any() and (r in roots[2:] or not clu.all()), r
+    outs = [torch.empty(n, dtype=torch.int32, device="cuda") for _ in range(200)]
+    for i, out in enumerate(outs):
+        g.run(int(ids[tiny[i % 60]]), level=out, opts=o)
+    g.sync()
+    for i, out in enumerate(outs):
+        size = (2, 3, 21)[i % 60 % 3]
+        lv = out.cpu().numpy()
+        assert (lv >= 0).sum() == size and lv[ids[tiny[i % 60]]] == 0 and lv.max() == (1, 2, 1)[i % 60 % 3], i
+    several = [int(ids[t]) for t in tiny[:30]]
+    g.run_multiroot(several, parent=parent, level=level, opts=o)
+    want = np.min(np.stack([np.where(x < 0, 1 << 30, x) for x in (oracle.levels(ref, r) for r in several)]), axis=0)
+    assert np.array_equal(level.cpu().numpy(), np.where(want == 1 << 30, -1, want))
+    g.close()
