@@ -314,32 +314,7 @@ __device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned l
             const unsigned long long mL = __shfl_sync(kMFull, miss, L);
             unsigned long long aL = __shfl_sync(kMFull, acc, L);
             bool live = has;
-            // (a row that finds the task list full goes on here)
-            for (int step = 0; __any_sync(kMFull, live); step++) {
-                if (step == kPullSteps) {
-                    if (live && gl == 0) {
-                        const long long nch = (qe - q + kPullChunk - 1) / kPullChunk;
-                        const unsigned long long t0 = atomicAdd(&c->ntask[slot], (unsigned long long)nch);
-                        if ((long long)t0 + nch <= p.task_cap) {
-                            for (long long k = 0; k < nch; k++) {
-                                MTask t;
-                                t.start = q + k * kPullChunk;
-                                t.len = (int)min((long long)kPullChunk, qe - t.start);
-                                t.v = (int)(base + L);
-                                p.tasks[t0 + k] = t;
-                            }
-                            live = false;
-                        } else {
-                            // what was reserved past the room left: tasks with nothing in them
-                            MTask t;
-                            t.start = 0;
-                            t.len = 0;
-                            t.v = (int)(base + L);
-                            for (long long k = (long long)t0; k < p.task_cap; k++) p.tasks[k] = t;
-                        }
-                    }
-                    live = __shfl_sync(kMFull, live, lane & ~3);
-                }
+            for (int step = 0; step < kPullSteps && __any_sync(kMFull, live); step++) {
                 unsigned long long x = 0;
                 const long long q4 = q + 4 * gl;   // a multiple of 4: the window was aligned
                 if (live && q4 < qe) {
@@ -356,6 +331,51 @@ __device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned l
                     q += 16;
                     live = (aL & mL) != mL && q < qe;
                 }
+            }
+            // the rest of a row: chunk tasks
+            if (live && gl == 0) {
+                const long long nch = (qe - q + kPullChunk - 1) / kPullChunk;
+                const unsigned long long t0 = atomicAdd(&c->ntask[slot], (unsigned long long)nch);
+                if ((long long)t0 + nch <= p.task_cap) {
+                    for (long long k = 0; k < nch; k++) {
+                        MTask t;
+                        t.start = q + k * kPullChunk;
+                        t.len = (int)min((long long)kPullChunk, qe - t.start);
+                        t.v = (int)(base + L);
+                        p.tasks[t0 + k] = t;
+                    }
+                    live = false;
+                } else {
+                    // what was reserved past the room left: tasks with nothing in them
+                    MTask t;
+                    t.start = 0;
+                    t.len = 0;
+                    t.v = (int)(base + L);
+                    for (long long k = (long long)t0; k < p.task_cap; k++) p.tasks[k] = t;
+                }
+            }
+            // rows that found the list full: the whole warp, 128 ids a step (left to its
+            // four lanes, a hub behind many rows of a hundred ids is a chain of a step per 16)
+            unsigned rest = __ballot_sync(kMFull, live && gl == 0);
+            while (rest) {
+                const int own = __ffs(rest) - 1;
+                rest &= rest - 1;
+                const long long re = __shfl_sync(kMFull, qe, own);
+                const unsigned long long want = __shfl_sync(kMFull, mL, own);
+                unsigned long long got = __shfl_sync(kMFull, aL, own);
+                for (long long r = __shfl_sync(kMFull, q, own); r < re && (got & want) != want; r += 128) {
+                    unsigned long long x = 0;
+                    const long long r4 = r + 4 * lane;
+                    if (r4 < re) {
+                        const int4 y = __ldg(reinterpret_cast<const int4*>(p.cols_bu + r4));
+                        const int ids[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                        for (int t = 0; t < 4; t++)
+                            if (r4 + t < re) x |= ldcg64(p.front + ids[t]);
+                    }
+                    got |= warp_or64(x);
+                }
+                if (lane == own) aL = got;
             }
             if (has && gl == 0) s_acc[wib][L] = aL;
         }

@@ -430,3 +430,43 @@ def test_cluster_episodes_of_one_level(gpu_lib, cluster, min_id):
     want = np.min(np.stack([np.where(x < 0, 1 << 30, x) for x in (oracle.levels(ref, r) for r in several)]), axis=0)
     assert np.array_equal(level.cpu().numpy(), np.where(want == 1 << 30, -1, want))
     g.close()
+
+
+def test_multi_hub_behind_a_full_task_list(gpu_lib):
+    """Bottom-up pulls of a batch where the rows of about 90 ids, one chunk task each, fill
+    the task list before the longest row, the last id's, asks for its thousands: the answers,
+    and that the row is not a chain of 16-id steps.  A step is one dependent read of ids and
+    masks, 0.5 to 2 us: 2 M ids are 125,000 steps of 16 (over 62 ms a level) and 15,625 of
+    128 (under 32 ms); the limit lies between."""
+    import torch
+    bfs = gpu_lib
+    rows, leaves = 200_000, 2_000_000
+    n = rows + leaves + 1
+    r = graphgen.erdos_renyi(rows, 45 * rows, seed=9)
+    leaf = np.arange(rows, rows + leaves, dtype=np.int32)
+    e = graphgen.EdgeList(n, np.concatenate([r.src, np.full(leaves, n - 1, np.int32)]), np.concatenate([r.dst, leaf]))
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    deg = np.diff(ref.offsets)
+    # rows longer than what a pull reads before it asks for a task, against the list's room
+    assert (deg[:rows] > 72).sum() > ref.cols.size // 512 + ref.cols.size // 256 + 1024
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+    roots = [3, rows + 5, n - 1]
+    level, parent = _buffers(n, len(roots))
+    o = bfs.options(mode=bfs.MODE_BU_ONLY)
+    g.run_multi(roots, level, parent=parent, opts=o)
+    g.sync()
+    want = [oracle.levels(ref, x) for x in roots]
+    assert np.array_equal(level.cpu().numpy().reshape(-1, n), np.stack(want))
+    assert np.array_equal(parent.cpu().numpy().reshape(-1, n), np.stack([oracle.min_parent(ref, w) for w in want]))
+    # one search that never reaches the hub: every level scans its row to the end
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    took = []
+    for _ in range(3):
+        ev[0].record()
+        g.run_multi(roots[:1], level[:n], opts=o)
+        ev[1].record()
+        ev[1].synchronize()
+        took.append(ev[0].elapsed_time(ev[1]))
+    levels = int(want[0].max()) + 1
+    assert min(took) < 40.0 * levels, took
+    g.close()
