@@ -40,6 +40,7 @@ constexpr int kMChunk = 512;      // edges per top-down chunk task
 constexpr int kMBigDeg = 256;     // rows above this become chunk tasks (the task lists are sized for it)
 constexpr int kPullChunk = 512;   // ids per chunk task of a long row (pulls, parents)
 constexpr int kPullSteps = 4;     // 16-id steps a 4-lane group pulls before the rest of the row becomes tasks
+constexpr int kPullEnd = 8;       // ... and of a row that is read to its end in so many
 constexpr int kPlaneMax = 15;     // largest level + 1 that the four planes hold
 constexpr unsigned kMFull = 0xffffffffu;
 
@@ -269,6 +270,10 @@ __device__ void ms_tasks_phase(const MultiParams& p, MCtrl* c, int slot, int* tq
 // steps becomes chunk tasks of kPullChunk ids for all warps (ms_bu_tasks_phase):
 // few steps here, as a group's are a chain (with 16 steps the groups of the level
 // that reads most of R-MAT 22 took 469 us for 30 M ids, the tasks 276 for 100 M).
+// A row that ends within kPullEnd steps is read to its end: its few ids as a task
+// cost a warp, an atomic and a place in the list that longer rows need
+// (Erdos-Renyi of 200 K vertices, 96 neighbours each, 40 roots: 469 us with such
+// tasks, 296 without; R-MAT 22 with 64 roots 2160 and 1978).
 // Bound by dependent reads (ids, then masks): one row at a time per warp left
 // two thirds of the cycles waiting at the level's barrier for the warps whose
 // vertices had long rows (R-MAT 20, 64 roots).
@@ -314,10 +319,11 @@ __device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned l
             const unsigned long long mL = __shfl_sync(kMFull, miss, L);
             unsigned long long aL = __shfl_sync(kMFull, acc, L);
             bool live = has;
-            for (int step = 0; step < kPullSteps && __any_sync(kMFull, live); step++) {
+            const int most = qe - q <= 16 * kPullEnd ? kPullEnd : kPullSteps;
+            for (int step = 0; __any_sync(kMFull, live && step < most); step++) {
                 unsigned long long x = 0;
                 const long long q4 = q + 4 * gl;   // a multiple of 4: the window was aligned
-                if (live && q4 < qe) {
+                if (live && step < most && q4 < qe) {
                     const int4 y = __ldg(reinterpret_cast<const int4*>(p.cols_bu + q4));
                     const int ids[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
@@ -326,7 +332,7 @@ __device__ void ms_bu_phase(const MultiParams& p, MCtrl* c, int slot, unsigned l
                 }
                 x |= __shfl_xor_sync(kMFull, x, 1);
                 x |= __shfl_xor_sync(kMFull, x, 2);
-                if (live) {
+                if (live && step < most) {
                     aL |= x;
                     q += 16;
                     live = (aL & mL) != mL && q < qe;

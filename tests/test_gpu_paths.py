@@ -470,3 +470,31 @@ def test_multi_hub_behind_a_full_task_list(gpu_lib):
     levels = int(want[0].max()) + 1
     assert min(took) < 40.0 * levels, took
     g.close()
+
+
+@pytest.mark.parametrize("k", [3, 64])
+def test_multi_pull_lengths(gpu_lib, k):
+    """Bottom-up pulls of rows of every length around where a group stops (72 ids), where it
+    goes on to the end (136) and where one chunk task becomes two (584, 1096), starting on
+    every offset of a 16-byte group."""
+    bfs = gpu_lib
+    rng = np.random.default_rng(k)
+    lens = list(range(60, 150)) + [582, 583, 584, 585, 586, 648, 1095, 1096, 1097, 1160]
+    m = 6000
+    src = np.concatenate([np.full(d, i) for i, d in enumerate(lens)])
+    dst = len(lens) + np.concatenate([rng.choice(m, d, replace=False) for d in lens])
+    n = len(lens) + m
+    ids = rng.permutation(n).astype(np.int32)
+    e = graphgen.EdgeList(n, ids[src], ids[dst])
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, hub_first=True)
+    roots = rng.choice(graphgen.pick_roots(e, 64, 5), k).tolist()
+    want = np.stack([oracle.levels(ref, r) for r in roots])
+    level, _ = _buffers(n, k)
+    for mode in (bfs.MODE_BU_ONLY, bfs.MODE_DO):
+        for rows in (bfs.BU_ROWS_BY_ID, bfs.BU_ROWS_HUB_FIRST):
+            level.fill_(-7)
+            g.run_multi(roots, level, opts=bfs.options(mode=mode, bu_rows=rows))
+            g.sync()
+            assert np.array_equal(level.cpu().numpy().reshape(k, n), want), (mode, rows)
+    g.close()
