@@ -42,6 +42,10 @@ constexpr int kPullChunk = 512;   // ids per chunk task of a long row (pulls, pa
 constexpr int kPullSteps = 4;     // 16-id steps a 4-lane group pulls before the rest of the row becomes tasks
 constexpr int kPullEnd = 8;       // ... and of a row that is read to its end in so many
 constexpr int kPlaneMax = 15;     // largest level + 1 that the four planes hold
+// a batch of levels of up to so many roots writes its rows as it goes: the planes are 32
+// bytes a vertex whatever the lanes (R-MAT 22: 8 roots 1140 us without, 1196 with planes,
+// 40 roots 1785 and 1470; Erdos-Renyi of 4 M vertices, 20 roots: 1372 and 1277)
+constexpr int kDirectLanes = 8;
 constexpr unsigned kMFull = 0xffffffffu;
 
 __device__ __forceinline__ long long m_gtid() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
@@ -218,6 +222,9 @@ __device__ void ms_td_phase(const MultiParams& p, MCtrl* c, int slot, const int*
             unsigned long long nb[4];
 #pragma unroll
             for (int q = 0; q < 4; q++) {
+                u[q] = -1;
+                nb[q] = 0;
+                if (k0 + q * 32 >= total) continue;   // (the same in every lane)
                 const int k = k0 + q * 32 + lane;
                 int j = 0;
 #pragma unroll
@@ -469,7 +476,10 @@ __device__ void ms_apply_phase(const MultiParams& p, MCtrl* c, int slot, int ite
 // as ms_apply_phase, old frontier bits dropped in the same pass, and the new
 // frontier listed in queue nq (null after a top-down level: the touched queue is
 // that list).  Four vertices per lane are in flight; read by read, one vertex at a
-// time, a nearly empty level took 95 us of latency at R-MAT 22.  Vertex by vertex in
+// time, a nearly empty level took 95 us of latency at R-MAT 22.  A warp's four groups of
+// 32 lie a whole grid apart, so that a graph of fewer vertices than the grid has threads
+// is spread over all warps (128 in a row to a warp instead, and the empty groups walked
+// too: a torus of 120^2, 40 roots, 121 levels, 2761 us; 1829 so).  Vertex by vertex in
 // the touched queue's order the masks, planes and offsets (112 bytes a vertex) are
 // random DRAM accesses: 918 K vertices of 4.2 M took 358 us.  In order, with few pull
 // steps and four pushes in flight, R-MAT 22 with 64 roots went from 1843 to 1576 us
@@ -482,18 +492,18 @@ __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int
     const long long gw = m_gtid() >> 5, nw = m_gthreads() >> 5;
     MStage st = m_stage();
     unsigned long long an = 0, am = 0, adone = 0, found = 0;
-    for (long long base = gw * 128; base < p.n; base += nw * 128) {
+    for (long long base = gw * 32; base < p.n; base += nw * 128) {
         unsigned long long x[4], f[4], s[4];
         long long deg[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const long long v = base + k * 32 + lane;
+            const long long v = base + k * nw * 32 + lane;
             x[k] = v < p.n ? ldcg64(p.next + v) : 0ull;
             f[k] = v < p.n ? ldcg64(p.front + v) : 0ull;
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const long long v = base + k * 32 + lane;
+            const long long v = base + k * nw * 32 + lane;
             s[k] = 0;
             deg[k] = 0;
             if (x[k]) {
@@ -503,7 +513,8 @@ __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const long long v = base + k * 32 + lane;
+            const long long v = base + k * nw * 32 + lane;
+            if (v - lane >= p.n) break;   // (the same in every lane)
             if (x[k]) {
                 p.next[v] = 0ull;
                 p.seen[v] = s[k] | x[k];
@@ -622,11 +633,21 @@ __device__ __forceinline__ int ms_decide(const MultiParams& p, int prev, long lo
     return (nf * (long long)p.beta < p.n) ? 0 : 1;
 }
 
+// The barrier after a bottom-up phase, and its number of chunk tasks: read once per CTA
+// (by every thread the counter's one line serves 16 times the requests), and not at
+// all where no row is long enough for a task.
+__device__ __forceinline__ bool bu_sync(const MultiParams& p, MCtrl* c, int slot, unsigned long long& ntask) {
+    if (p.long_rows) return grid_sync_read(&c->b, p.expected, p.timeout_ns, &c->ntask[slot], &ntask, 1);
+    if (threadIdx.x == 0) ntask = 0;
+    return grid_sync(&c->b, p.expected, p.timeout_ns);
+}
+
 // ---------------------------------------------------------------- persistent driver
 
 __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
     __shared__ LaneSmem L;
     load_lanes(p, L);
+    __shared__ unsigned long long ntask;   // a bottom-up level's chunk tasks
     MCtrl* c = p.ctrl;
     const unsigned long long active = p.active;
     bool direct = p.planes == nullptr;
@@ -680,8 +701,8 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
                 ms_apply_phase(p, c, slot, it, active, L, direct, tq, touched);
         } else {
             ms_bu_phase(p, c, slot, active);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            if (ld_relaxed64(&c->ntask[slot]) > 0) {
+            if (!bu_sync(p, c, slot, ntask)) return;
+            if (ntask > 0) {
                 ms_bu_tasks_phase(p, c, slot, active);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
@@ -892,6 +913,7 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_serve_kernel(MultiParams p, in
                                                                 unsigned long long drop) {
     __shared__ LaneSmem L;
     load_lanes(p, L);
+    __shared__ unsigned long long ntask;   // a bottom-up level's chunk tasks
     MCtrl* c = p.ctrl;
     const unsigned long long active = p.active;
     const long long tid = m_gtid(), nth = m_gthreads();
@@ -943,8 +965,8 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_serve_kernel(MultiParams p, in
                 ms_apply_phase(p, c, slot, it, active, L, true, tq, touched);
         } else {
             ms_bu_phase(p, c, slot, active);
-            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
-            if (ld_relaxed64(&c->ntask[slot]) > 0) {
+            if (!bu_sync(p, c, slot, ntask)) return;
+            if (ntask > 0) {
                 ms_bu_tasks_phase(p, c, slot, active);
                 if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
             }
@@ -1076,6 +1098,8 @@ static MultiParams multi_params(bfs_graph* g, MultiWork& w, const bfs_options& o
     p.beta = opt.beta;
     p.planes = w.planes;
     p.big_deg = std::max(opt.td_big_degree, bfsk::kMBigDeg);
+    // a pull reads at least five ids of a row in its first window, then 16 a step
+    p.long_rows = g->max_degree > 5 + 16 * bfsk::kPullEnd;
     p.timeout_ns = (unsigned long long)(opt.timeout_ms > 0 ? opt.timeout_ms : 10000) * 1000000ull;
     p.expected = (unsigned)w.grid + (unsigned)(g->debug_barrier_extra > 0 ? g->debug_barrier_extra : 0);
     return p;
@@ -1101,6 +1125,7 @@ bfs_status multi_launch(bfs_graph* g, const int32_t* roots_host, int32_t k, int3
         MultiParams p = multi_params(g, w, opt);
         p.active = (kk == 64) ? ~0ull : ((1ull << kk) - 1ull);
         p.level0 = t.rows[0];
+        if (!parent && kk <= bfsk::kDirectLanes) p.planes = nullptr;
         void* args[] = {&p};
         BFS_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)bfsk::bfs_multi_kernel, dim3(w.grid), dim3(w.block),
                                                  args, 0, s));

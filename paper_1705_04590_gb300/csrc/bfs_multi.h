@@ -71,6 +71,7 @@ struct MultiParams {
     const int* roots;
     unsigned long long active;
     int mode, alpha, beta, big_deg;
+    int long_rows;                 // the graph has rows long enough for a bottom-up chunk task
     unsigned long long timeout_ns;
     unsigned expected;
 };

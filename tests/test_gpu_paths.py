@@ -498,3 +498,24 @@ def test_multi_pull_lengths(gpu_lib, k):
             g.sync()
             assert np.array_equal(level.cpu().numpy().reshape(k, n), want), (mode, rows)
     g.close()
+
+
+@pytest.mark.parametrize("n", [31, 33, 155_649, 311_296, 622_597])
+@pytest.mark.parametrize("k", [8, 9])
+def test_multi_sizes_around_the_grid(gpu_lib, n, k):
+    """Batches on graphs just below, above and at several times the grid's threads, with as
+    many roots as write their rows as they go and one more (which keeps level planes)."""
+    bfs = gpu_lib
+    e = graphgen.erdos_renyi(n, 3 * n, seed=n)
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+    roots = np.random.default_rng(n).choice(graphgen.pick_roots(e, 6, 5), k).tolist()
+    lv = {r: oracle.levels(ref, r) for r in set(roots)}
+    want = np.stack([lv[r] for r in roots])
+    level, _ = _buffers(n, k)
+    for mode in (bfs.MODE_DO, bfs.MODE_BU_ONLY, bfs.MODE_TD_ONLY):
+        level.fill_(-7)
+        g.run_multi(roots, level, opts=bfs.options(mode=mode))
+        g.sync()
+        assert np.array_equal(level.cpu().numpy().reshape(k, n), want), mode
+    g.close()
