@@ -98,6 +98,7 @@ struct SingleParams {
     // directed graph the transpose's: the in-edge rows)
     const long long* __restrict__ off_bu;
     const unsigned char* __restrict__ deg8_in;   // directed: min(in-degree, 255)
+    int min_rows;     // MIN_ID: parents of top-down levels are looked for after the last level
     int directed;     // 1: off/cols are out-edge rows, off_bu/cols_bu in-edge rows
     const unsigned* __restrict__ isolated;
     long long n, nnz, W;
@@ -939,10 +940,25 @@ __device__ void td_min_pass(const SingleParams& p, int d, const int* q, long lon
     }
 }
 
-// ... and the vertices that cluster levels discovered (`lv`: one bit per level
-// byte; their frontiers live in shared memory and their rows are short), after
-// the last level: the first neighbour one level closer in each sorted row, a
-// lane per short row, the warp together for a longer one.
+// Where the rows are short (max degree <= kMinRowsDeg) and the offers many, that is
+// left for after the last level instead (min_parent_rows): a row is read up to its first
+// hit, which comes soon when kMinRowsPer or more offers meet per discovered vertex, and
+// nothing keeps a thread long.  That pass sweeps all vertices, so it has to save n offers,
+// with kMinPassCost for a pass and its barrier.  Top-down only, offers at every level
+// and by this rule: Erdos-Renyi of 16 neighbours, 4 M vertices 1303 and 1025 us, 40 M
+// 16.9 and 10.5 ms; a torus of 1000^2 without clusters 9503 and 6518 us (with
+// kMinRowsPer 6 9552: its levels offer 4).  Direction-optimizing searches, whose
+// top-down levels meet few vertices twice, stay at 319 us (rows at every level: 521).
+// Rows of 180 neighbours gain nothing (520 and 542 us, 300 K vertices).
+constexpr long long kMinRowsDeg = 64, kMinRowsPer = 3, kMinPassCost = 1 << 14;
+__device__ __forceinline__ bool leave_to_rows(const SingleParams& p, long long mf, long long nnext, long long offered) {
+    return p.min_rows && mf >= kMinRowsPer * nnext && mf + offered >= p.n;
+}
+
+// ... these, and the vertices that cluster levels discovered (their frontiers live in
+// shared memory and their rows are short): the first neighbour one level closer in
+// each sorted row, a lane per short row, the warp together for a longer one.  `lv`:
+// one bit per level byte.
 __device__ void min_parent_rows(const SingleParams& p, const unsigned* lv) {
     constexpr int kShort = 64;
     const int lane = lane_id();
@@ -2185,6 +2201,8 @@ struct LoopState {
     unsigned long long t_start, t_mid;
     unsigned long long epi;          // cluster episodes so far
     int d, prev, qsel, bsel;         // level; last direction; which queue / bitmap holds the frontier
+    int rows;                        // kMinId: min_parent_rows has vertices to look at
+    long long offered;               // kMinId: edges offered again so far, and a pass's fixed cost in edges
     int no_clu;                      // the level a cluster episode just handed back (the grid takes it)
     // counter slot of the frontier.  It moves on with the grid's levels alone: a cluster
     // episode uses and writes none, so after it the next slot is clear, as the last grid
@@ -2204,12 +2222,14 @@ struct LoopState {
 template <bool kMinId, bool kHub, bool kClu, bool kDir>
 __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(SingleParams p) {
     Ctrl* c = p.ctrl;
-    __shared__ unsigned s_clu_lv[kMinId && kClu ? 8 : 1];   // level bytes that cluster levels discovered
+    // kMinId: level bytes whose vertices have their parents looked for after the last
+    // level (min_parent_rows)
+    __shared__ unsigned s_row_lv[kMinId ? 8 : 1];
     __shared__ LevelCtr s_ctr;                      // the last completed level's counters
     __shared__ volatile LoopState S;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    if constexpr (kMinId && kClu) {
-        if (threadIdx.x < 8) s_clu_lv[threadIdx.x] = 0u;
+    if constexpr (kMinId) {
+        if (threadIdx.x < 8) s_row_lv[threadIdx.x] = 0u;
     }
     if (lead) c->t_enter = globaltimer_ns();
     init_phase(p);
@@ -2244,6 +2264,8 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
         S.qsel = 0;
         S.bsel = 0;
         S.epi = 0;
+        S.rows = 0;
+        S.offered = 0;
         S.no_clu = -1;
         S.slot = 0;
         S.t_start = lead ? globaltimer_ns() : 0;
@@ -2267,9 +2289,10 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 if constexpr (kMinId) {
                     for (int L = S.d + 1; L <= cs.d; L++) {
                         const int b = min(L, (int)kLvDeep);
-                        s_clu_lv[b >> 5] |= 1u << (b & 31);
+                        s_row_lv[b >> 5] |= 1u << (b & 31);
                         if (b == kLvDeep) break;
                     }
+                    S.rows = 1;
                 }
                 S.epi = S.epi + 1;
                 S.d = cs.d;
@@ -2286,6 +2309,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
         }
         // the level's counters collect in lv[snext]; the slot after it is cleared
         const int snext = next_slot(S.slot);
+        bool to_rows = false;   // kMinId: the level's parents are left to min_parent_rows
         if (lead) {
             c->lv[next_slot(snext)].zero();
             S.t_mid = 0;
@@ -2313,10 +2337,13 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 if (!level_sync(p, snext, s_ctr)) return;
             }
             if constexpr (kMinId) {
-                if (s_ctr.tail > 0) {
+                to_rows = leave_to_rows(p, S.mf, (long long)s_ctr.tail, S.offered);
+                if (s_ctr.tail > 0 && !to_rows) {
                     td_min_pass(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, s_ctr);
                     // the next level writes this queue and the hub lists
                     if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+                } else {
+                    __syncthreads();   // every thread has read S
                 }
             }
         } else {
@@ -2389,6 +2416,15 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 p.rec[S.d] = r;
             }
             if (nf_next > 0) {
+                if constexpr (kMinId) {
+                    if (to_rows) {
+                        const int b = min(S.d + 1, (int)kLvDeep);
+                        s_row_lv[b >> 5] |= 1u << (b & 31);
+                        S.rows = 1;
+                    } else if (dir == TD) {
+                        S.offered = S.offered + S.mf + kMinPassCost;
+                    }
+                }
                 S.reached = S.reached + nf_next;
                 // what the unreached lose: in-degrees (undirected: both sums coincide)
                 S.mu = S.mu - (!kDir ? mf_next : dir == TD ? (long long)s_ctr.dsum_in : macc);
@@ -2409,10 +2445,10 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
         c->t_levels = globaltimer_ns();
     }
     // every level ended at a grid barrier, so all staged bytes are visible here
-    if constexpr (kMinId && kClu) {
+    if constexpr (kMinId) {
         __syncthreads();
-        if (S.epi > 0) {
-            min_parent_rows(p, s_clu_lv);
+        if (S.rows) {
+            min_parent_rows(p, s_row_lv);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
         }
     }
@@ -3162,6 +3198,7 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     p.beta = opt.beta;
     p.parent_mode = opt.parent_mode;
     p.big_deg = opt.td_big_degree > 0 ? opt.td_big_degree : 96;
+    p.min_rows = g->max_degree <= bfsk::kMinRowsDeg ? 1 : 0;
     p.td_chunk = opt.td_chunk > 0 ? opt.td_chunk : bfsk::kDefaultChunk;
     hub_regions(p);
     p.clu_c = 1;

@@ -519,3 +519,52 @@ def test_multi_sizes_around_the_grid(gpu_lib, n, k):
         g.sync()
         assert np.array_equal(level.cpu().numpy().reshape(k, n), want), mode
     g.close()
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("shape", ["er", "er_wide", "cap64", "cap65", "ladder", "path"])
+def test_min_parents_of_short_rows(gpu_lib, shape, directed):
+    """Minimum-id parents on graphs whose rows are short: levels that offer theirs edge by
+    edge and levels that leave them to the pass after the last one, in one search; rows just
+    within and past the length that allows it, and levels past the byte staging."""
+    bfs = gpu_lib
+    rng = np.random.default_rng(8)
+    if shape.startswith("cap"):
+        # a random graph and a star of 64 or 65 leaves among its vertices
+        n, cap = 4000, int(shape[3:])
+        e = graphgen.erdos_renyi(n, 3 * n, seed=8)
+        keep = (e.src != 7) & (e.dst != 7)
+        leaf = rng.choice(np.arange(8, n, dtype=np.int32), cap, replace=False)
+        e = graphgen.EdgeList(n, np.concatenate([e.src[keep], np.full(cap, 7, np.int32)]),
+                              np.concatenate([e.dst[keep], leaf]))
+    else:
+        e = {"er": lambda: graphgen.erdos_renyi(20_000, 160_000, seed=8),
+             "er_wide": lambda: graphgen.erdos_renyi(300_001, 600_000, seed=8),
+             "ladder": lambda: _mesh(3, 900, True, 3), "path": lambda: graphgen.path(600)}[shape]()
+    if directed and shape in ("ladder", "path"):
+        e = graphgen.EdgeList(e.n, np.concatenate([e.src, e.dst[::2]]), np.concatenate([e.dst, e.src[::2]]))
+    if directed:
+        out, inn = oracle.build_digraph(e.n, e.src, e.dst)
+    else:
+        out = inn = oracle.build_csr(e.n, e.src, e.dst)
+    if shape.startswith("cap") and not directed:
+        assert out.degree().max() == cap
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, directed=directed)
+    level, parent = _buffers(e.n)
+    row = np.repeat(np.arange(e.n), np.diff(inn.offsets))
+    for root in graphgen.pick_roots(e, 3, 2).tolist():
+        _, want, _ = oracle.bfs_topdown(out, root)
+        up = (want[row] > 0) & (want[inn.cols] == want[row] - 1)
+        pmin = np.full(e.n, e.n, np.int64)
+        np.minimum.at(pmin, row[up], inn.cols[up])
+        pmin[pmin == e.n] = -1
+        pmin[root] = root
+        for mode in (bfs.MODE_TD_ONLY, bfs.MODE_DO, bfs.MODE_RANDOM):
+            for with_level in (True, False):
+                parent.fill_(-7)
+                g.run(root, parent=parent, level=level if with_level else None,
+                      opts=bfs.options(mode=mode, seed=5, parent_mode=bfs.PARENT_MIN_ID, cluster_size=1))
+                g.sync()
+                assert np.array_equal(parent.cpu().numpy(), pmin), (root, mode, with_level)
+                assert not with_level or np.array_equal(level.cpu().numpy(), want), (root, mode)
+    g.close()
