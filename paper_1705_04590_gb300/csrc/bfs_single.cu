@@ -1545,10 +1545,14 @@ __device__ void bu_misses(const SingleParams& p, int d, const unsigned* fcur, un
     long_flush(lst, longlist, longcnt);
 }
 
-// 16-id steps of a 4-lane group before the whole warp takes what is left of the row,
-// 128 ids a step: a group with a long row otherwise keeps its warp's other seven
-// waiting (256 R-MAT graphs in one: 1.7 M long rows 446 us, 263 us so)
-constexpr int kLongSteps = 8;
+// 16-id steps of the 4-lane groups before the whole warp takes what is left of a row,
+// 128 ids a step, once no more than kLongFew groups have one: a group with a long row
+// otherwise keeps its warp's other seven waiting (256 R-MAT graphs in one: 1.7 M long
+// rows 446 us, 263 us so).  While most groups are busy they read as many ids a step
+// together as the warp would, stop sooner each, and start no row anew (bottom-up only,
+// Erdos-Renyi of 760 neighbours, 262 K vertices: 3134 us with every row handed over
+// after its eight steps, 2253 so; of 1000, 100 K vertices, 837 and 874).
+constexpr int kLongSteps = 8, kLongFew = 4;
 
 // Bottom-up, phase B: the long list.  Groups of 4 lanes take one searcher
 // each (8 per warp); a group reads 16 ids per step (one int4 per lane, in row
@@ -1577,7 +1581,9 @@ __device__ void bu_phase_b(const SingleParams& p, int d, const unsigned* fcur, u
         long long hitpos = -1;
         int pv = -1;
         bool live = u >= 0;
-        for (int step = 0; step < kLongSteps && __any_sync(kFull, live); step++) {
+        for (int step = 0;; step++) {
+            const int groups = __popc(__ballot_sync(kFull, live)) >> 2;
+            if (groups == 0 || (step >= kLongSteps && groups <= kLongFew)) break;
             unsigned hb = 0;
             int4 x = make_int4(0, 0, 0, 0);
             if (live && pos < e0) {
@@ -1608,7 +1614,7 @@ __device__ void bu_phase_b(const SingleParams& p, int d, const unsigned* fcur, u
             }
             pos += 16;
         }
-        // a row past its steps: the whole warp, 128 ids at a time
+        // the rows left: the whole warp, 128 ids at a time
         unsigned rest = __ballot_sync(kFull, live && gl == 0);
         while (rest) {
             const int L = __ffs(rest) - 1;
