@@ -568,3 +568,40 @@ def test_min_parents_of_short_rows(gpu_lib, shape, directed):
                 assert np.array_equal(parent.cpu().numpy(), pmin), (root, mode, with_level)
                 assert not with_level or np.array_equal(level.cpu().numpy(), want), (root, mode)
     g.close()
+
+
+@pytest.mark.parametrize("deg", [130, 140, 152, 300, 1100])
+@pytest.mark.parametrize("long_rows", [1, 4, 5, 9, 0])
+def test_bottom_up_long_rows_in_a_warp(gpu_lib, deg, long_rows):
+    """Bottom-up searches with 1, 4, 5 and 9 rows past what the 4-lane groups read before the
+    whole warp may take them, and with all rows (0) that long: levels, parents, counts."""
+    bfs = gpu_lib
+    rng = np.random.default_rng(deg + long_rows)
+    n = 3000
+    if long_rows == 0:
+        e = graphgen.erdos_renyi(n, n * deg // 2, seed=deg)
+    else:
+        # the long rows' neighbours are the upper half; the search starts far from them
+        h = np.arange(long_rows, dtype=np.int32)
+        t = np.concatenate([rng.choice(np.arange(n // 2, n, dtype=np.int32), deg, replace=False) for _ in h])
+        r = np.arange(long_rows, n, dtype=np.int32)
+        ids = rng.permutation(n).astype(np.int32)
+        e = graphgen.EdgeList(n, ids[np.concatenate([np.repeat(h, deg), r[:-1:7], r[:-3:5]])],
+                              ids[np.concatenate([t, r[1::7], r[3::5]])])
+    ref = oracle.build_csr(e.n, e.src, e.dst)
+    labels = oracle.components(ref)
+    g = bfs.Graph.from_edges(e.src, e.dst, e.n, hub_first=True)
+    level, parent = _buffers(n)
+    for root in graphgen.pick_roots(e, 2, 3).tolist() + [int(e.dst[0])]:
+        want = oracle.levels(ref, root)
+        for rows, scan in ((bfs.BU_ROWS_BY_ID, ref), (bfs.BU_ROWS_HUB_FIRST, oracle.hub_first(ref))):
+            for mode, omode in ((bfs.MODE_BU_ONLY, oracle.MODE_BU), (bfs.MODE_DO, oracle.MODE_DO)):
+                info = g.run(root, parent=parent, level=level, stats=True, record_levels=1024,
+                             opts=bfs.options(mode=mode, bu_rows=rows))
+                pa = parent.cpu().numpy()
+                assert np.array_equal(level.cpu().numpy(), want), (root, mode, rows)
+                assert oracle.certify(ref, root, want, pa, labels) == (0, -1), (root, mode, rows)
+                s = oracle.do_schedule(scan, want, omode)
+                for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext", "scanned", "examined"]):
+                    assert np.array_equal(info["records"][:, col], getattr(s, name)), (root, mode, rows, name)
+    g.close()
