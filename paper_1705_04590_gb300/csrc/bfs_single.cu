@@ -762,6 +762,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
     unsigned long long* tail = &p.ctrl->lv[snext].tail;
     WarpStage st = warp_stage();
     st.pf = nf < kPrefetchNf;
+    unsigned chunks = 0;   // of this lane's heavy rows, for the level's record
     // A small frontier is spread over every warp (fewer vertices per warp, so
     // each warp's edges take one gather round instead of several dependent ones).
     const long long per = nf >= nw * 32 ? 32 : max(1LL, (nf + nw - 1) / nw);
@@ -797,9 +798,7 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
                     raise_status(&p.ctrl->b, kDevOverflow);
                 }
             }
-            // the record's aux: chunks, whatever the slices
-            const int nch = warp_sum(big ? (int)((unsigned)(deg + p.td_chunk - 1) / (unsigned)p.td_chunk) : 0);
-            if (lane == 0) atomicAdd(&p.ctrl->lv[snext].ntask, (unsigned long long)nch);
+            if (big) chunks += (unsigned)(deg + p.td_chunk - 1) / (unsigned)p.td_chunk;
         }
         const int incl = warp_inclusive_scan(mydeg);
         const int total = __shfl_sync(kFull, incl, 31);
@@ -819,6 +818,10 @@ __device__ void td_phase(const SingleParams& p, int d, const int* qcur, long lon
             const int v = act ? __ldg(p.cols + sj + (k - exj)) : 0;
             td_visit<kDir, kNow>(p, d, uj, v, act, st, qnext, tail, acc_m);
         }
+    }
+    if (__any_sync(kFull, chunks != 0)) {
+        chunks = __reduce_add_sync(kFull, chunks);
+        if (lane == 0) atomicAdd(&p.ctrl->lv[snext].ntask, (unsigned long long)chunks);
     }
     block_flush<kDir>(p, st, qnext, tail, acc_m);
     acc_h += st.hv;
