@@ -113,7 +113,9 @@ typedef struct {
                               chunks of this many edges is cut into 4^j slices, 64..4096
                               (0 = tuned default 128) */
     int32_t ctas_per_sm;   /* CTAs per SM of the persistent single-source launch, 1 .. the resident
-                              maximum (0 = the maximum); fewer means fewer arrivals per grid barrier */
+                              maximum; fewer means fewer arrivals per grid barrier.  0 = automatic: 1 on
+                              graphs of up to 2^18 vertices unless the mode is top-down only, else the
+                              maximum */
     int32_t cluster_size;  /* CSR single-source searches of an undirected graph: CTAs per thread-block
                               cluster (2, 4, 8 or 16), whose first cluster runs top-down levels with
                               a small frontier alone (frontier in distributed shared memory, one
@@ -381,8 +383,8 @@ bfs_status bfs_run_csr_noalloc(const int64_t* row_offsets, const int32_t* col_id
  * (roots_host) for a grid of direction thresholds alpha in {6,14,24,32,96},
  * beta in {12,24,64,128} and top-down hub cut-offs td_big_degree in
  * {64,96,256}; then, from the winner, the top-down chunk size td_chunk in
- * {128,256,512,1024}, then ctas_per_sm in {1, the maximum}, then (CSR,
- * undirected) cluster_size in {1, 8, 16}, one knob at a
+ * {128,256,512,1024}, then ctas_per_sm in {1, the resident maximum (0 where
+ * the default is that)}, then (CSR, undirected) cluster_size in {1, 8, 16}, one knob at a
  * time.  Each configuration runs once for warm-up, then the k roots timed with
  * CUDA events; the fastest mean goes to *best (other fields from `base`, or
  * the defaults when base is NULL).  Levels do not depend on these choices

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "bfs_internal.h"
+#include "launch_shape.h"
 
 namespace bfsrt {
 
@@ -427,7 +428,6 @@ bfs_status bfs_autotune(bfs_graph* g, const int32_t* roots_host, int32_t k, cons
     static const int betas[] = {12, 24, 64, 128};
     static const int bigs[] = {64, 96, 256};
     static const int chunks[] = {128, 256, 512, 1024};
-    static const int ctas[] = {1, 0};   // 1 CTA per SM, or as many as fit
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     BFS_CUDA_TRY(cudaEventCreate(&e0));
     BFS_CUDA_TRY(cudaEventCreate(&e1));
@@ -475,6 +475,8 @@ bfs_status bfs_autotune(bfs_graph* g, const int32_t* roots_host, int32_t k, cons
         consider(o);
     }
     const bfs_options chunk_win = win;
+    int ctas[2];
+    tuner_ctas(g->n, BFS_MODE_DO, g->sm_count, g->single.grid, ctas);
     for (int c : ctas) {
         if (st != BFS_OK) break;
         bfs_options o = chunk_win;

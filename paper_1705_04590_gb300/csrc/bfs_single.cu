@@ -41,6 +41,7 @@
 
 #include "bfs_common.cuh"
 #include "bfs_internal.h"
+#include "launch_shape.h"
 
 namespace bfsk {
 
@@ -48,7 +49,6 @@ namespace bfsk {
 #define BFS_BLOCK 512
 #endif
 constexpr int kBlock = BFS_BLOCK;  // CSR kernel
-constexpr long long kSmallN = 1LL << 18;   // graphs up to this size launch one CTA per SM
 constexpr int kDBlock = 1024;   // DCSC kernel (one CTA per vertex block)
 constexpr int kWarps = 32;      // shared-memory per-warp arrays sized for up to 1024 threads
 constexpr int kChunk = 256;    // td_chunk of the allocation-free entry point
@@ -3029,6 +3029,8 @@ __global__ void k_static_isolated(const long long* __restrict__ off, long long n
 
 namespace bfsrt {
 
+static_assert(kModeTdOnly == BFS_MODE_TD_ONLY, "launch_shape.h");
+
 using bfsk::Ctrl;
 using bfsk::SingleParams;
 using bfsk::Hub;
@@ -3218,7 +3220,6 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     p.seed = opt.seed;
     p.timeout_ns = (unsigned long long)(opt.timeout_ms > 0 ? opt.timeout_ms : 10000) * 1000000ull;
     const unsigned extra = (unsigned)(g->debug_barrier_extra > 0 ? g->debug_barrier_extra : 0);
-    p.expected = (unsigned)w.grid + extra;
     p.tile_ptr = nullptr;
     p.jc = nullptr;
     p.cp = nullptr;
@@ -3228,20 +3229,8 @@ bfs_status single_launch_work(bfs_graph* g, SingleWork& w, const int32_t* roots_
     p.Bw = 0;
     p.dcsc_stream = 0;
     const bool dcsc = opt.layout == BFS_LAYOUT_DCSC_TILED;
-    int grid = w.grid, block = w.block;
-    if (opt.ctas_per_sm > 0 && (long long)opt.ctas_per_sm * g->sm_count < grid) {
-        grid = opt.ctas_per_sm * g->sm_count;
-        p.expected = (unsigned)grid + extra;
-    }
-    // a small graph's levels are the chain of their reads and barriers, not work to
-    // spread: one CTA per SM halves the arrivals of a barrier (R-MAT 12: 50.6 us with
-    // 304 CTAs, 47.8 with 152, 49.2 with 8; R-MAT 18: 81.0, 77.6 and 161; R-MAT 20 is
-    // even at 107 / 108).  A search that stays top-down reads every edge with scattered
-    // claims, and has those to spread (R-MAT 17: 140 us with 152, 134 with 304)
-    if (g->n <= bfsk::kSmallN && opt.mode != BFS_MODE_TD_ONLY && opt.ctas_per_sm <= 0 && grid > g->sm_count) {
-        grid = g->sm_count;
-        p.expected = (unsigned)grid + extra;
-    }
+    int grid = search_grid(g->n, opt.mode, opt.ctas_per_sm, g->sm_count, w.grid), block = w.block;
+    p.expected = (unsigned)grid + extra;
     size_t dyn = bfsk::kSingleDynSmem;
     if (dcsc) {
         const DcscTiles& D = g->dcsc;
