@@ -13,8 +13,8 @@
 //             v: level_i[v] = iteration + 1 - start_i.
 // A batch keeps the levels bit-sliced while it runs (64 lanes x 4 bits = one
 // 32-byte sector per vertex) and writes the 64 level rows once, at the end, in
-// whole lines; a search deeper than four bits hold writes the rows it has then
-// and goes on writing them directly.  The same sectors give the minimum-id
+// whole lines; a search that finds vertices deeper than four bits hold writes the
+// rows it has then and goes on writing them directly.  The same sectors give the minimum-id
 // parents: one read of a neighbour's sector compares all 64 lanes at once.
 // Direction per iteration from the union frontier with the same rule as the
 // single-source search (m_f * alpha > m_u; n_f * beta < n).  Levels do not
@@ -591,6 +591,20 @@ __device__ void ms_rows_phase(const MultiParams& p, unsigned long long active) {
     }
 }
 
+// The levels of the frontier that iteration `iter` found (its `len` vertices listed in fq).
+__device__ void ms_frontier_rows(const MultiParams& p, int iter, const LaneSmem& L, const int* fq, long long len) {
+    const long long tid = m_gtid(), nth = m_gthreads();
+    for (long long i = tid; i < len; i += nth) {
+        const int v = __ldcg(fq + i);
+        unsigned long long bits = ldcg64(p.front + v);
+        while (bits) {
+            const int i2 = __ffsll((long long)bits) - 1;
+            bits &= bits - 1;
+            L.rows[i2][v] = iter + 1 - L.start[i2];
+        }
+    }
+}
+
 // Fill the level rows of lanes in `mask` with -1 (rows of n entries).
 __device__ void ms_fill_rows(const MultiParams& p, unsigned long long mask, const LaneSmem& L) {
     const long long tid = m_gtid(), nth = m_gthreads();
@@ -681,12 +695,6 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
         const long long flen = (long long)ld_relaxed64(&c->qlen[qsel]);
         unsigned long long* tlen = &c->qlen[qsel ^ 1];
         const int dir = ms_decide(p, prev, flen, mf, mu);
-        if (!direct && it + 2 > kPlaneMax) {
-            // deeper than the planes: the rows as they stand (every CTA is past the last
-            // apply's barrier; the first write into a row from here on is after the next)
-            ms_rows_phase(p, active);
-            direct = true;
-        }
         if (dir == 0) {
             ms_td_phase(p, c, slot, fq, flen, tq, tlen);
             if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
@@ -722,6 +730,15 @@ __global__ void __launch_bounds__(kMBlock, 2) bfs_multi_kernel(MultiParams p) {
         mu -= (long long)ld_relaxed64(&c->mdone[slot]);
         mf = (long long)ld_relaxed64(&c->accm[slot]);
         prev = dir;
+        if (!direct && it + 2 > kPlaneMax) {
+            // vertices past the planes, which hold nothing of them: the rows as the planes
+            // have them, then these vertices' levels
+            ms_rows_phase(p, active);
+            direct = true;
+            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+            ms_frontier_rows(p, it, L, qsel ? p.q1 : p.q0, nt);
+            if (!grid_sync(&c->b, p.expected, p.timeout_ns)) return;
+        }
     }
     if (!direct) ms_rows_phase(p, active);
 }

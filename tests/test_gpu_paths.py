@@ -605,3 +605,41 @@ def test_bottom_up_long_rows_in_a_warp(gpu_lib, deg, long_rows):
                 for col, name in enumerate(["dir", "nf", "mf", "nnext", "mnext", "scanned", "examined"]):
                     assert np.array_equal(info["records"][:, col], getattr(s, name)), (root, mode, rows, name)
     g.close()
+
+
+def test_multi_parents_at_the_planes_depth(gpu_lib):
+    """A batch with parents whose deepest level is 13, 14 (the last one that the planes hold)
+    and 15, on a graph with hubs: the answers, and that the one of 14 is served from the
+    planes like the one of 13.  Past them the parents come from a scan of every row for
+    every search, a hundred times the work here; one level more may double the planes' time."""
+    import torch
+    bfs = gpu_lib
+    took = {}
+    for depth in (13, 14, 15):
+        r = graphgen.rmat(16, seed=1616)
+        ref = oracle.build_csr(r.n, r.src, r.dst)
+        hub = int(np.argmax(ref.degree()))
+        far = oracle.levels(ref, hub)
+        # a path on the hub: its end is `depth` levels from the vertices farthest from the hub
+        tail = depth - int(far.max())
+        assert tail > 0
+        path = np.concatenate([[hub], np.arange(r.n, r.n + tail)]).astype(np.int32)
+        e = graphgen.EdgeList(r.n + tail, np.concatenate([r.src, path[:-1]]), np.concatenate([r.dst, path[1:]]))
+        ref = oracle.build_csr(e.n, e.src, e.dst)
+        roots = [e.n - 1] * 2 + np.flatnonzero(far >= 0)[:30].tolist()
+        want = np.stack([oracle.levels(ref, x) for x in roots])
+        assert want.max() == depth
+        g = bfs.Graph.from_edges(e.src, e.dst, e.n)
+        level, parent = _buffers(e.n, len(roots))
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        for _ in range(4):
+            ev[0].record()
+            g.run_multi(roots, level, parent=parent)
+            ev[1].record()
+            ev[1].synchronize()
+            took[depth] = min(took.get(depth, 1e9), ev[0].elapsed_time(ev[1]))
+        assert np.array_equal(level.cpu().numpy().reshape(-1, e.n), want), depth
+        assert np.array_equal(parent.cpu().numpy().reshape(-1, e.n),
+                              np.stack([oracle.min_parent(ref, w) for w in want])), depth
+        g.close()
+    assert took[14] < 2 * took[13], took
