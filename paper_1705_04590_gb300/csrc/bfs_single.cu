@@ -2430,7 +2430,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                         const int b = min(S.d + 1, (int)kLvDeep);
                         s_row_lv[b >> 5] |= 1u << (b & 31);
                         S.rows = 1;
-                    } else if (dir == TD) {
+                    } else if (dir == TD && p.min_rows) {
                         S.offered = S.offered + S.mf + kMinPassCost;
                     }
                 }
