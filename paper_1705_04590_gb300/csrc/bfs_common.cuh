@@ -3,8 +3,9 @@
 // Memory-model notes used throughout:
 //  * Anything written by another CTA during the same launch (visited /
 //    frontier bitmaps, queues, counters) is read with ld.global.cg (L2 only):
-//    the per-SM L1 is not coherent, and a line cached at an earlier level
-//    would be stale at a later one.
+//    the per-SM L1 is not coherent, so a line may only be kept in it over a
+//    phase that does not write it, between two grid barriers (whose acquire
+//    drops what L1 held).  One read does: the tiles' frontier segments (seg_bit).
 //  * The graph (row offsets, column ids, isolated-vertex bitmap) is read-only
 //    for the life of a launch and goes through the non-coherent path (__ldg).
 //  * Grid-wide ordering comes from grid_sync(): a bounded sense barrier
@@ -218,9 +219,9 @@ __device__ __forceinline__ bool grid_sync(BarrierState* c, unsigned expected, ui
     return s_ok != 0;
 }
 
-// The barrier, and then `words` counters (at most 32, one line) into shared
+// The barrier, and then `words` counters (at most 32, two lines) into shared
 // memory by the first warp of each CTA.  Read by every warp instead, the
-// counters' one L2 line serves 16 times the requests one after another: 2.5 us
+// counters' L2 lines serve 16 times the requests one after another: 2.5 us
 // a counter at 304 CTAs of 16 warps, as long as the barrier itself.
 __device__ __forceinline__ bool grid_sync_read(BarrierState* c, unsigned expected, uint64_t timeout_ns,
                                                const void* src, void* dst, int words) {

@@ -546,7 +546,7 @@ __device__ void ms_apply_all_phase(const MultiParams& p, MCtrl* c, int slot, int
     block_add4(an, am, adone, 0, &c->accn[slot], &c->accm[slot], &c->mdone[slot], nullptr);
 }
 
-// Clear the three masks and both queue counters (grid-stride).
+// a[0..cnt) to zero (grid-stride; a is 16-byte aligned).
 __device__ void ms_clear_words(unsigned long long* a, long long cnt) {
     const long long tid = m_gtid(), nth = m_gthreads();
     const ulonglong2 z = make_ulonglong2(0ull, 0ull);
@@ -554,6 +554,7 @@ __device__ void ms_clear_words(unsigned long long* a, long long cnt) {
     if ((cnt & 1) && tid == 0) a[cnt - 1] = 0ull;
 }
 
+// The three masks, and the level planes where the launch keeps them.
 __device__ void ms_clear_phase(const MultiParams& p) {
     ms_clear_words(p.seen, p.n);
     ms_clear_words(p.front, p.n);

@@ -664,9 +664,12 @@ __device__ __forceinline__ WarpStage warp_stage_dcsc() { return warp_stage_in(g_
 // L2 anyway, and a grid in one window claims the same bitmap words at once (R-MAT 21
 // and 24, top-down levels of 10^7 and 10^8 hub edges: 372 and 1741 us row by row, 428
 // and 1924 by windows); past two slices per td_chunk vertices, the claims are so many
-// that every order meets the same sectors (R-MAT 26, 10^9 edges: even).  Nothing
-// depends on the even spread but speed.  Neither order needs a list of slices: from
-// the classes' row counts alone a slice's number gives its row and place (hub_slice).
+// that every order meets the same sectors (R-MAT 26, 10^9 edges: even).  At 2^25
+// vertices, where the arrays start to exceed L2, the orders are even (us a search:
+// R-MAT top-down only 5900 by windows and 5907 row by row, direction-optimizing 455 and
+// 460; power law 7779 and 7772, 570 and 568).  Nothing depends on the even spread but
+// speed.  Neither order needs a list of slices: from the classes' row counts alone a
+// slice's number gives its row and place (hub_slice).
 constexpr int kHubWin = 3;
 constexpr long long kHubWinN = 1LL << 25;
 
@@ -896,7 +899,8 @@ __device__ void hub_phase(const SingleParams& p, int d, const LevelCtr& ctr, int
 // whatever the degrees of the discovered vertices: finding the parents from the
 // discovered side instead has a thread scan each row up to its first hit, and a
 // hub found early scans most of a long one (R-MAT 20: 3.9 and 24 ms a search in
-// such a pass against 0.15 ms for the levels; with this one 0.17 ms in all).
+// such a pass against 0.15 ms for the levels; with this one 0.17 ms in all).  Where
+// there are no hubs that scan can be the cheaper way: leave_to_rows.
 // Bound by its scattered level-byte reads, like the level.
 __device__ __forceinline__ void min_offer(const SingleParams& p, int d, int u, int v) {
     if (get_level(p, v) == d + 1) atomicMin(p.parent + v, u);
@@ -1266,9 +1270,9 @@ __device__ void bu_phase_a(const SingleParams& p, int d, const unsigned* fcur, u
 // neighbour in the frontier; over the hub-first rows that first neighbour is
 // the hit for most searchers on R-MAT graphs.  So phase A reads, per searcher,
 // only first[v] (the first id of its row, bit 31: more neighbours follow), a
-// per-vertex plane.  A warp takes 32 completed-bitmap words (1024 vertices) at a
-// time and compacts their searchers onto lanes (a warp prefix sum), one
-// searcher per lane per round, software-pipelined three deep: round r+2's plane
+// per-vertex plane.  A warp takes up to 32 completed-bitmap words (1024 vertices,
+// bu_chunk_words) at a time and compacts their searchers onto lanes (a warp prefix
+// sum), one searcher per lane per round, software-pipelined three deep: round r+2's plane
 // value and round r+1's frontier probe are in flight while round r consumes its
 // probe.  Hits are collected per word in shared memory and written as whole
 // next-frontier words (the warp owns its chunk's words).  A hit stores no
@@ -2226,8 +2230,9 @@ struct LoopState {
 // kDir: a directed graph (accm: out-degrees found top-down, in-degrees bottom-up;
 // the other sum in dsum_in, dsum_out).
 // Variants, so that the passes of one take no registers from another (all in
-// one kernel: 24 to 290 bytes of spills per thread; apart: none to 36 without
-// cluster levels).
+// one kernel: 24 to 290 bytes of spill stores per thread; apart: none for the
+// hub-first rows, 28 for the id-ordered ones, 48 with minimum-id parents, 56 and 76 on
+// directed graphs, 128 to 136 with cluster levels).
 template <bool kMinId, bool kHub, bool kClu, bool kDir>
 __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(SingleParams p) {
     Ctrl* c = p.ctrl;
