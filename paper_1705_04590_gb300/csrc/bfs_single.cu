@@ -959,7 +959,7 @@ __device__ void td_min_pass(const SingleParams& p, int d, const int* q, long lon
 // Rows of 180 neighbours gain nothing (520 and 542 us, 300 K vertices).
 constexpr long long kMinRowsDeg = 64, kMinRowsPer = 3, kMinPassCost = 1 << 14;
 __device__ __forceinline__ bool leave_to_rows(const SingleParams& p, long long mf, long long nnext, long long offered) {
-    return p.min_rows && mf >= kMinRowsPer * nnext && mf + offered >= p.n;
+    return mf >= kMinRowsPer * nnext && mf + offered >= p.n;
 }
 
 // ... these, and the vertices that cluster levels discovered (their frontiers live in
@@ -2351,7 +2351,7 @@ __global__ void __launch_bounds__(kBlock, BFS_MIN_BLOCKS) bfs_single_kernel(Sing
                 if (!level_sync(p, snext, s_ctr)) return;
             }
             if constexpr (kMinId) {
-                to_rows = leave_to_rows(p, S.mf, (long long)s_ctr.tail, S.offered);
+                to_rows = p.min_rows && leave_to_rows(p, S.mf, (long long)s_ctr.tail, S.offered);
                 if (s_ctr.tail > 0 && !to_rows) {
                     td_min_pass(p, S.d, S.qsel ? p.queue1 : p.queue0, S.nf, s_ctr);
                     // the next level writes this queue and the hub lists
