@@ -340,8 +340,8 @@ bfs_status bfs_run_multiroot(bfs_graph* g, const int32_t* roots_host, int32_t k,
  * neighbour one level closer (BFS_PARENT_MIN_ID semantics).  The first call
  * allocates its work buffers, about 64 bytes a vertex (half of it four planes that
  * hold the lanes' levels by bits, which the rows are written from at the end;
- * where they cannot be had, the search writes the rows as it goes, with the
- * same results).  Asynchronous on `stream`.  Errors: INVALID, OOM, CUDA.
+ * where they cannot be had, past level 14, and for up to 8 roots without
+ * parents, the search writes the rows as it goes, with the same results).  Asynchronous on `stream`.  Errors: INVALID, OOM, CUDA.
  */
 bfs_status bfs_run_multi(bfs_graph* g, const int32_t* roots_host, int32_t k, int32_t* level_dev,
                          int32_t* parent_dev, const bfs_options* opt, void* stream);
